@@ -157,8 +157,8 @@ __device__ __forceinline__ void face_adj(double* gG, int q0, double gY, unsigned
     dm4_grad((rec >> 6) & 7, gMm, t1, t2); gkL += t1; gkC += t2;  // Mm from (kL, kC)
     dm4_grad((rec >> 3) & 7, gMp, t1, t2); gkC += t1; gkR += t2;  // Mp from (kC, kR)
   } else {
-    dm4_grad((rec >> 3) & 7, gMp, t1, t2); gkL += t1; gkC += t2;  // mirrored: Mp from (kL, kC)
-    dm4_grad((rec >> 6) & 7, gMm, t1, t2); gkC += t1; gkR += t2;  // Mm from (kC, kR)
+    dm4_grad((rec >> 3) & 7, gMp, t1, t2); gkC += t1; gkL += t2;  // mirrored: Mp from (kC, kL)
+    dm4_grad((rec >> 6) & 7, gMm, t1, t2); gkR += t1; gkC += t2;  // Mm from (kR, kC)
   }
   // gradients of the line differences h_j = G[q0+j] - G[q0+j-1], j = 1..4
   double gh1, gh2, gh3, gh4;
@@ -193,7 +193,7 @@ __device__ __forceinline__ bool passive_fed(const DomDev& dm, const unsigned cha
   return !active[dm.block0 + blk] && (nb_active(dm, active, blk, d, -1) || nb_active(dm, active, blk, d, 1));
 }
 
-// Backward of one LIMO3 value Y(a, b) at a face from its recorded piece (limo3_y_sel):
+// Backward of one LIMO3 value Y(a, b) at a face from its recorded piece:
 // dY/da, dY/db of the piece. Inside the 2e-12-wide blend band of the switch the exact
 // derivative carries a factor 1e12 through the blend weight; there the piece of the
 // nearer half (unlimited or limited) is taken.

@@ -91,9 +91,11 @@ struct amrfd_handle {
   int dev = 0, nsm = 0;
   // tile of the flux pass
   int seg = 32, lines = 32, threads = 0;
+  int tile_cells = 0;               // cells (lines x stride) a tile's shared memory holds
   size_t flux_smem = 0;             // dynamic shared memory of one flux launch
   int flux_grid = 0;
   int launch_threads = 0;           // threads of one flux CTA
+  int part = 16;                    // cells of a sweep part (choose_part)
   // work lists (full, grouped per block in work order) and per-block ranges
   std::vector<int> dom_fbeg, dom_fend, dom_cbeg, dom_cend;  // per domain, in the full lists
   int nfgroups = 0;
@@ -202,6 +204,11 @@ int build_items(amrfd_handle* h) {
       const int ext = span * dm.be[dir];
       const int nseg = (ext + h->seg - 1) / h->seg;
       const int slen0 = (ext + nseg - 1) / nseg;  // balanced segments
+      // lines of an item: those of the tile, more where a shorter segment leaves the CTA's
+      // threads and shared memory room for them
+      const int fit = h->tile_cells / tile_stride(slen0);
+      const int lines = std::min(std::min(32, fit),
+                                 std::max(h->lines, h->threads / (h->nv * sweep_parts(slen0, h->part))));
       g_owner.push_back(g);
       g_stride.push_back(dir == 0 ? 1 : (dir == 1 ? dm.nb[0] : dm.nb[0] * dm.nb[1]));
       g_span.push_back(span);
@@ -209,12 +216,12 @@ int build_items(amrfd_handle* h) {
       for (int sg = 0; sg < nseg; sg++) {
         const int s0 = sg * slen0;
         const int sl = std::min(slen0, ext - s0);
-        for (int l0 = 0; l0 < nlines; l0 += h->lines) {
+        for (int l0 = 0; l0 < nlines; l0 += lines) {
           FluxItem it{};
           it.dom = d; it.blk = b; it.l0 = l0;
           it.s0 = (short)s0; it.slen = (unsigned short)sl;
           it.d = (unsigned char)dir;
-          it.nl = (unsigned char)std::min(h->lines, nlines - l0);
+          it.nl = (unsigned char)std::min(lines, nlines - l0);
           fi.push_back(it);
         }
       }
@@ -255,6 +262,8 @@ int build_items(amrfd_handle* h) {
 // Device-side work lists of the live groups (flux items) and active blocks (cell items).
 int compact(amrfd_handle* h, cudaStream_t s) {
   CompactParams p{};
+  p.doms = h->d_dom;
+  p.flux_items = 1;
   p.active = h->d_active;
   CompactList& f = p.list;
   f.ngroups = h->nfgroups;
@@ -264,6 +273,7 @@ int compact(amrfd_handle* h, cudaStream_t s) {
   f.item_bytes = sizeof(FluxItem);
   f.in = h->d_fall; f.out = h->d_fact;
   CK(launch_compact(p, s));
+  p.flux_items = 0;
   CompactList& c = p.list;
   c.ngroups = h->nblocks;
   c.owner = h->d_grp[6]; c.stride = h->d_grp[7]; c.span = h->d_grp[8]; c.beg = h->d_grp[9]; c.cnt = h->d_grp[10];
@@ -290,8 +300,8 @@ int configure_tile(amrfd_handle* h, int seg, int lines, int threads) {
   h->threads = threads;
   h->launch_threads = threads;
   h->flux_smem = smem;
-  CK(flux_set_smem(h->cfg.physics, h->nv, smem));
-  CK(flux_rec_set_smem(h->cfg.physics, h->nv, smem));
+  h->tile_cells = lines * SS;
+  CK(flux_allow_smem(h->cfg.physics, h->nv));
   int per_sm = 0;
   CK(flux_occupancy(h->cfg.physics, h->nv, h->cfg.recon == AMRFD_LIMO3, threads, smem, &per_sm));
   if (per_sm < 1) return AMRFD_ERR_INVALID_ARG;
@@ -302,17 +312,64 @@ int configure_tile(amrfd_handle* h, int seg, int lines, int threads) {
   return AMRFD_OK;
 }
 
-// Threads of a flux CTA: one per (sweep part, line, variable) of a full tile; a segment
-// of 32 cells or more is swept in parts of at least 16 cells (sweep_parts in the kernels).
-// One thread per (variable, line, part) sweep; with MP5, when a variable's sweeps fill
-// whole warps in parts of 16 cells or more, also the threads that sweep the costliest
-// variable in twice as many parts (flux_phase_b).
-int default_threads(int nv, int lines, int seg, bool mp5) {
-  const int parts = seg >= 32 ? seg / 16 : 1;
-  int tasks = nv * lines * parts;
-  if (mp5 && seg >= 32 && (lines * parts) % 32 == 0) tasks += lines * parts;
-  int t = ((tasks + 31) / 32) * 32;
-  return std::max(64, std::min(t, kFluxMaxThreads));
+// Cells of a sweep part. Sixteen (a part reads six halo cells besides its own) where
+// that fills the GPU with 20 warps per SM; shorter parts, hence shorter chains of dependent
+// faces and more warps, where it does not: a launch then lasts as long as one sweep (128^2
+// Euler blast: 43 us with 4 cells, 95 with whole segments of 16 in FP64; on the 256^3 MHD
+// blast parts of 8 to 12 measured 5 to 15 % slower than 16).
+int choose_part(const amrfd_handle* h) {
+  long long cells = 0;
+  for (auto& dm : h->hdom) cells += dm.ncell;
+  const long long faces = cells * h->cfg.ndim * h->nv / 32, room = 20LL * h->nsm;
+  return faces >= 16 * room ? 16 : (faces >= 8 * room ? 8 : 4);
+}
+
+// Sweeps per line of the longest segment of a dimension, as build_items cuts it.
+int line_sweeps(const amrfd_handle* h, int seg) {
+  int most = 1;
+  for (auto& dm : h->hdom)
+    for (int d = 0; d < h->cfg.ndim; d++) {
+      const int run = std::max(1, seg / dm.be[d]), ext = std::min(run, dm.nb[d]) * dm.be[d];
+      const int nseg = (ext + seg - 1) / seg, slen = (ext + nseg - 1) / nseg;
+      most = std::max(most, sweep_parts(slen, h->part));
+    }
+  return most;
+}
+
+// Threads of a flux CTA: one per (variable, line, part) sweep of a full tile; with extra =
+// 1 or 3 also those that sweep the costliest variable in two or four times as many parts
+// (flux_phase_b), with MP5.
+int tile_threads(const amrfd_handle* h, int seg, int lines, int extra) {
+  const int tasks = (h->nv + (h->cfg.recon == AMRFD_MP5 ? extra : 0)) * lines * line_sweeps(h, seg);
+  return std::max(64, std::min((tasks + 31) / 32 * 32, kFluxMaxThreads));
+}
+
+// Lines of a tile whose sweeps fill `threads` threads (at most): CTAs of 320 threads run two
+// on an SM, CTAs of 160 four (96 registers per thread), and the FP64 pipe of one's phase A
+// runs under the integer work of another's phase B.
+int tile_lines(const amrfd_handle* h, int seg, int threads) {
+  if (h->cfg.ndim == 1) return 1;
+  const int sweeps = h->nv * line_sweeps(h, seg);
+  int lines = 32;
+  while (lines > 1 && (sweeps * lines > threads || 16 * h->nv * lines * (seg + 7) > threads * 360)) lines /= 2;
+  return lines;
+}
+
+// The default tile. Segments of 32 cells, 16 where the domains are too small to fill the GPU
+// otherwise. 320 threads from sixteen tiles per CTA on (3D blast of 128^3: 1.19 against
+// 1.25 ms per launch with 160; 3D Euler in ragged blocks 0.65 against 0.77), 160 below
+// (512^2: 0.111 against 0.119 ms, the last wave of tiles shorter).
+void default_tile(const amrfd_handle* h, int& seg, int& lines, int& threads) {
+  seg = h->part == 16 ? 32 : 16;
+  lines = tile_lines(h, seg, kFluxMaxThreads);
+  long long cells = 0;
+  for (auto& dm : h->hdom) cells += dm.ncell;
+  if (cells * h->cfg.ndim / ((long long)seg * lines) >= 32LL * h->nsm) {
+    threads = kFluxMaxThreads;
+  } else {
+    lines = tile_lines(h, seg, 160);
+    threads = tile_threads(h, seg, lines, 1);
+  }
 }
 
 unsigned long long* slot(amrfd_handle* h, int k) { return h->d_slot + (size_t)k * h->ndom * 4; }
@@ -351,6 +408,7 @@ FluxParams flux_params(amrfd_handle* h, const double* Uk, const double* Un, int 
   p.gm1 = h->cfg.gamma - 1.0;
   p.ndim = h->cfg.ndim;
   p.P = h->lines;
+  p.part = h->part;
   int S = 1;
   for (auto& dm : h->hdom)
     for (int d = 0; d < h->cfg.ndim; d++) S = std::max(S, std::min(dm.n[d], h->seg));
@@ -495,9 +553,14 @@ int enqueue_step(amrfd_handle* h, double* U, const double* dt, cudaStream_t s, b
   const int ph = h->cfg.physics, nv = h->nv;
   CK(cudaMemsetAsync(h->d_slot, 0, sizeof(unsigned long long) * h->ns * h->ndom * 4, s));
   CK(cudaMemsetAsync(h->d_tlow, 0, sizeof(unsigned) * h->ns * h->ndom * 4, s));
-  if (batched) CK(cudaMemsetAsync(h->d_counters, 0, sizeof(int) * 2 * kMaxStages, s));
-  const int cgrid = 8 * h->nsm;
   const std::vector<int> live = batched ? std::vector<int>() : live_domains(h);
+  // Items differ in cost (limiters): taken from a counter, where blocks take more than one
+  // and one launch covers the pass (96x80x64 Euler blast, 5 stages: 3.85 ms with a fixed
+  // share per block, 3.10 ms from the counter).
+  const bool counted =
+      batched || (live.size() == 1 && h->dom_fend[live[0]] - h->dom_fbeg[live[0]] > h->flux_grid);
+  if (counted) CK(cudaMemsetAsync(h->d_counters, 0, sizeof(int) * 2 * kMaxStages, s));
+  const int cgrid = 8 * h->nsm;
   // speeds of U^n (with the CFL rate when the step computes its own dt)
   {
     int rc = speeds_from_scratch(h, U, 0, cfl_dt ? 1 : 0, batched, live, s);
@@ -528,7 +591,7 @@ int enqueue_step(amrfd_handle* h, double* U, const double* dt, cudaStream_t s, b
       // flux pass: items of passive blocks inside a live domain are skipped in the kernel
       for (int d : live) {
         fp.items = h->d_fall; fp.item0 = h->dom_fbeg[d]; fp.nitems = h->dom_fend[d] - h->dom_fbeg[d];
-        fp.counter = nullptr;
+        fp.counter = counted ? h->d_counters + 2 * (i - 1) : nullptr;
         Tick tk(h, K_FLUX, s);
         CK(launch_flux(ph, nv, fp, std::min(fp.nitems, h->flux_grid), h->launch_threads, h->flux_smem, s));
       }
@@ -678,8 +741,10 @@ int amrfd_create(amrfd_handle** out, const amrfd_config* cfg, const amrfd_domain
   for (int d = 0; d < cfg->ndim; d++) CKH(cudaMalloc(&h->d_L[d], sizeof(double) * h->nelem));
   CKH(cudaMalloc(&h->d_W, sizeof(double) * std::max<size_t>(1, h->nw_elem)));
   CKH(cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking));
-  const int lines = cfg->ndim == 1 ? 1 : 32;
-  rc = configure_tile(h, 32, lines, default_threads(h->nv, lines, 32, h->cfg.recon == AMRFD_MP5));
+  h->part = choose_part(h);
+  int seg, lines, threads;
+  default_tile(h, seg, lines, threads);
+  rc = configure_tile(h, seg, lines, threads);
   if (rc) return fail(rc);
   rc = compact(h, s);
   if (rc) return fail(rc);
@@ -1112,20 +1177,23 @@ int amrfd_autotune(amrfd_handle* h, double* U, const double* dt_dev, void* strea
     if (rc) return rc;
   }
   const int segs[] = {16, 32, 64};
-  const int lines_c[] = {8, 16, 32};
   int best_seg = h->seg, best_lines = h->lines, best_thr = h->threads;
   float best = 1e30f;
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
   for (int sg : segs) {
-    for (int ln : lines_c) {
-      if (h->cfg.ndim == 1 && ln != 1) continue;
-      for (int mul = 1; mul <= 2; mul++) {
-        const int def = default_threads(h->nv, ln, sg, h->cfg.recon == AMRFD_MP5);
-        const int thr = std::min(kFluxMaxThreads, def * mul);
-        if (mul == 2 && thr == def) continue;
-        if (configure_tile(h, sg, h->cfg.ndim == 1 ? 1 : ln, thr)) continue;
+    int prev = 0;
+    for (int full : {160, kFluxMaxThreads}) {
+      const int ln = tile_lines(h, sg, full);
+      if (ln == prev) continue;
+      prev = ln;
+      int last = 0;
+      for (int extra : {0, 1, 3}) {
+        const int thr = tile_threads(h, sg, ln, extra);
+        if (thr == last) continue;
+        last = thr;
+        if (configure_tile(h, sg, ln, thr)) continue;
         if (compact(h, s)) continue;
         FluxParams fp = flux_params(h, U, U, 0);
         fp.items = h->d_fact; fp.nitems_dev = h->d_counts; fp.counter = h->d_counters;

@@ -1,10 +1,10 @@
 // amrfd_device.cuh -- device-side building blocks of the FD-MP5 update.
 //
-// FP64 issue rate on GB300 is 1/64 of FP32, so everything that can be done
-// exactly without the FP64 pipe is: comparisons, min/max, minmod, median and
-// sign logic run on the integer pipe over the IEEE bit patterns (all exact), and
-// the FP64 operations that remain are issued in the pipe's fastest form, DFMAs
-// whose operands are all registers (see "FP64 operations as register FMAs").
+// FP64 issue rate on GB300 is 1/64 of FP32, so everything that can be done exactly
+// without the FP64 pipe is: the reconstruction sweeps run in exact fixed point
+// (amrfd_sweep.cuh), comparisons and sign logic on the integer pipe over the IEEE bit
+// patterns, and the FP64 operations that remain are issued in the pipe's fastest form,
+// DFMAs whose operands are all registers (see "FP64 operations as register FMAs").
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -16,7 +16,7 @@ namespace amrfd {
 enum { PH_EULER = 0, PH_MHD = 1 };
 
 // Descriptor checks of the checked builds: a flux item lies inside its domain and its
-// tile fits the shared-memory layout (P lines, SS doubles per line); a cell item lies
+// tile fits the shared memory (P lines of SS doubles); a cell item lies
 // inside its block.
 __device__ __forceinline__ bool flux_item_ok(const DomDev* doms, int ndom, int ndim, int P, int SS,
                                              const FluxItem& it) {
@@ -26,8 +26,9 @@ __device__ __forceinline__ bool flux_item_ok(const DomDev* doms, int ndom, int n
   if (d >= ndim || it.blk < 0 || it.blk >= dm.nb[0] * dm.nb[1] * dm.nb[2]) return false;
   const int od1 = d == 0 ? 1 : 0, od2 = d == 2 ? 1 : 2;
   const int bd = (d == 0 ? it.blk % dm.nb[0] : (d == 1 ? (it.blk / dm.nb[0]) % dm.nb[1] : it.blk / (dm.nb[0] * dm.nb[1])));
-  return it.nl >= 1 && it.nl <= P && it.l0 >= 0 && it.l0 + it.nl <= dm.be[od1] * dm.be[od2] && it.s0 >= 0 &&
-         it.slen >= 1 && it.slen + 2 * kGhost <= SS && bd * dm.be[d] + it.s0 + it.slen <= dm.n[d];
+  return it.nl >= 1 && it.nl * tile_stride(it.slen) <= P * SS && it.l0 >= 0 &&
+         it.l0 + it.nl <= dm.be[od1] * dm.be[od2] && it.s0 >= 0 && it.slen >= 1 &&
+         bd * dm.be[d] + it.s0 + it.slen <= dm.n[d];
 }
 
 __device__ __forceinline__ bool cell_item_ok(const DomDev* doms, int ndom, const CellItem& ci) {
@@ -61,13 +62,6 @@ __device__ __forceinline__ long long abits(double x) {
   return r;
 }
 
-// Sign bit of x as 0/1 (in PTX, for the same reason).
-__device__ __forceinline__ unsigned sbit(double x) {
-  unsigned r;
-  asm("{\n\t.reg .b64 t;\n\tmov.b64 t, %1;\n\tshr.u64 t, t, 63;\n\tcvt.u32.u64 %0, t;\n\t}" : "=r"(r) : "d"(x));
-  return r;
-}
-
 __device__ __forceinline__ long long okey(double x) {
   long long b = dbits(x);
   return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
@@ -94,65 +88,6 @@ __device__ __forceinline__ double imax(double a, double b) {
   return r;
 }
 
-// minmod(a,b) = (sgn a + sgn b)/2 * min(|a|,|b|): the smaller-magnitude argument
-// when both have the same sign, else zero.
-__device__ __forceinline__ double iminmod(double a, double b) {
-  double r;
-  asm("{\n\t.reg .b64 xa, xb, ma, mb, t;\n\t.reg .pred p, q;\n\t"
-      "mov.b64 xa, %1;\n\tmov.b64 xb, %2;\n\t"
-      "and.b64 ma, xa, 0x7fffffffffffffff;\n\tand.b64 mb, xb, 0x7fffffffffffffff;\n\t"
-      "setp.lt.u64 p, ma, mb;\n\tselp.b64 t, xa, xb, p;\n\t"
-      "xor.b64 ma, xa, xb;\n\tsetp.lt.s64 q, ma, 0;\n\tselp.b64 t, 0, t, q;\n\t"
-      "mov.b64 %0, t;\n\t}"
-      : "=d"(r) : "d"(a), "d"(b));
-  return r;
-}
-
-// median(x, y, z) -- one of its arguments, no rounding
-__device__ __forceinline__ double imedian(double x, double y, double z) {
-  return imax(imin(x, y), imin(imax(x, y), z));
-}
-
-// x <= c for a finite non-negative constant c (NaN compares false)
-__device__ __forceinline__ bool ile_pos(double x, double c) {
-  unsigned r;
-  asm("{\n\t.reg .b64 xa, xc, ka;\n\t.reg .pred p;\n\t"
-      "mov.b64 xa, %1;\n\tmov.b64 xc, %2;\n\t" AMRFD_OKEY("ka", "xa")
-      "setp.le.s64 p, ka, xc;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(r) : "d"(x), "d"(c));
-  return r != 0;
-}
-
-// x * 2^K exactly. The exponent field is adjusted on the integer pipe when the
-// result stays a normal number (or x is +-0); otherwise (subnormal or near-overflow
-// input, never met in practice) one FP64 multiply in an out-of-line call.
-static __device__ __noinline__ double dscale_slow(double x, double f) { return x * f; }
-
-template <int K>
-__device__ __forceinline__ double dscale(double x) {
-  double r;
-  unsigned ok;
-  constexpr long long inc = (long long)K << 52;
-  constexpr long long lo = (long long)(1 + (K < 0 ? -K : 0)) << 52;   // smallest exponent field allowed
-  constexpr long long hi = (long long)(2046 - (K > 0 ? K : 0)) << 52;  // largest exponent field allowed
-  asm("{\n\t.reg .b64 xa, m, e, y;\n\t.reg .pred pz, plo, phi, pok;\n\t"
-      "mov.b64 xa, %2;\n\t"
-      "and.b64 m, xa, 0x7fffffffffffffff;\n\t"
-      "and.b64 e, xa, 0x7ff0000000000000;\n\t"
-      "setp.eq.s64 pz, m, 0;\n\t"
-      "setp.ge.s64 plo, e, %3;\n\t"
-      "setp.le.s64 phi, e, %4;\n\t"
-      "and.pred pok, plo, phi;\n\t"
-      "or.pred pok, pok, pz;\n\t"
-      "add.s64 y, xa, %5;\n\t"
-      "selp.b64 y, xa, y, pz;\n\t"
-      "mov.b64 %0, y;\n\t"
-      "selp.u32 %1, 1, 0, pok;\n\t}"
-      : "=d"(r), "=r"(ok) : "d"(x), "l"(lo), "l"(hi), "l"(inc));
-  if (__builtin_expect(ok == 0, 0)) r = dscale_slow(x, K >= 0 ? (double)(1LL << (K >= 0 ? K : 0)) : 1.0 / (double)(1LL << (K < 0 ? -K : 0)));
-  return r;
-}
-
 // -x by flipping the sign bit (in PTX: the compiler would otherwise emit an FP64 add)
 __device__ __forceinline__ double dneg(double x) {
   double r;
@@ -171,52 +106,6 @@ __device__ __forceinline__ float f32_trunc_abs(long long ax) {
   return r;
 }
 
-// FP64 evaluation of the acceptance test, out of line so that it costs nothing
-// unless taken.
-static __device__ __noinline__ bool mp_accept_slow(double X, double mp, double eps) {
-  return ile_pos(X * (X - mp), eps);
-}
-
-// The MP acceptance test fl(X * fl(X - mp)) <= eps, decided exactly as the FP64
-// expression decides it. Signs are read from the bit patterns; a product of
-// like-signed factors is estimated in FP32 with a rigorous error bound (inputs
-// truncated to 23 bits, three FP32 roundings, the two FP64 roundings), and only
-// an estimate within the bound of eps falls back to the FP64 evaluation.
-__device__ __forceinline__ bool mp_accept(double X, double mp, double eps) {
-  long long ax, am;
-  unsigned quick, opp;
-  // sign analysis on the bit patterns: X = +-0 (product +-0), X == mp (zero
-  // difference), or X and X - mp of opposite sign (product <= 0) accept at once
-  asm("{\n\t.reg .b64 bx, bm, kx, km;\n\t.reg .pred p, q, r;\n\t"
-      "mov.b64 bx, %4;\n\tmov.b64 bm, %5;\n\t"
-      "and.b64 %0, bx, 0x7fffffffffffffff;\n\tand.b64 %1, bm, 0x7fffffffffffffff;\n\t"
-      AMRFD_OKEY("kx", "bx") AMRFD_OKEY("km", "bm")
-      "setp.eq.s64 p, %0, 0;\n\tsetp.eq.s64 q, kx, km;\n\tor.pred p, p, q;\n\t"
-      "setp.gt.s64 q, kx, km;\n\tsetp.ge.s64 r, bx, 0;\n\txor.pred q, q, r;\n\tor.pred p, p, q;\n\t"
-      "selp.u32 %2, 1, 0, p;\n\t"
-      "xor.b64 kx, bx, bm;\n\tsetp.lt.s64 q, kx, 0;\n\tselp.u32 %3, 1, 0, q;\n\t}"
-      : "=l"(ax), "=l"(am), "=r"(quick), "=r"(opp) : "d"(X), "d"(mp));
-  if (quick) return true;
-  const int ex = (int)(ax >> 52), em = (int)(am >> 52);
-  // |X|, |mp| < 2^-60: fl(X - mp) <= 2^-59 and the product is at most 2^-119
-  if (ex < 963 && em < 963 && dbits(eps) >= (904LL << 52)) return true;
-  const bool in_range = ex >= 963 && ex <= 1083 && (am == 0 || (em >= 963 && em <= 1083));
-  if (in_range) {
-    const float fx = f32_trunc_abs(ax);
-    const float fm0 = am == 0 ? 0.0f : f32_trunc_abs(am);
-    // |X - mp| = |X| - s mp with s = sign(X): the subtrahend keeps its magnitude, its
-    // sign is flipped when mp and X have opposite signs
-    const float fm = opp ? -fm0 : fm0;
-    const float df = fx - fm;
-    const float pe = fx * df;
-    const float bound = 9.5367431640625e-07f * fmaf(fx, fx + fabsf(fm), fabsf(pe));  // 2^-20 (...)
-    const float ef = (float)eps;
-    if (pe + bound < ef * 0.99999809f) return true;   // ef (1 - 2^-19)
-    if (pe - bound > ef * 1.00000191f) return false;  // ef (1 + 2^-19)
-  }
-  return mp_accept_slow(X, mp, eps);
-}
-
 // ------------------------------------------------ FP64 operations as register FMAs
 // GB300 issues a DFMA whose three operands are registers at 19.6 G warp instructions/s,
 // and a DADD, a DMUL or a DFMA with an immediate or constant-bank operand at 16.5 G/s
@@ -227,9 +116,8 @@ __device__ __forceinline__ bool mp_accept(double X, double mp, double eps) {
 // constants are read from a mutable device array through an opaque load, so the
 // compiler can neither fold them back into immediates nor read them from the constant
 // bank.
-enum { K_ONE, K_MZ, K_HALF, K_C22, K_C4, K_C48, K_C6, K_ZERO, K_C26, K_C54, K_C83, K_TWO, K_THIRD, K_C16, K_COUNT };
-static __device__ double g_regk[K_COUNT] = {1.0, -0.0, 0.5, 22.0 / 60.0, 4.0 / 60.0, 48.0 / 60.0, 6.0 / 60.0, 0.0,
-                                            26.0 / 60.0, 54.0 / 60.0, 8.0 / 3.0, 2.0, 1.0 / 3.0, 1.6};
+enum { K_ONE, K_MZ, K_HALF, K_C4, K_C6, K_ZERO, K_C26, K_C54, K_COUNT };
+static __device__ double g_regk[K_COUNT] = {1.0, -0.0, 0.5, 4.0 / 60.0, 6.0 / 60.0, 0.0, 26.0 / 60.0, 54.0 / 60.0};
 
 // Constant K_* as a register value (an opaque load at this point of the code).
 __device__ __forceinline__ double ldk(int i) {
@@ -242,116 +130,19 @@ __device__ __forceinline__ double radd(double x, double y, double one) { return 
 __device__ __forceinline__ double rsub(double x, double y, double one) { return fma(x, one, -y); }
 __device__ __forceinline__ double rmul(double c, double x, double mz) { return fma(c, x, mz); }
 
-// 2 (f_or - f_i) of MP5 from the differences: (-4 Dm + 22 D0 + 48 D1 - 6 Dp) / 60, mirrored
-// (all signs flipped) for NEG; every sweep forms it with this one operation order. The
-// weights are loaded where they are used, which keeps them out of the sweep's registers.
-template <bool NEG>
-__device__ __forceinline__ double mp5_x(double Dm, double D0, double D1, double Dp) {
-  const double mz = ldk(K_MZ), c22 = ldk(K_C22), c4 = ldk(K_C4), c48 = ldk(K_C48), c6 = ldk(K_C6);
-  const double x0 = fma(NEG ? -c22 : c22, D0, mz);
-  const double x1 = fma(NEG ? c4 : -c4, Dm, x0);
-  const double x2 = fma(NEG ? -c48 : c48, D1, x1);
-  return fma(NEG ? c6 : -c6, Dp, x2);
-}
-
-// minmod4(4 ka - kb, 4 kb - ka, ka, kb): the curvature-limited second difference at
-// a face from the curvatures of its two cells. Zero unless ka, kb share a sign; then,
-// with s the smaller and l the larger in magnitude, 4 l - s never wins and the
-// result is 4 s - l if it keeps the sign and is smaller than s, else s (one FMA).
-// Selections and the sign flip of l are integer operations.
-__device__ __forceinline__ double dm4(double ka, double kb) {
-  double sm, nl;
-  unsigned same;
-  asm("{\n\t.reg .b64 a, b, ma, mb, s, l, t;\n\t.reg .pred p, q, z;\n\t"
-      "mov.b64 a, %3;\n\tmov.b64 b, %4;\n\t"
-      "and.b64 ma, a, 0x7fffffffffffffff;\n\tand.b64 mb, b, 0x7fffffffffffffff;\n\t"
-      "setp.lt.u64 p, ma, mb;\n\t"
-      "selp.b64 s, a, b, p;\n\tselp.b64 l, b, a, p;\n\t"
-      "xor.b64 l, l, 0x8000000000000000;\n\t"
-      "xor.b64 t, a, b;\n\tsetp.ge.s64 q, t, 0;\n\t"
-      "setp.ne.s64 z, ma, 0;\n\tand.pred q, q, z;\n\t"
-      "setp.ne.s64 z, mb, 0;\n\tand.pred q, q, z;\n\t"
-      "mov.b64 %0, s;\n\tmov.b64 %1, l;\n\tselp.u32 %2, 1, 0, q;\n\t}"
-      : "=d"(sm), "=d"(nl), "=r"(same) : "d"(ka), "d"(kb));
-  if (!same) return 0.0;
-  const double t = fma(4.0, sm, nl);
-  double r;
-  asm("{\n\t.reg .b64 s, t, ms, mt, x;\n\t.reg .pred p, q;\n\t"
-      "mov.b64 s, %1;\n\tmov.b64 t, %2;\n\t"
-      "and.b64 ms, s, 0x7fffffffffffffff;\n\tand.b64 mt, t, 0x7fffffffffffffff;\n\t"
-      "setp.lt.u64 p, mt, ms;\n\tselp.b64 x, t, s, p;\n\t"
-      "xor.b64 ms, s, t;\n\tsetp.lt.s64 q, ms, 0;\n\t"
-      "setp.eq.s64 p, mt, 0;\n\tor.pred q, q, p;\n\t"
-      "selp.b64 x, 0, x, q;\n\tmov.b64 %0, x;\n\t}"
-      : "=d"(r) : "d"(sm), "d"(t));
-  return r;
-}
-
-// ---------------------------------------------------------- MP5 in difference form
+// ------------------------------------------------ MP5's pieces, for the discrete adjoint
 // MP5 (Suresh & Huynh 1997) at face i+1/2 from (f_{i-2}, ..., f_{i+2}), written in
 // differences Dm = f_{i-1}-f_{i-2}, D0 = f_i-f_{i-1}, D1 = f_{i+1}-f_i, Dp = f_{i+2}-f_{i+1}
 // and the curvature-limited second differences Mp (at i+1/2) and Mm (at i-1/2):
 //   f_or - f_i = (11 D0 - 2 Dm + 24 D1 - 3 Dp)/60,  f_mp - f_i = minmod(D1, 4 D0),
 //   f_ul - f_i = 4 D0,  f_md - f_i = D1/2 - Mp/2,  f_lc - f_i = D0/2 + 4 Mm/3,
 // with the acceptance test (f_or - f_i)(f_or - f_mp) <= eps and otherwise
-// median(f_or, f_min, f_max). Everything is carried at twice its value, which makes
-// the halvings and the factor 4 exact exponent shifts; the result is
-// 2 (f_face - f_i). NEG evaluates the mirror-image stencil whose differences are
-// the negatives of the ones passed in (the right-biased reconstruction).
-// eps16 = 16 eps: 4 eps for values doubled twice (splitting without the 1/2, and here).
-//
-// mp5_rel2_r also reports whether the acceptance test failed (rej). CARRY takes the
-// curvature-limited second differences Mp, Mm from the caller (carried along the line);
-// otherwise they are formed here, only when the test fails, from the curvatures of cells
-// i-1, i, i+1 with the operands and order of the carried ones (for NEG, of the mirrored
-// stencil), so both forms give the same result.
-template <bool NEG, bool CARRY>
-__device__ __forceinline__ double mp5_rel2_r(double Dm, double D0, double D1, double Dp, double Mp, double Mm,
-                                             double eps16, bool& rej, double one) {
-  const double X = mp5_x<NEG>(Dm, D0, D1, Dp);  // 2 (f_or - f_i)
-  const double d0 = NEG ? dneg(D0) : D0;
-  const double d1 = NEG ? dneg(D1) : D1;
-  const double ul = dscale<3>(d0);     // 2 (f_ul - f_i)
-  const double d1x2 = dscale<1>(d1);   // 2 (f_{i+1} - f_i)
-  const double mp = iminmod(d1x2, ul);  // 2 (f_mp - f_i)
-  rej = false;
-  if (mp_accept(X, mp, eps16)) return X;
-  rej = true;
-  if (!CARRY) {
-    if (!NEG) {
-      const double k0 = rsub(D1, D0, one);
-      Mp = dm4(k0, rsub(Dp, D1, one));
-      Mm = dm4(rsub(D0, Dm, one), k0);
-    } else {
-      const double k0 = rsub(D0, D1, one);
-      Mp = dm4(rsub(D1, Dp, one), k0);
-      Mm = dm4(k0, rsub(Dm, D0, one));
-    }
-  }
-  const double md = rsub(d1, Mp, one);          // 2 (f_md - f_i)
-  const double lc = fma(ldk(K_C83), Mm, d0);    // 2 (f_lc - f_i)
-  const double fmin = imax(imin(imin(0.0, d1x2), md), imin(imin(0.0, ul), lc));
-  const double fmax = imin(imax(imax(0.0, d1x2), md), imax(imax(0.0, ul), lc));
-  return imedian(X, fmin, fmax);
-}
-
-// ------------------------------------------------ selection-tracking variants
-// The same operations as mp5_rel2_r / dm4 (bit-identical results), also reporting
-// which linear piece produced the value, for the discrete adjoint.
+// median(f_or, f_min, f_max). The sweeps (amrfd_sweep.cuh) record which piece they took; the
+// adjoint works on twice the value, 2 (f_face - f_i), of the splitting G = 2 F^{+-}. NEG is
+// the mirror-image stencil, whose differences are the negatives of the ones used.
 enum { SEL_X = 0, SEL_ZERO = 1, SEL_D1 = 2, SEL_MD = 3, SEL_UL = 4, SEL_LC = 5 };
 
-__device__ __forceinline__ void imin_sel(double a, int ca, double b, int cb, double& r, int& cr) {
-  const bool t = okey(a) < okey(b);
-  r = t ? a : b;
-  cr = t ? ca : cb;
-}
-__device__ __forceinline__ void imax_sel(double a, int ca, double b, int cb, double& r, int& cr) {
-  const bool t = okey(a) < okey(b);
-  r = t ? b : a;
-  cr = t ? cb : ca;
-}
-
-// Gradient of the MP5 value (mp5_rel2_r) w.r.t. (Dm, D0, D1, Dp, Mp, Mm) for the piece `code`, times g.
+// Gradient of the MP5 value w.r.t. (Dm, D0, D1, Dp, Mp, Mm) for the piece `code`, times g.
 template <bool NEG>
 __device__ __forceinline__ void mp5_rel2_grad(int code, double g, double& gDm, double& gD0, double& gD1,
                                               double& gDp, double& gMp, double& gMm) {
@@ -372,81 +163,14 @@ __device__ __forceinline__ void mp5_rel2_grad(int code, double g, double& gDm, d
   }
 }
 
-// dm4 with the chosen piece: 0 zero, 1 ka, 2 kb, 3 4 ka - kb, 4 4 kb - ka.
-__device__ __forceinline__ double dm4_sel(double ka, double kb, int& code) {
-  const long long a = dbits(ka), b = dbits(kb);
-  const long long M = 0x7fffffffffffffffLL;
-  const long long ma = a & M, mb = b & M;
-  code = 0;
-  if (((a ^ b) < 0) | (ma == 0) | (mb == 0)) return 0.0;
-  const bool as = ma < mb;
-  const double sm = as ? ka : kb, lg = as ? kb : ka;
-  const long long ms = as ? ma : mb;
-  const double t = fma(4.0, sm, -lg);
-  const long long bt = dbits(t);
-  if (((bt ^ dbits(sm)) < 0) | ((bt & M) == 0)) return 0.0;
-  if ((bt & M) < ms) { code = as ? 3 : 4; return t; }
-  code = as ? 1 : 2;
-  return sm;
-}
-
+// Gradient of minmod4(4 ka - kb, 4 kb - ka, ka, kb) for its piece: 0 zero, 1 ka, 2 kb,
+// 3 4 ka - kb, 4 4 kb - ka.
 __device__ __forceinline__ void dm4_grad(int code, double g, double& gka, double& gkb) {
   gka = gkb = 0.0;
   if (code == 1) gka = g;
   else if (code == 2) gkb = g;
   else if (code == 3) { gka = 4.0 * g; gkb = -g; }
   else if (code == 4) { gkb = 4.0 * g; gka = -g; }
-}
-
-// mp5_rel2_r without CARRY (bit-identical value) that also records the pieces taken: the
-// curvature-limited second differences are formed only where the acceptance test fails,
-// with dm4_sel, and the median's selections are tracked. rec = piece of the value | piece
-// of Mp << 3 | piece of Mm << 6 (the curvature pieces are 0 where the value is f_or,
-// which reads neither).
-template <bool NEG>
-__device__ __forceinline__ double mp5_rel2_rec(double Dm, double D0, double D1, double Dp, double eps16, int& rec,
-                                               double one) {
-  const double X = mp5_x<NEG>(Dm, D0, D1, Dp);
-  const double d0 = NEG ? dneg(D0) : D0;
-  const double d1 = NEG ? dneg(D1) : D1;
-  const double ul = dscale<3>(d0);
-  const double d1x2 = dscale<1>(d1);
-  const double mp = iminmod(d1x2, ul);
-  rec = SEL_X;
-  if (mp_accept(X, mp, eps16)) return X;
-  double Mp, Mm;
-  int cp, cm;
-  if (!NEG) {
-    const double k0 = rsub(D1, D0, one);
-    Mp = dm4_sel(k0, rsub(Dp, D1, one), cp);
-    Mm = dm4_sel(rsub(D0, Dm, one), k0, cm);
-  } else {
-    const double k0 = rsub(D0, D1, one);
-    Mp = dm4_sel(rsub(D1, Dp, one), k0, cp);
-    Mm = dm4_sel(k0, rsub(Dm, D0, one), cm);
-  }
-  const double md = rsub(d1, Mp, one);
-  const double lc = fma(ldk(K_C83), Mm, d0);
-  double a, b, fmin, fmax, t1, t2, t3;
-  int ca, cb, cmin, cmax, c1, c2, c3;
-  imin_sel(0.0, SEL_ZERO, d1x2, SEL_D1, a, ca);
-  imin_sel(a, ca, md, SEL_MD, a, ca);
-  imin_sel(0.0, SEL_ZERO, ul, SEL_UL, b, cb);
-  imin_sel(b, cb, lc, SEL_LC, b, cb);
-  imax_sel(a, ca, b, cb, fmin, cmin);
-  imax_sel(0.0, SEL_ZERO, d1x2, SEL_D1, a, ca);
-  imax_sel(a, ca, md, SEL_MD, a, ca);
-  imax_sel(0.0, SEL_ZERO, ul, SEL_UL, b, cb);
-  imax_sel(b, cb, lc, SEL_LC, b, cb);
-  imin_sel(a, ca, b, cb, fmax, cmax);
-  imin_sel(X, SEL_X, fmin, cmin, t1, c1);
-  imax_sel(X, SEL_X, fmin, cmin, t2, c2);
-  imin_sel(t2, c2, fmax, cmax, t3, c3);
-  double r;
-  int code;
-  imax_sel(t1, c1, t3, c3, r, code);
-  rec = code | (cp << 3) | (cm << 6);
-  return r;
 }
 
 // Reciprocal of a positive normal double: FP32 seed from the leading bits (integer
@@ -645,11 +369,11 @@ __device__ __forceinline__ void prim_w(const double* u, double gm1, double* w) {
 
 // Physical flux along D from U and its derived quantities, then the Lax-Friedrichs
 // split in doubled form G^{+-} = F +- alpha U (= 2 F^{+-}); psi's flux is c_h^2 B_D.
+// one, mz: 1 and -0 in registers.
 template <int PHYS, int NV, int D>
 __device__ __forceinline__ void split_flux_w(const double* u, const double* w, double alpha, double ch2,
-                                             double* gp, double* gm) {
+                                             double one, double mz, double* gp, double* gm) {
   double f[NV];
-  const double one = ldk(K_ONE), mz = ldk(K_MZ);
   if (PHYS == PH_EULER) {
     constexpr int nm = NV - 2;
     const double p = w[nm], vd = w[D];

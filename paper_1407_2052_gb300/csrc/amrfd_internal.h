@@ -2,6 +2,12 @@
 #pragma once
 #include <cstdint>
 
+#ifdef __CUDACC__
+#define AMRFD_BOTH __host__ __device__
+#else
+#define AMRFD_BOTH
+#endif
+
 namespace amrfd {
 
 constexpr int kGhost = 3;       // MP5 needs cells i-2..i+3 around face i+1/2
@@ -54,8 +60,20 @@ struct FluxItem {
   unsigned short slen;
   unsigned char d;
   unsigned char nl;
-  unsigned char pad[6];
+  unsigned char live;  // ItemLive bits, kept by the compaction of the work lists
+  unsigned char pad[5];
 };
+// Shared-memory layout of an item's tile: nl lines of tile_stride(slen) doubles per variable
+// and sign (an odd stride: lines fall into different banks).
+constexpr AMRFD_BOTH int tile_stride(int slen) { return (slen + 2 * kGhost) | 1; }
+// Parts of a segment's sweep, 0.6 to 1.2 times `part` cells each where the segment has
+// them: one thread per (variable, part, line); each part reads its six halo cells itself.
+constexpr AMRFD_BOTH int sweep_parts(int slen, int part) {
+  return (slen + part * 13 / 16) / part > 1 ? (slen + part * 13 / 16) / part : 1;
+}
+// Activity of the blocks an item touches: any / every block of its segment, and every
+// block of the segment and of its three halo cells on both sides.
+enum ItemLive : unsigned char { kLiveAny = 1, kLiveAll = 2, kLiveHalo = 4 };
 static_assert(sizeof(FluxItem) == 24, "FluxItem layout");
 
 // One cell-wise work item: block-local cells [c0, c0+cnt) of block `blk` (x fastest).

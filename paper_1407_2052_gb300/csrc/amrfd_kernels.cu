@@ -19,6 +19,7 @@
 
 #include "amrfd_device.cuh"
 #include "amrfd_kernels.cuh"
+#include "amrfd_sweep.cuh"
 
 namespace amrfd {
 
@@ -211,46 +212,122 @@ __device__ __forceinline__ double glm_speed(const unsigned long long* s0, int nd
   return ch;
 }
 
-// Phase A of a flux item: the tile's G^{+-} (lines x segment + halo) into shared
-// memory, cells start, start + stride, ... of the tile.
+// Splitting speed of an item's direction (raised to c_h with GLM) and c_h^2.
+template <int D>
+__device__ __forceinline__ double item_alpha(const FluxParams& p, const FluxItem& it, double& ch2) {
+  const unsigned long long* sk = p.araw + (size_t)it.dom * 4;
+  const unsigned long long* s0 = p.araw0 + (size_t)it.dom * 4;
+  const double ch = p.glm ? glm_speed(s0, p.ndim) : 0.0;
+  ch2 = ch * ch;
+  return imax(bitsd((long long)sk[D]), ch);
+}
+
+// The cell whose values stand at coordinate g along dimension d (g may lie up to three cells
+// outside): periodic wrap, the edge cell (zero gradient) or the mirror image; odd: the
+// variables a mirror negates.
+__device__ __forceinline__ int halo_cell(const DomDev& dm, int d, int g, unsigned& odd) {
+  const int n = dm.n[d];
+  odd = 0u;
+  if (g < 0) {
+    const int b = dm.bc[d][0];
+    odd = dm.asym[d][0];
+    return b == 0 ? g + n : (b == 1 ? 0 : -1 - g);
+  }
+  if (g >= n) {
+    const int b = dm.bc[d][1];
+    odd = dm.asym[d][1];
+    return b == 0 ? g - n : (b == 1 ? n - 1 : 2 * n - 1 - g);
+  }
+  return g;
+}
+
+__device__ __forceinline__ int exponent(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) - 1023; }
+
+// Rounds the G^{+-} that are tiny on their cell's own flux scale to whole multiples of
+// 2^-96 of it: rho a^2 for momentum, sqrt(rho) a^2 and a^3 for B and psi (a the splitting
+// speed, exponents only). Ahead of a front such components fall off by binades per cell
+// down to underflow; whole multiples of one unit keep the sweeps' exact sums within 110
+// bits there. The change is 2^-43 of the scale's FP64 rounding, and components above 2^-43
+// of the scale keep all their bits.
+template <int PHYS, int NV>
+__device__ __forceinline__ void round_tiny(double rho, int ea, double* gp, double* gm) {
+  const int er = exponent(rho);
+  constexpr int m0 = 1, m1 = PHYS == PH_EULER ? NV - 1 : 4;
+  // exponents (biased) below which the last mantissa bit lies under the unit
+  const int tm = min(er + 2 * ea + (1023 + 52 - 96), 2046), tb = min((er >> 1) + 2 * ea + (1023 + 52 - 96), 2046),
+            tp = min((er >> 1) + 3 * ea + (1023 + 52 - 96), 2046);
+  bool any = false;
+#pragma unroll
+  for (int v = m0; v < NV; v++) {
+    if (PHYS == PH_EULER ? v >= m1 : v == 4) continue;
+    const int t = (v < m1 ? tm : (v < 8 ? tb : tp)) << 20;
+    const int a = __double2hiint(gp[v]) & 0x7fffffff, b = __double2hiint(gm[v]) & 0x7fffffff;
+    any |= (unsigned)(a - 1) < (unsigned)(t - 1) || (unsigned)(b - 1) < (unsigned)(t - 1);
+  }
+  if (!any) return;
+#pragma unroll
+  for (int v = m0; v < NV; v++) {
+    if (PHYS == PH_EULER ? v >= m1 : v == 4) continue;
+    const int t = v < m1 ? tm : (v < 8 ? tb : tp);
+#pragma unroll
+    for (int s = 0; s < 2; s++) {
+      double& g = s ? gm[v] : gp[v];
+      const long long x = dbits(g);
+      const int r = t - (int)((x >> 52) & 0x7ff);  // mantissa bits under the unit
+      if (r <= 0) continue;
+      const int k = r < 53 ? r : 53;
+      const long long y = (x + (1ll << (k - 1))) & ~((1ll << (k < 52 ? k : 52)) - 1);
+      g = bitsd(r > 53 ? 0ll : y);
+    }
+  }
+}
+
+// Phase A of a flux item along D: the tile's G^{+-} (lines x segment + halo) into shared
+// memory. FP64-bound: 33 of its ~150 instructions per cell, one per 64 cycles; the index
+// arithmetic keeps no division and no block lookup in the loop (on the 1024^2 vortex the
+// phase alone takes 0.152 ms of a launch, 87 % of it FP64 issue).
 template <int PHYS, int NV, int D>
-__device__ __forceinline__ void flux_phase_a(const FluxParams& p, const DomDev& dm, const FluxItem& it,
-                                             const int o[3], double alpha, double ch2, double* sm, int start,
-                                             int stride) {
+__device__ __forceinline__ void flux_phase_a(const FluxParams& p, const DomDev& dm, const FluxItem& it, double* sm) {
   constexpr int od1 = D == 0 ? 1 : 0;
   constexpr int od2 = D == 2 ? 1 : 2;
   const int W = it.slen + 2 * kGhost;
   const int nl = it.nl;
-  const int P = p.P, SS = p.SS;
-  const double gm1 = p.gm1;
-  for (int c = start; c < nl * W; c += stride) {
-    int pl, j;
-    if (D == 0) { pl = c / W; j = c - pl * W; }
-    else { j = c / nl; pl = c - j * nl; }
-    const int line = it.l0 + pl;
-    const int a1 = line % dm.be[od1], a2 = line / dm.be[od1];
-    int x[3];
-    x[od1] = o[od1] + a1;
-    x[od2] = o[od2] + a2;
-    int g = o[D] + it.s0 + j - kGhost;
-    unsigned odd = 0u;  // mirror ghosts: variables negated
-    if (g < 0) {
-      const int b = dm.bc[D][0];
-      odd = dm.asym[D][0];
-      g = b == 0 ? g + dm.n[D] : (b == 1 ? 0 : -1 - g);
-    } else if (g >= dm.n[D]) {
-      const int b = dm.bc[D][1];
-      odd = dm.asym[D][1];
-      g = b == 0 ? g - dm.n[D] : (b == 1 ? dm.n[D] - 1 : 2 * dm.n[D] - 1 - g);
+  const int P = nl, SS = tile_stride(it.slen);
+  double ch2;
+  const double alpha = item_alpha<D>(p, it, ch2);
+  const double gm1 = p.gm1, one = ldk(K_ONE), mz = ldk(K_MZ);
+  const int ea = exponent(alpha);
+  const int sx[3] = {1, dm.n[0], dm.n[0] * dm.n[1]};
+  int o[3];
+  block_coords(dm, it.blk, o);
+  const int e1 = dm.be[od1];
+  const int l1 = it.l0 % e1, l2 = it.l0 / e1;  // the first line
+  const int g0 = o[D] + it.s0 - kGhost;
+  const bool live = (it.live & kLiveHalo) != 0;
+  // cells threadIdx.x, threadIdx.x + blockDim.x, ... of the tile, neighbouring threads along x
+  const int inner = D == 0 ? W : nl, outer = D == 0 ? nl : W;
+  int ou = threadIdx.x / inner, in = threadIdx.x - ou * inner;
+  const int dou = blockDim.x / inner, din = blockDim.x - dou * inner;
+  for (; ou < outer; ou += dou, in += din) {
+    if (in >= inner) {
+      in -= inner;
+      if (++ou >= outer) break;
     }
-    x[D] = g;
-    AMRFD_GUARD(p.err, g >= 0 && g < dm.n[D] && x[od1] < dm.n[od1] && x[od2] < dm.n[od2] && pl < P && j < SS,
-                continue)
-    const int nbk = dm.block0 + ((x[2] / dm.be[2]) * dm.nb[1] + x[1] / dm.be[1]) * dm.nb[0] + x[0] / dm.be[0];
-    const bool act = p.active[nbk] != 0;
-    const double* base = act ? p.Uk : p.Un;
-    const long long idx = ((long long)x[2] * dm.n[1] + x[1]) * dm.n[0] + x[0];
-    const double* src = base + dm.off + idx;
+    const int pl = D == 0 ? ou : in, j = D == 0 ? in : ou;
+    int a1 = l1 + pl, a2 = l2;
+    while (a1 >= e1) { a1 -= e1; a2++; }
+    unsigned odd;
+    const int g = halo_cell(dm, D, g0 + j, odd);
+    const int x1 = o[od1] + a1, x2 = o[od2] + a2;
+    AMRFD_GUARD(p.err, g >= 0 && g < dm.n[D] && x1 < dm.n[od1] && x2 < dm.n[od2] && pl < P && j < SS, continue)
+    const long long idx = (long long)x1 * sx[od1] + (long long)x2 * sx[od2] + (long long)g * sx[D];
+    bool act = true;
+    if (!live) {  // a passive block is near: its cells are read as U^n
+      int x[3];
+      x[od1] = x1; x[od2] = x2; x[D] = g;
+      act = p.active[dm.block0 + ((x[2] / dm.be[2]) * dm.nb[1] + x[1] / dm.be[1]) * dm.nb[0] + x[0] / dm.be[0]] != 0;
+    }
+    const double* src = (act ? p.Uk : p.Un) + dm.off + idx;
     constexpr int NW = NumW<PHYS, NV>::value;
     double u[NV], w[NW], gp[NV], gmn[NV];
 #pragma unroll
@@ -269,7 +346,8 @@ __device__ __forceinline__ void flux_phase_a(const FluxParams& p, const DomDev& 
     } else {
       prim_w<PHYS, NV>(u, gm1, w);
     }
-    split_flux_w<PHYS, NV, D>(u, w, alpha, ch2, gp, gmn);
+    split_flux_w<PHYS, NV, D>(u, w, alpha, ch2, one, mz, gp, gmn);
+    round_tiny<PHYS, NV>(u[0], ea, gp, gmn);
 #pragma unroll
     for (int v = 0; v < NV; v++) {
       sm[((0 * NV + v) * P + pl) * SS + j] = gp[v];
@@ -278,284 +356,12 @@ __device__ __forceinline__ void flux_phase_a(const FluxParams& p, const DomDev& 
   }
 }
 
-// Recording sweep of one (line, variable): MP5 on both biases at faces k = 3..slen+3 of
-// the line's extended index (cell j = k-1 left of face k), then the flux difference
-// Fsum_{k-1} - Fsum_k of the segment's cell k-4 stored to out[(k-4) ostr] where wmask has
-// its bit (the factor 1/(2 dx) is applied by the stage combination). With
-// Fsum_k = G+_{k-1} + G-_k + (Y+_k + Y-_k)/2, the difference is formed from what the sweep
-// holds, (S_{k-1} - S_k)/2 - (G+_{k-1} - G+_{k-2}) - (G-_k - G-_{k-1}) with S = Y+ + Y-: no
-// subtraction of two fluxes of the size of G, and two shared-memory reads per face (each
-// array's newest value; the previous one is kept in a register). Per face and bias it
-// records which linear piece the limiter took and the pieces of the two curvature limiters
-// it read (mp5_rel2_rec, 3 bits each): tp/tm point at the line's records, face k goes to
-// index f0 + k - 3 if below fend (face n of a periodic line, fmod = n, as face 0).
-__device__ __forceinline__ void flux_sweep_rec(const double* g, const double* h, int slen, double eps16,
-                                               unsigned short* tp, unsigned short* tm, int f0, int fend, int fmod,
-                                               double* out, long long ostr, unsigned long long wmask, double one) {
-  double Pd1 = rsub(g[1], g[0], one), Pd2 = rsub(g[2], g[1], one), Pd3 = rsub(g[3], g[2], one),
-         Pd4 = rsub(g[4], g[3], one);
-  double Md2 = rsub(h[2], h[1], one), Md3 = rsub(h[3], h[2], one), Md4 = rsub(h[4], h[3], one),
-         Md5 = rsub(h[5], h[4], one);
-  double gl = g[4], hl = h[5];  // the last values read, g[k+1] and h[k+2]
-  double Sprev = 0.0;
-  const int kend = slen + 3;
-  for (int k = 3; k <= kend; ++k) {
-    int yp, ym;
-    const double Yp = mp5_rel2_rec<false>(Pd1, Pd2, Pd3, Pd4, eps16, yp, one);
-    const double Ym = mp5_rel2_rec<true>(Md5, Md4, Md3, Md2, eps16, ym, one);
-    const int f = f0 + k - 3;
-    if (f < fend) {
-      const int fi = f >= fmod ? f - fmod : f;
-      tp[fi] = (unsigned short)yp;
-      tm[fi] = (unsigned short)ym;
-    }
-    const double S = radd(Yp, Ym, one);
-    if (k > 3 && ((wmask >> (k - 4)) & 1ull))
-      out[(long long)(k - 4) * ostr] = fma(ldk(K_HALF), rsub(Sprev, S, one), -radd(Pd2, Md3, one));
-    Sprev = S;
-    if (k < kend) {
-      const double gn = g[k + 2], hn = h[k + 3];
-      Pd1 = Pd2; Pd2 = Pd3; Pd3 = Pd4; Pd4 = rsub(gn, gl, one); gl = gn;
-      Md2 = Md3; Md3 = Md4; Md4 = Md5; Md5 = rsub(hn, hl, one); hl = hn;
-    }
-  }
-}
-
-// Plain MP5 sweep, same fluxes as flux_sweep_rec. The curvature-limited second
-// differences serve only faces that fail the acceptance test, so a warp (32 lines of
-// one variable) carries them along the line only while some lane keeps failing: after
-// a face where one did, it forms them from the current differences (the operands of
-// the carried ones) and carries them; after a face where none did, it drops them and
-// forms them per face at failing faces only (mp5_rel2_r without CARRY).
-// Every lane in `lanes` must call this with the same slen (the face votes pair up).
-// Returns the number of faces after which some lane had failed (the same in every lane):
-// the warp's limiter work, which phase B uses to balance the variables' sweeps.
-__device__ __forceinline__ int flux_sweep_adaptive(const double* g, const double* h, int slen, double eps16,
-                                                   double* out, long long ostr, unsigned long long wmask,
-                                                   unsigned lanes, double one) {
-  int busy = 0;
-  double Pd1 = rsub(g[1], g[0], one), Pd2 = rsub(g[2], g[1], one), Pd3 = rsub(g[3], g[2], one),
-         Pd4 = rsub(g[4], g[3], one);
-  double Md2 = rsub(h[2], h[1], one), Md3 = rsub(h[3], h[2], one), Md4 = rsub(h[4], h[3], one),
-         Md5 = rsub(h[5], h[4], one);
-  double Pk3 = 0.0, Mk4 = 0.0, PM2 = 0.0, PM3 = 0.0, MM3 = 0.0, MM4 = 0.0;
-  bool carry = false;
-  double gl = g[4], hl = h[5];  // the last values read, g[k+1] and h[k+2]
-  double Sprev = 0.0;
-  const int kend = slen + 3;
-  for (int k = 3; k <= kend; ++k) {
-    // left-biased reconstruction of G^+ centred on cell k-1, right-biased of G^-
-    // centred on cell k (mirror image)
-    double Yp, Ym;
-    bool rp, rm;
-    if (carry) {
-      Yp = mp5_rel2_r<false, true>(Pd1, Pd2, Pd3, Pd4, PM3, PM2, eps16, rp, one);
-      Ym = mp5_rel2_r<true, true>(Md5, Md4, Md3, Md2, MM3, MM4, eps16, rm, one);
-    } else {
-      Yp = mp5_rel2_r<false, false>(Pd1, Pd2, Pd3, Pd4, 0.0, 0.0, eps16, rp, one);
-      Ym = mp5_rel2_r<true, false>(Md5, Md4, Md3, Md2, 0.0, 0.0, eps16, rm, one);
-    }
-    const double S = radd(Yp, Ym, one);
-    if (k > 3 && ((wmask >> (k - 4)) & 1ull))
-      out[(long long)(k - 4) * ostr] = fma(ldk(K_HALF), rsub(Sprev, S, one), -radd(Pd2, Md3, one));
-    Sprev = S;
-    if (k < kend) {
-      const bool want = __any_sync(lanes, rp || rm);
-      const double gn = g[k + 2], hn = h[k + 3];
-      Pd1 = Pd2; Pd2 = Pd3; Pd3 = Pd4; Pd4 = rsub(gn, gl, one); gl = gn;
-      Md2 = Md3; Md3 = Md4; Md4 = Md5; Md5 = rsub(hn, hl, one); hl = hn;
-      if (want && carry) {
-        const double pk = rsub(Pd4, Pd3, one);
-        PM2 = PM3;
-        PM3 = dm4(Pk3, pk);
-        Pk3 = pk;
-        const double mk = rsub(Md5, Md4, one);
-        MM3 = MM4;
-        MM4 = dm4(Mk4, mk);
-        Mk4 = mk;
-      } else if (want) {
-        const double Pk2 = rsub(Pd3, Pd2, one), Mk3 = rsub(Md4, Md3, one);
-        Pk3 = rsub(Pd4, Pd3, one);
-        Mk4 = rsub(Md5, Md4, one);
-        PM2 = dm4(rsub(Pd2, Pd1, one), Pk2);
-        PM3 = dm4(Pk2, Pk3);
-        MM3 = dm4(rsub(Md3, Md2, one), Mk3);
-        MM4 = dm4(Mk3, Mk4);
-      }
-      carry = want;
-      busy += want;
-    }
-  }
-  return busy;
-}
-
-// LIMO3 (Cada & Torrilhon 2009) in product form: with a = delta_{i-1/2} and
-// b = delta_{i+1/2} (G units), the correction b phi(theta) of u_i + b phi / 2 is
-//   unlimited  b phi_3 = (2 b + a) / 3,
-//   limited    b phi^_3 = s max(0, min(y3, max(-a'/2, min(2 a', y3, 1.6 |b|))))
-// evaluated on a' = s a, y3' = s y3, s = sign(b): multiplying the limiter's terms by
-// |b| keeps their order, so no theta = a/b is formed (b = 0 gives 0, the limit). The
-// switch eta = (a^2 + b^2) / (4 (r dx)^2) (G = 2 F^{+-}) picks the unlimited value
-// inside the asymptotic region, the limited one outside, and blends linearly over
-// |eta - 1| < 1e-12.
-__device__ __forceinline__ double limo3_y(double a, double b, double s2, long long tlo, long long thi, double esc,
-                                          double mz) {
-  const double y3 = rmul(fma(ldk(K_TWO), b, a), ldk(K_THIRD), mz);
-  const long long bs = abits(s2);  // s2 = a^2 + b^2 >= 0: its bit pattern orders like its value
-  if (bs <= tlo) return y3;
-  const bool neg = sbit(b) != 0;
-  const double ap = neg ? dneg(a) : a;
-  const double y3p = neg ? dneg(y3) : y3;
-  const double bp = neg ? dneg(b) : b;
-  double t = imin(imin(dscale<1>(ap), y3p), rmul(ldk(K_C16), bp, mz));
-  t = imax(dscale<-1>(dneg(ap)), t);
-  t = imin(y3p, t);
-  t = imax(0.0, t);
-  const double yl = neg ? dneg(t) : t;
-  if (bs >= thi) return yl;
-  const double z = fma(s2, esc, -1.0) * 1e12;
-  return 0.5 * ((1.0 - z) * y3 + (1.0 + z) * yl);
-}
-
-// limo3_y (bit-identical value) that also reports the piece it took, for the discrete
-// adjoint: bits 0-2 the limited piece (0 zero, 1 y3, 2 -a/2, 3 2a, 4 1.6 b, each as a
-// function of the unsigned a, b), bits 3-4 the mode (0 unlimited, 1 limited, 2 / 3 inside
-// the blend band on its unlimited / limited half).
-__device__ __forceinline__ double limo3_y_sel(double a, double b, double s2, long long tlo, long long thi,
-                                              double esc, int& code, double mz) {
-  const double y3 = rmul(fma(ldk(K_TWO), b, a), ldk(K_THIRD), mz);
-  const long long bs = abits(s2);
-  if (bs <= tlo) { code = 0; return y3; }
-  const bool neg = sbit(b) != 0;
-  const double ap = neg ? dneg(a) : a;
-  const double y3p = neg ? dneg(y3) : y3;
-  const double bp = neg ? dneg(b) : b;
-  double t;
-  int c;
-  imin_sel(dscale<1>(ap), 3, y3p, 1, t, c);
-  imin_sel(t, c, rmul(ldk(K_C16), bp, mz), 4, t, c);
-  imax_sel(dscale<-1>(dneg(ap)), 2, t, c, t, c);
-  imin_sel(y3p, 1, t, c, t, c);
-  imax_sel(0.0, 0, t, c, t, c);
-  const double yl = neg ? dneg(t) : t;
-  if (bs >= thi) { code = c | (1 << 3); return yl; }
-  const double z = fma(s2, esc, -1.0) * 1e12;
-  code = c | ((z < 0.0 ? 2 : 3) << 3);
-  return 0.5 * ((1.0 - z) * y3 + (1.0 + z) * yl);
-}
-
-// LIMO3 sweep of one (line, variable): faces k = 3..slen+3 as in flux_sweep_rec; G^+ from
-// cells k-2..k (centre k-1), G^- mirrored from cells k+1..k-1 (centre k). The squares of
-// the differences are carried along the line (each enters two faces' switch), and the
-// switch compares a^2 + b^2 with (1 -+ 1e-12)/esc.
-__device__ __forceinline__ void limo3_sweep(const double* g, const double* h, int slen, double esc, double* out,
-                                            long long ostr, unsigned long long wmask) {
-  const long long tlo = __double_as_longlong((1.0 - 1e-12) / esc), thi = __double_as_longlong((1.0 + 1e-12) / esc);
-  const double one = ldk(K_ONE), mz = ldk(K_MZ);
-  double Pa = rsub(g[2], g[1], one), Pb = rsub(g[3], g[2], one);  // delta_{i-1/2}, delta_{i+1/2} of G^+ at face 3
-  double Mb = rsub(h[3], h[2], one), Ma = rsub(h[4], h[3], one);  // mirrored: -delta_{i+1/2}, -delta_{i-1/2} of G^-
-  double Pa2 = rmul(Pa, Pa, mz), Pb2 = rmul(Pb, Pb, mz), Ma2 = rmul(Ma, Ma, mz), Mb2 = rmul(Mb, Mb, mz);
-  double gl = g[3], hl = h[4];  // the last values read, g[k] and h[k+1]
-  double Sprev = 0.0;
-  const int kend = slen + 3;
-  for (int k = 3; k <= kend; ++k) {
-    const double Yp = limo3_y(Pa, Pb, radd(Pa2, Pb2, one), tlo, thi, esc, mz);
-    const double Ym = limo3_y(Ma, Mb, radd(Ma2, Mb2, one), tlo, thi, esc, mz);
-    const double S = rsub(Yp, Ym, one);
-    if (k > 3 && ((wmask >> (k - 4)) & 1ull))
-      out[(long long)(k - 4) * ostr] = fma(ldk(K_HALF), rsub(Sprev, S, one), -radd(Pa, Mb, one));
-    Sprev = S;
-    if (k < kend) {
-      const double gn = g[k + 1], hn = h[k + 2];
-      Pa = Pb; Pa2 = Pb2; Pb = rsub(gn, gl, one); Pb2 = rmul(Pb, Pb, mz); gl = gn;
-      Mb = Ma; Mb2 = Ma2; Ma = rsub(hn, hl, one); Ma2 = rmul(Ma, Ma, mz); hl = hn;
-    }
-  }
-}
-
-// limo3_sweep that also records, per face and bias, the piece LIMO3 took (limo3_y_sel),
-// faces f0 + k - 3 below fend as flux_sweep_rec records them.
-__device__ __forceinline__ void limo3_sweep_rec(const double* g, const double* h, int slen, double esc,
-                                                unsigned short* tp, unsigned short* tm, int f0, int fend, int fmod,
-                                                double* out, long long ostr, unsigned long long wmask) {
-  const long long tlo = __double_as_longlong((1.0 - 1e-12) / esc), thi = __double_as_longlong((1.0 + 1e-12) / esc);
-  const double one = ldk(K_ONE), mz = ldk(K_MZ);
-  double Pa = rsub(g[2], g[1], one), Pb = rsub(g[3], g[2], one);
-  double Mb = rsub(h[3], h[2], one), Ma = rsub(h[4], h[3], one);
-  double Pa2 = rmul(Pa, Pa, mz), Pb2 = rmul(Pb, Pb, mz), Ma2 = rmul(Ma, Ma, mz), Mb2 = rmul(Mb, Mb, mz);
-  double gl = g[3], hl = h[4];  // the last values read, g[k] and h[k+1]
-  double Sprev = 0.0;
-  const int kend = slen + 3;
-  for (int k = 3; k <= kend; ++k) {
-    int cp, cm;
-    const double Yp = limo3_y_sel(Pa, Pb, radd(Pa2, Pb2, one), tlo, thi, esc, cp, mz);
-    const double Ym = limo3_y_sel(Ma, Mb, radd(Ma2, Mb2, one), tlo, thi, esc, cm, mz);
-    const int f = f0 + k - 3;
-    if (f < fend) {
-      const int fi = f >= fmod ? f - fmod : f;  // face n of a periodic line is face 0
-      tp[fi] = (unsigned short)cp;
-      tm[fi] = (unsigned short)cm;
-    }
-    const double S = rsub(Yp, Ym, one);
-    if (k > 3 && ((wmask >> (k - 4)) & 1ull))
-      out[(long long)(k - 4) * ostr] = fma(ldk(K_HALF), rsub(Sprev, S, one), -radd(Pa, Mb, one));
-    Sprev = S;
-    if (k < kend) {
-      const double gn = g[k + 1], hn = h[k + 2];
-      Pa = Pb; Pa2 = Pb2; Pb = rsub(gn, gl, one); Pb2 = rmul(Pb, Pb, mz); gl = gn;
-      Mb = Ma; Mb2 = Ma2; Ma = rsub(hn, hl, one); Ma2 = rmul(Ma, Ma, mz); hl = hn;
-    }
-  }
-}
-
-// Splitting speed of an item's direction (raised to c_h with GLM) and c_h^2.
-template <int D>
-__device__ __forceinline__ double item_alpha(const FluxParams& p, const FluxItem& it, double& ch2) {
-  const unsigned long long* sk = p.araw + (size_t)it.dom * 4;
-  const unsigned long long* s0 = p.araw0 + (size_t)it.dom * 4;
-  const double ch = p.glm ? glm_speed(s0, p.ndim) : 0.0;
-  ch2 = ch * ch;
-  return imax(bitsd((long long)sk[D]), ch);
-}
-
-// Whether any / every block the item's segment runs through is active.
-__device__ __forceinline__ bool item_live(const FluxParams& p, const FluxItem& item, bool& all_live) {
-  const DomDev& dm = p.doms[item.dom];
-  const int d = item.d;
-  const int bidx[3] = {item.blk % dm.nb[0], (item.blk / dm.nb[0]) % dm.nb[1], item.blk / (dm.nb[0] * dm.nb[1])};
-  const int stride = d == 0 ? 1 : (d == 1 ? dm.nb[0] : dm.nb[0] * dm.nb[1]);
-  const int c0 = bidx[d] * dm.be[d] + item.s0;
-  const int b0 = c0 / dm.be[d], b1 = (c0 + item.slen - 1) / dm.be[d];
-  const int g0 = dm.block0 + item.blk + (b0 - bidx[d]) * stride;
-  bool live = false;
-  all_live = true;
-  for (int b = b0; b <= b1; b++) {
-    const bool a = p.active[g0 + (b - b0) * stride] != 0;
-    live |= a;
-    all_live &= a;
-  }
-  return live;
-}
-
-// Parts of a segment's sweep: a segment of 32 cells or more is swept in np equal parts
-// of at least 16 cells (np the largest divisor of slen up to slen/16), one thread per
-// (variable, part, line); each part recomputes the face at its left end, as a 16-cell
-// segment does. Longer segments then cost less halo work in phase A (6 cells per
-// segment) without leaving phase-B threads idle. Equal parts keep every sweep of an
-// item equally long, which the adaptive sweep's per-face votes need.
-constexpr int kPartMin = 16;
-__device__ __forceinline__ int sweep_parts(int slen) {
-  int np = slen / kPartMin;
-  while (np > 1 && slen % np) np--;
-  return np > 1 ? np : 1;
-}
-
-// The variable whose MP5 sweeps cost clearly most, from the CTA's decaying per-variable
-// counts of limiter faces (cost[v]), or -1: its count must exceed the runner-up's by an
-// eighth (and a few faces).
+// The variable whose MP5 sweeps cost clearly most and into how many times the parts it is
+// worth sweeping it (1, 2 or 4), from the CTA's decaying per-variable counts of limiter
+// faces per full part (cost[v], four times the recent average).
 template <int NV>
-__device__ __forceinline__ int hot_variable(const unsigned* cost) {
-  int h = -1;
+__device__ __forceinline__ int hot_variable(const unsigned* cost, int plen, int& split) {
+  int h = 0;
   unsigned m1 = 0u, m2 = 0u;
 #pragma unroll
   for (int v = 0; v < NV; v++) {
@@ -563,155 +369,118 @@ __device__ __forceinline__ int hot_variable(const unsigned* cost) {
     if (c > m1) { m2 = m1; m1 = c; h = v; }
     else if (c > m2) m2 = c;
   }
-  return m1 > m2 + (m2 >> 3) + 4u ? h : -1;
+  split = m1 < (unsigned)plen || m1 < 2u * m2 ? 1 : (m1 < 2u * (unsigned)plen ? 2 : 4);
+  return h;
 }
 
 // Phase B of a flux item: one thread per (variable, part, line) sweeps the part's faces
-// and stores L_D of its cells (MODE 0: MP5; 1: MP5 recording the limiter pieces;
-// 2: LIMO3; 3: LIMO3 recording its pieces). The loop runs warp by warp: every lane of a
-// warp takes the same number of trips, so that the adaptive sweep's per-face votes see
-// exactly the lanes holding work, all of them sweeping parts of the same length.
-// Balance (MODE 0): a variable whose faces fail the MP5 acceptance test far more often
-// than the others' (noise in one variable, a contact discontinuity) makes its warps the
-// slowest, and the others wait for them at the CTA barrier. The costliest variable `hot`
-// (hot_variable, from the CTA's earlier items) is then swept in twice as many parts of
-// half the length, on twice the warps, when every variable's tasks fill whole warps and
-// the CTA has threads for the extra tasks. A face's value does not depend on the part
-// that computes it, so the results are the same bit for bit. Each warp adds its limiter
-// face count to cost_new[v].
-template <int PHYS, int NV, int D, int MODE>
+// and stores 60 times the flux difference of its cells (fixed_sweep; MODE 0: MP5; 1: MP5
+// recording the limiter pieces; 2: LIMO3; 3: LIMO3 recording its pieces). The loop runs
+// warp by warp: every lane of a warp takes the same number of trips, so that the sweeps'
+// votes see exactly the lanes holding work.
+// Balance (MP5): a face at which the limiter is needed costs about three times another
+// face, so a variable limited at most of its faces (noise, a contact) would keep the CTA's
+// other warps waiting at the barrier. Where the CTA has the threads, that variable
+// (hot_variable, from the CTA's earlier items) is swept in two or four times as many parts.
+// A face's value does not depend on the part that computes it.
+template <int NV, int MODE>
 __device__ __forceinline__ void flux_phase_b(const FluxParams& p, const DomDev& dm, const FluxItem& it,
-                                             const int o[3], bool all_live, const double* sm,
-                                             const unsigned* cost, unsigned* cost_new) {
+                                             const double* sm, const unsigned* cost, unsigned* cost_new) {
   constexpr bool REC = MODE == 1 || MODE == 3;
+  constexpr bool LIMO = MODE >= 2;
+  const int d = it.d;
   const int nl = it.nl, slen = it.slen;
-  const int np = sweep_parts(slen);
-  // MP5 acceptance (f_or - f_i)(f_or - f_mp) <= 1e-10 for F^{+-}; G = 2 F^{+-} and the
-  // doubled relative values of mp5_rel2_r scale the product by 16 (exactly)
-  const double eps16 = 16.0 * 1e-10;
-  constexpr int od1 = D == 0 ? 1 : 0;
-  constexpr int od2 = D == 2 ? 1 : 2;
-  const int f0 = o[D] + it.s0;
-  const long long nlines = (long long)dm.n[od1] * dm.n[od2];
-  const int bstride = D == 0 ? 1 : (D == 1 ? dm.nb[0] : dm.nb[0] * dm.nb[1]);
-  const int bo = it.blk - (o[D] / dm.be[D]) * bstride;  // block index with coordinate D = 0
+  const int np = sweep_parts(slen, p.part), P = nl, SS = tile_stride(slen);
+  const int n = dm.n[d], be = dm.be[d];
+  int o[3];
+  block_coords(dm, it.blk, o);
+  const int bstride = d == 0 ? 1 : (d == 1 ? dm.nb[0] : dm.nb[0] * dm.nb[1]);
+  const int ostr = d == 0 ? 1 : (d == 1 ? dm.n[0] : dm.n[0] * dm.n[1]);
+  const int od = d == 0 ? o[0] : (d == 1 ? o[1] : o[2]);
+  const int f0 = od + it.s0;
+  const unsigned char* row = p.active + dm.block0 + it.blk - (od / be) * bstride;  // blocks along the sweep
   // faces the segment's sweeps record (REC): those it owns, f0 .. f0 + slen - 1, and the
   // face after it where no segment owning that face runs: at an outflow or mirror end of
   // the line, or before a passive block (whose segments the forward pass skips; the
   // adjoint reads the face there). On a periodic line face n is face 0.
   int fend = f0 + slen;
-  {
-    const bool at_end = f0 + slen == dm.n[D];
-    if (at_end && dm.bc[D][1] != 0) fend++;
-    else if (REC && !p.active[dm.block0 + bo + ((at_end ? 0 : f0 + slen) / dm.be[D]) * bstride]) fend++;
+  if constexpr (REC) {
+    const bool at_end = fend == n;
+    if (at_end && dm.bc[d][1] != 0) fend++;
+    else if (!row[((at_end ? 0 : fend) / be) * bstride]) fend++;
   }
-  const int fmod = dm.bc[D][1] == 0 ? dm.n[D] : dm.n[D] + 1;
+  const int fmod = dm.bc[d][1] == 0 ? n : n + 1;
   // cells of the segment inside active blocks (a segment through several blocks may
   // cross a passive one; every line of the item crosses the same blocks)
   unsigned long long wmask = slen >= 64 ? ~0ull : ((1ull << slen) - 1ull);
-  if (!all_live) {
+  if (!(it.live & kLiveAll)) {
     for (int j = 0; j < slen; j++)
-      if (!p.active[dm.block0 + bo + ((o[D] + it.s0 + j) / dm.be[D]) * bstride]) wmask &= ~(1ull << j);
+      if (!row[((f0 + j) / be) * bstride]) wmask &= ~(1ull << j);
   }
-  const long long ostr = D == 0 ? 1 : (D == 1 ? (long long)dm.n[0] : (long long)dm.n[0] * dm.n[1]);
-  double* Ld = p.L[D] + dm.off;
-  const int nh = nl * np;  // tasks per variable
-  int hot = -1;
-  if (MODE == 0 && nh % 32 == 0 && (slen / np) % 2 == 0 && slen / np >= 2 * 8 && nh * (NV + 1) <= (int)blockDim.x)
-    hot = hot_variable<NV>(cost);
-  const int total = nh * NV + (hot >= 0 ? nh : 0);
+  // the two dimensions across the lines
+  const int e1 = d == 0 ? dm.be[1] : dm.be[0];
+  const int s1 = d == 0 ? dm.n[0] : 1, s2 = d == 2 ? dm.n[0] : dm.n[0] * dm.n[1];
+  const int l1 = it.l0 % e1, l2 = it.l0 / e1;
+  const int o1 = d == 0 ? o[1] : o[0], o2 = d == 2 ? o[1] : o[2];
+  double* Ld = p.L[d] + dm.off;
+  const int nh = nl * np;
+  int hot = 0, split = 1;
+  if (!LIMO) {
+    hot = hot_variable<NV>(cost, slen / np, split);
+    while (split > 1 && (nh * split % 32 || slen / (np * split) < 4 || nh * (NV - 1 + split) > (int)blockDim.x))
+      split >>= 1;
+  }
+  const int nhot = split > 1 ? nh * split : 0, total = nh * (NV - (nhot > 0)) + nhot;
   const int lane = threadIdx.x & 31;
-  const double one = ldk(K_ONE);
+  const double rdx = p.limo3_r * dm.dx[d];
   for (int t0 = threadIdx.x - lane; t0 < total; t0 += blockDim.x) {
     const int t = t0 + lane;
     const bool valid = t < total;
-    int plen = slen / np;
-    int pl = 0, v = 0, q = 0;
-    if (valid) {  // a warp holds consecutive parts and lines of one variable
-      if (hot < 0) {
-        pl = t % nl;
-        const int r = t / nl;
-        q = r % np;
-        v = r / np;
-      } else if (t < 2 * nh) {  // the hot variable first: 2 np parts of plen / 2 cells
-        v = hot;
-        plen >>= 1;
-        pl = t % nl;
-        q = t / nl;
-      } else {
-        const int u = t - 2 * nh, vi = u / nh, r = u - vi * nh;
-        v = vi < hot ? vi : vi + 1;
-        pl = r % nl;
-        q = r / nl;
-      }
-    }
-    const int p0 = q * plen;
     const unsigned vm = __ballot_sync(0xffffffffu, valid);
     if (!valid) continue;
-    const double* g = sm + ((0 * NV + v) * p.P + pl) * p.SS + p0;
-    const double* h = sm + ((1 * NV + v) * p.P + pl) * p.SS + p0;
-    const int line = it.l0 + pl;
-    const int a1 = line % dm.be[od1], a2 = line / dm.be[od1];
-    int x[3];
-    x[od1] = o[od1] + a1;
-    x[od2] = o[od2] + a2;
-    x[D] = o[D] + it.s0 + p0;
-    double* out = Ld + (long long)v * dm.ncell + ((long long)x[2] * dm.n[1] + x[1]) * dm.n[0] + x[0];
-    const unsigned long long pmask = (wmask >> p0) & (plen >= 64 ? ~0ull : ((1ull << plen) - 1ull));
-    if constexpr (MODE == 2) {
-      const double rdx = p.limo3_r * dm.dx[D];
-      limo3_sweep(g, h, plen, 0.25 / (rdx * rdx), out, ostr, pmask);
-    } else if constexpr (REC) {
-      const long long ld = (long long)(o[od2] + a2) * dm.n[od1] + (o[od1] + a1);
-      unsigned short* tp = p.tape + dm.tape_off[D] + ((long long)(v * 2 + 0) * nlines + ld) * (dm.n[D] + 1);
-      unsigned short* tm = p.tape + dm.tape_off[D] + ((long long)(v * 2 + 1) * nlines + ld) * (dm.n[D] + 1);
-      // a part records the faces it owns: its left face and interior faces; the
-      // segment's last part also the faces the segment owns at its right end
-      const int fe = q == np - 1 ? fend : f0 + p0 + plen;
-      if constexpr (MODE == 3) {
-        const double rdx = p.limo3_r * dm.dx[D];
-        limo3_sweep_rec(g, h, plen, 0.25 / (rdx * rdx), tp, tm, f0 + p0, fe, fmod, out, ostr, pmask);
-      } else {
-        flux_sweep_rec(g, h, plen, eps16, tp, tm, f0 + p0, fe, fmod, out, ostr, pmask, one);
-      }
+    // lines within parts within variables, the hot variable's parts first
+    int v, r, parts = np;
+    if (t < nhot) {
+      v = hot;
+      r = t;
+      parts *= split;
     } else {
-      const int busy = flux_sweep_adaptive(g, h, plen, eps16, out, ostr, pmask, vm, one);
-      if (lane == __ffs(vm) - 1 && busy) atomicAdd(cost_new + v, (unsigned)busy);
+      v = (t - nhot) / nh;
+      r = t - nhot - v * nh;
+      if (nhot) v += v >= hot;
     }
+    const int q = r / nl, pl = r - q * nl;
+    const int p0 = q * slen / parts, len = (q + 1) * slen / parts - p0;
+    const double* g = sm + (v * P + pl) * SS + p0;
+    int a1 = l1 + pl, a2 = l2;
+    while (a1 >= e1) { a1 -= e1; a2++; }
+    const int x1 = o1 + a1, x2 = o2 + a2;
+    double* out = Ld + (long long)v * dm.ncell + (long long)x1 * s1 + (long long)x2 * s2 + (long long)(f0 + p0) * ostr;
+    const unsigned long long pmask = (wmask >> p0) & (len >= 64 ? ~0ull : ((1ull << len) - 1ull));
+    unsigned short *tp = nullptr, *tm = nullptr;
+    if constexpr (REC) {
+      const int n1 = d == 0 ? dm.n[1] : dm.n[0], n2 = d == 2 ? dm.n[1] : dm.n[2];
+      const long long ld = (long long)x2 * n1 + x1;
+      tp = p.tape + dm.tape_off[d] + ((long long)(v * 2) * n1 * n2 + ld) * (n + 1);
+      tm = tp + (long long)n1 * n2 * (n + 1);
+    }
+    // a part records the faces it owns: its left face and interior faces; the
+    // segment's last part also the faces the segment owns at its right end
+    const int fe = p0 + len == slen ? fend : f0 + p0 + len;
+    const line_t gl = (line_t)__cvta_generic_to_shared(g);
+    const int limited = fixed_sweep<LIMO, REC>(gl, line_at(gl, NV * P * SS), len, 4.0 * rdx * rdx, out, ostr, pmask,
+                                               tp, tm, f0 + p0, fe, fmod, vm);
+    if (!LIMO && limited) atomicMax(cost_new + v, (unsigned)(limited * (parts / np)));
   }
-}
-
-// One flux item by the whole CTA: phase A, barrier, phase B, barrier.
-// cost[0..NV) holds the CTA's decaying per-variable limiter counts, cost[16..16+NV) this
-// item's; every count of the previous item was added before the barrier that ended it.
-template <int PHYS, int NV, int D, int MODE>
-__device__ __forceinline__ void flux_item(const FluxParams& p, const FluxItem& it, double* sm, bool all_live,
-                                          unsigned* cost) {
-  if (threadIdx.x < NV) {
-    const unsigned c = cost[threadIdx.x];
-    cost[threadIdx.x] = c - (c >> 2) + cost[16 + threadIdx.x];
-    cost[16 + threadIdx.x] = 0u;
-  }
-  const DomDev dm = load_dom(p.doms + it.dom);
-  int o[3];
-  block_coords(dm, it.blk, o);
-  double ch2;
-  const double alpha = item_alpha<D>(p, it, ch2);
-  flux_phase_a<PHYS, NV, D>(p, dm, it, o, alpha, ch2, sm, threadIdx.x, blockDim.x);
-  __syncthreads();
-  flux_phase_b<PHYS, NV, D, MODE>(p, dm, it, o, all_live, sm, cost, cost + 16);
-  __syncthreads();
 }
 
 template <int PHYS, int NV, int MODE>
 __global__ void __launch_bounds__(kFluxMaxThreads, 2) flux_kernel(FluxParams p) {
   extern __shared__ double sm[];
   __shared__ int s_it;
-  __shared__ unsigned s_cost[32];
-  if (threadIdx.x < 16) {  // each slot pair is read (flux_item) by the thread that zeroes it
-    s_cost[threadIdx.x] = 0u;
-    s_cost[16 + threadIdx.x] = 0u;
-  }
+  __shared__ unsigned s_cost[32];  // limiter faces per variable: decaying sum, this item's
+  if (threadIdx.x < 32) s_cost[threadIdx.x] = 0u;
+  __syncthreads();
   const int nitems = p.nitems_dev ? *p.nitems_dev : p.nitems;
   int it;
   if (p.counter) {
@@ -725,13 +494,22 @@ __global__ void __launch_bounds__(kFluxMaxThreads, 2) flux_kernel(FluxParams p) 
   constexpr int maxd = PHYS == PH_EULER ? NV - 2 : 3;
   while (it < nitems) {
     const FluxItem item = p.items[p.item0 + it];
-    bool all_live = false;
-    bool live = true;
+    bool live = (item.live & kLiveAny) != 0;
     AMRFD_GUARD(p.err, flux_item_ok(p.doms, p.ndom, p.ndim, p.P, p.SS, item), live = false)
-    live = live && item_live(p, item, all_live);
-    if (live && item.d == 0) flux_item<PHYS, NV, 0, MODE>(p, item, sm, all_live, s_cost);
-    if constexpr (maxd > 1) { if (live && item.d == 1) flux_item<PHYS, NV, (maxd > 1 ? 1 : 0), MODE>(p, item, sm, all_live, s_cost); }
-    if constexpr (maxd > 2) { if (live && item.d == 2) flux_item<PHYS, NV, (maxd > 2 ? 2 : 0), MODE>(p, item, sm, all_live, s_cost); }
+    if (live) {  // phase A, barrier, phase B, barrier
+      const DomDev& dm = p.doms[item.dom];
+      if (threadIdx.x < NV) {  // the last item's counts were added before its last barrier
+        const unsigned c = s_cost[threadIdx.x];
+        s_cost[threadIdx.x] = c - (c >> 2) + s_cost[16 + threadIdx.x];
+        s_cost[16 + threadIdx.x] = 0u;
+      }
+      if (item.d == 0) flux_phase_a<PHYS, NV, 0>(p, dm, item, sm);
+      if constexpr (maxd > 1) { if (item.d == 1) flux_phase_a<PHYS, NV, (maxd > 1 ? 1 : 0)>(p, dm, item, sm); }
+      if constexpr (maxd > 2) { if (item.d == 2) flux_phase_a<PHYS, NV, (maxd > 2 ? 2 : 0)>(p, dm, item, sm); }
+      __syncthreads();
+      flux_phase_b<NV, MODE>(p, dm, item, sm, s_cost, s_cost + 16);
+      __syncthreads();
+    }
     if (p.counter) {
       if (threadIdx.x == 0) s_it = atomicAdd(p.counter, 1);
       __syncthreads();
@@ -890,10 +668,11 @@ __global__ void __launch_bounds__(256) combine_kernel(CombParams p) {
     block_coords(dm, ci.blk, o);
     const double dt = p.dt[ci.dom];
     const double dtb = dt * p.co.b;
-    // L = sum_d (Fsum_{i-1/2} - Fsum_{i+1/2}) / (2 dx_d), Fsum in units of 2 F^
-    const double w0 = dtb * (0.5 / dm.dx[0]);
-    const double w1 = p.ndim > 1 ? dtb * (0.5 / dm.dx[1]) : 0.0;
-    const double w2 = p.ndim > 2 ? dtb * (0.5 / dm.dx[2]) : 0.0;
+    // L = sum_d (Fsum_{i-1/2} - Fsum_{i+1/2}) / (2 dx_d), Fsum in units of 2 F^; the flux pass
+    // stores 60 times the differences
+    const double w0 = dtb * (1.0 / (120.0 * dm.dx[0]));
+    const double w1 = p.ndim > 1 ? dtb * (1.0 / (120.0 * dm.dx[1])) : 0.0;
+    const double w2 = p.ndim > 2 ? dtb * (1.0 / (120.0 * dm.dx[2])) : 0.0;
     const bool damp = PHYS == PH_MHD && p.final_stage && p.glm_cr > 0.0;
     if (damp) {
       if (threadIdx.x == 0) {
@@ -1020,14 +799,45 @@ __global__ void __launch_bounds__(1024) compact_scan_kernel(CompactParams p) {
   if (threadIdx.x == 0) *p.list.count = carry;
 }
 
+// ItemLive bits of a flux item.
+__device__ __forceinline__ unsigned char item_liveness(const CompactParams& p, const FluxItem& item) {
+  const DomDev& dm = p.doms[item.dom];
+  const int d = item.d, be = dm.be[d];
+  const int bstride = d == 0 ? 1 : (d == 1 ? dm.nb[0] : dm.nb[0] * dm.nb[1]);
+  int o[3];
+  block_coords(dm, item.blk, o);
+  const int od = d == 0 ? o[0] : (d == 1 ? o[1] : o[2]);
+  const unsigned char* row = p.active + dm.block0 + item.blk - (od / be) * bstride;
+  const int c0 = od + item.s0, c1 = c0 + item.slen;
+  bool any = false, all = true;
+  for (int b = c0 / be; b <= (c1 - 1) / be; b++) {
+    const bool a = row[b * bstride] != 0;
+    any |= a;
+    all &= a;
+  }
+  bool halo = all;
+  for (int j = 1; j <= kGhost && halo; j++) {
+    unsigned odd;
+    halo = row[halo_cell(dm, d, c0 - j, odd) / be * bstride] && row[halo_cell(dm, d, c1 - 1 + j, odd) / be * bstride];
+  }
+  return (unsigned char)((any ? kLiveAny : 0) | (all ? kLiveAll : 0) | (halo ? kLiveHalo : 0));
+}
+
+// Copies the live groups' items; flux items of every group get their liveness bits first
+// (the plain path runs through the full list).
 __global__ void __launch_bounds__(256) compact_copy_kernel(CompactParams p) {
   const int w = p.list.item_bytes / 4;
-  const unsigned* in = (const unsigned*)p.list.in;
+  unsigned* in = (unsigned*)p.list.in;
   unsigned* out = (unsigned*)p.list.out;
   for (int i = blockIdx.x; i < p.list.ngroups; i += gridDim.x) {
     const int d = p.list.dst[i];
-    if (d < 0) continue;
     const int b = p.list.beg[i], c = p.list.cnt[i];
+    if (p.flux_items) {
+      FluxItem* fi = (FluxItem*)p.list.in + b;
+      for (int t = threadIdx.x; t < c; t += blockDim.x) fi[t].live = item_liveness(p, fi[t]);
+      __syncthreads();
+    }
+    if (d < 0) continue;
     for (int t = threadIdx.x; t < c * w; t += blockDim.x) out[(size_t)d * w + t] = in[(size_t)b * w + t];
   }
 }
@@ -1060,27 +870,26 @@ cudaError_t launch_flux(int physics, int nv, const FluxParams& p, int grid, int 
   return cudaGetLastError();
 }
 
-cudaError_t flux_set_smem(int physics, int nv, size_t smem) {
-#define CALL(PH, NVV)                                                                                     \
-  do {                                                                                                     \
-    cudaError_t e = cudaFuncSetAttribute(flux_kernel<PH, NVV, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                         (int)smem);                                                       \
-    if (e != cudaSuccess) return e;                                                                        \
-    return cudaFuncSetAttribute(flux_kernel<PH, NVV, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-  } while (0)
-  AMRFD_DISPATCH(physics, nv, CALL);
-#undef CALL
-  return cudaSuccess;
+// Lets a kernel take all the dynamic shared memory a block may have. The attribute belongs
+// to the function, not to a handle or a launch: set to one handle's tile it would refuse
+// another handle's larger one.
+cudaError_t allow_smem(const void* fn) {
+  cudaFuncAttributes at;
+  cudaError_t e = cudaFuncGetAttributes(&at, fn);
+  int dev = 0, most = 0;
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)at.sharedSizeBytes);
 }
 
-cudaError_t flux_rec_set_smem(int physics, int nv, size_t smem) {
-#define CALL(PH, NVV)                                                                                     \
-  do {                                                                                                     \
-    cudaError_t e = cudaFuncSetAttribute(flux_kernel<PH, NVV, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                         (int)smem);                                                       \
-    if (e != cudaSuccess) return e;                                                                        \
-    return cudaFuncSetAttribute(flux_kernel<PH, NVV, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-  } while (0)
+cudaError_t flux_allow_smem(int physics, int nv) {
+#define CALL(PH, NVV)                                                                               \
+  for (const void* fn : {(const void*)flux_kernel<PH, NVV, 0>, (const void*)flux_kernel<PH, NVV, 1>, \
+                         (const void*)flux_kernel<PH, NVV, 2>, (const void*)flux_kernel<PH, NVV, 3>}) { \
+    cudaError_t e = allow_smem(fn);                                                                 \
+    if (e != cudaSuccess) return e;                                                                 \
+  }
   AMRFD_DISPATCH(physics, nv, CALL);
 #undef CALL
   return cudaSuccess;

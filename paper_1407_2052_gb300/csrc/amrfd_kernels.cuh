@@ -47,8 +47,8 @@ struct FluxParams {
   const unsigned long long* araw0;  // speeds slot of U^n (GLM speed c_h)
   double gm1;
   int ndim;
-  int P;                        // lines per tile (smem layout)
-  int SS;                       // smem stride of one line (>= max segment + 6, odd)
+  int P, SS;                    // the launch's shared memory holds P lines of stride SS
+  int part;                     // cells of a sweep part (sweep_parts)
   int glm;
   unsigned short* tape;         // limiter pieces of every face (recording pass) or nullptr
   int limo3;                    // reconstruction: 0 MP5, 1 LIMO3
@@ -107,9 +107,11 @@ struct CompactList {
   int* dst;                    // scratch: destination offset per group
   int* count;                  // device: number of items kept
   int item_bytes;
-  const void* in; void* out;
+  void* in; void* out;
 };
 struct CompactParams {
+  const DomDev* doms;
+  int flux_items;              // the list holds FluxItems: keep their liveness bits
   const unsigned char* active;
   CompactList list;
 };
@@ -195,11 +197,11 @@ cudaError_t launch_psi_fac(const unsigned long long* araw0, const double* dt, do
                            double cr, int glm, cudaStream_t s);
 cudaError_t launch_speeds(int physics, int nv, const SpeedParams& p, int grid, int block, cudaStream_t s);
 cudaError_t launch_flux(int physics, int nv, const FluxParams& p, int grid, int block, size_t smem, cudaStream_t s);
-cudaError_t flux_rec_set_smem(int physics, int nv, size_t smem);
 cudaError_t launch_combine(int physics, int nv, const CombParams& p, int grid, int block, cudaStream_t s);
 cudaError_t launch_dt(const DtParams& p, cudaStream_t s);
 cudaError_t launch_compact(const CompactParams& p, cudaStream_t s);
-cudaError_t flux_set_smem(int physics, int nv, size_t smem);
+cudaError_t allow_smem(const void* fn);
+cudaError_t flux_allow_smem(int physics, int nv);
 cudaError_t flux_occupancy(int physics, int nv, int limo3, int block, size_t smem, int* per_sm);
 
 }  // namespace amrfd

@@ -1,0 +1,869 @@
+// amrfd_sweep.cuh -- reconstruction sweeps of the flux pass in exact fixed point.
+//
+// GB300 issues one FP64 warp instruction (an FMA, or a conversion to or from a 64-bit
+// type) per 64 cycles and SM sub-partition, an integer one per 1-2 cycles. The sweeps
+// therefore hold G^{+-} of the line as fixed-point numbers of three signed 22-bit limbs in
+// 32-bit registers: MP5 and LIMO3 are linear in the cells once the limiter's piece is
+// known, with whole coefficients after scaling by 60, so a face flux is a short integer dot
+// product without rounding, and the flux difference of a cell is exact until its one
+// conversion to double. What is decided by comparing (the acceptance test, min, max,
+// median, minmod) is decided in FP32 on differences rounded from the exact ones, with a
+// rigorous error bound; a comparison that FP32 cannot settle is made in exact 128-bit
+// arithmetic.
+//
+// Measured, the whole flux launch (FP64 sweeps before, these after): 1024^2 MHD vortex 768
+// and 360 us, 256^3 MHD blast in noise 16.1 and 10.6 ms (it limits at half its faces; 7.3
+// without), 128^3 MHD blast with LIMO3 2.12 and 0.97 ms. What bounds them now: integer
+// issue (50 to 60 % of the slots, about 490 instructions a face and warp where the limiter
+// runs, 230 where not) and, at 40 %, the FP64 pipe (phase A and one conversion a cell).
+//
+// Scale. A sweep works at one power-of-two scale at which every cell of its part is a whole
+// number: of 66 bits (three limbs) where the cells' exponents span at most 13 binades, else
+// of 110 bits (five limbs, about 1.8 times the work). Nothing is rounded then, so the
+// results do not depend on the scale, hence not on where a sweep starts. A part that spans
+// more than 110 bits is left to exact_cell, which takes every cell by itself and rounds a
+// seven-cell window to the 110-bit unit of its largest value only where the window itself
+// spans more. Values below 2^-988 count as zero, and a window holding a value of 2^1008 or
+// more gives NaN.
+#pragma once
+#include <math.h>
+#include <stdint.h>
+
+#ifdef __CUDACC__
+#include <cuda_runtime.h>
+#define AMRFD_HD __device__ __forceinline__
+#define AMRFD_HD_CALL static __device__ __noinline__
+#define AMRFD_TABLE static __device__ const
+#define AMRFD_ANY(lanes, p) __any_sync((lanes), (p))
+typedef unsigned line_t;  // shared-memory address of a line of doubles
+#else  // a host compiler: one lane, for the tests of the arithmetic
+#define AMRFD_HD static inline
+#define AMRFD_HD_CALL static inline
+#define AMRFD_TABLE static const
+#define AMRFD_ANY(lanes, p) (p)
+typedef const double* line_t;
+struct float4 { float x, y, z, w; };
+static inline float4 make_float4(float x, float y, float z, float w) { return {x, y, z, w}; }
+#endif
+
+namespace amrfd {
+
+constexpr int kLimb = 22;                    // bits per limb
+constexpr int kLimbMask = (1 << kLimb) - 1;
+constexpr int kExpMax = 2030;                // largest biased exponent of a scale's top
+constexpr int kExpUnit = 87;                 // smallest biased exponent of a scale's lob
+
+constexpr float kTiny = 1e-27f;
+
+template <int N>
+struct Limbs {  // a fixed-point number: sum of v[l] 2^(22 l) units
+  int v[N];
+};
+// binades below the top exponent whose 53-bit values are whole numbers of N limbs
+constexpr int room(int n) { return n * kLimb - 53; }
+// floats of differences are in units of 2^float_shift(N) fixed-point units (a top limb has
+// the same weight for every N)
+constexpr int float_shift(int n) { return n * kLimb - 46; }
+
+AMRFD_HD unsigned shf_l(unsigned lo, unsigned hi, int s) {  // high word of (hi:lo) << (s & 31)
+#ifdef __CUDACC__
+  return __funnelshift_l(lo, hi, s);
+#else
+  s &= 31;
+  return s ? (hi << s) | (lo >> (32 - s)) : hi;
+#endif
+}
+AMRFD_HD unsigned shf_r(unsigned lo, unsigned hi, int s) {  // low word of (hi:lo) >> (s & 31)
+#ifdef __CUDACC__
+  return __funnelshift_r(lo, hi, s);
+#else
+  s &= 31;
+  return s ? (lo >> s) | (hi << (32 - s)) : lo;
+#endif
+}
+AMRFD_HD void words(double x, int& hi, unsigned& lo) {
+#ifdef __CUDACC__
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "d"(x));
+#else
+  union { double d; unsigned long long u; } c;
+  c.d = x;
+  hi = (int)(unsigned)(c.u >> 32);
+  lo = (unsigned)c.u;
+#endif
+}
+// The words of element j of a line.
+AMRFD_HD void cell_words(line_t l, int j, int& hi, unsigned& lo) {
+#ifdef __CUDACC__
+  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(lo), "=r"(hi) : "r"(l + 8u * (unsigned)j));
+#else
+  words(l[j], hi, lo);
+#endif
+}
+AMRFD_HD line_t line_at(line_t l, int j) {
+#ifdef __CUDACC__
+  return l + 8u * (unsigned)j;
+#else
+  return l + j;
+#endif
+}
+AMRFD_HD int cell_hi(line_t l, int j) {
+#ifdef __CUDACC__
+  int hi;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(hi) : "r"(l + 8u * (unsigned)j + 4u));
+  return hi;
+#else
+  int hi;
+  unsigned lo;
+  words(l[j], hi, lo);
+  return hi;
+#endif
+}
+AMRFD_HD double from_words(int hi, unsigned lo) {
+#ifdef __CUDACC__
+  double x;
+  asm("mov.b64 %0, {%1, %2};" : "=d"(x) : "r"(lo), "r"(hi));
+  return x;
+#else
+  union { double d; unsigned long long u; } c;
+  c.u = ((unsigned long long)(unsigned)hi << 32) | lo;
+  return c.d;
+#endif
+}
+// 2^e as a double, 0 or infinity beyond the normal range
+AMRFD_HD double pow2d(int e) {
+  const int b = e + 1023;
+  return from_words(b < 1 ? 0 : (b > 2046 ? 0x7ff00000 : b << 20), 0u);
+}
+
+// The limbs of a value whose exponent lies in [lob >> 20, (lob >> 20) + 13] (or zero): the
+// mantissa shifted left. lob = (exponent whose mantissa's last bit is the unit) << 20.
+AMRFD_HD Limbs<3> limbs(int hi, unsigned lo, int lob) {
+  const int x = hi & 0x7fffffff;
+  const int L = (x - lob) >> 20;
+  const unsigned m = ((unsigned)hi & 0xfffffu) | 0x100000u;
+  const int sg = x ? ((hi >> 31) | 1) : 0;
+  const unsigned w0 = shf_l(0u, lo, L), w1 = shf_l(lo, m, L), w2 = shf_l(m, 0u, L);
+  Limbs<3> r;
+  r.v[0] = (int)(w0 & (unsigned)kLimbMask) * sg;
+  r.v[1] = (int)(shf_r(w0, w1, 22) & (unsigned)kLimbMask) * sg;
+  r.v[2] = (int)shf_r(w1, w2, 12) * sg;
+  return r;
+}
+
+// The limbs of any value below the top, rounded to the unit (half away from zero; exact for
+// whole multiples of it).
+AMRFD_HD Limbs<5> limbs_wide(int hi, unsigned lo, int lob) {
+  const int x = hi & 0x7fffffff;
+  int L = (x - lob) >> 20;
+  unsigned long long m = ((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32) | lo;
+  if (L < 0) {
+    m = L < -54 ? 0ull : (m + (1ull << (-L - 1))) >> -L;
+    L = 0;
+  }
+  const int sg = x ? ((hi >> 31) | 1) : 0;
+  Limbs<5> r;
+#pragma unroll
+  for (int l = 0; l < 5; l++) {
+    const int p = kLimb * l - L;  // first bit of the limb in m
+    const unsigned long long t = p >= 0 ? (p < 64 ? m >> p : 0ull) : (p > -kLimb ? m << -p : 0ull);
+    r.v[l] = (int)((unsigned)t & (unsigned)kLimbMask) * sg;
+  }
+  return r;
+}
+template <int N>
+AMRFD_HD Limbs<N> to_limbs(int hi, unsigned lo, int lob) {
+  if constexpr (N == 3) return limbs(hi, lo, lob);
+  else return limbs_wide(hi, lo, lob);
+}
+
+// A difference of two limb numbers (limbs below 2^24, exact in FP32) as a float in units of
+// 2^float_shift(N): relative error <= 2^-23 (a prefix that cancels leaves an exact sum).
+template <int N>
+AMRFD_HD float to_float(const Limbs<N>& d) {
+  float f = (float)d.v[N - 1] * 16777216.0f;  // 2^24
+  float w = 4.0f;
+#pragma unroll
+  for (int l = N - 2; l >= 0; l--) {
+    f = fmaf((float)d.v[l], w, f);
+    w *= 2.384185791015625e-07f;  // 2^-22
+  }
+  return f;
+}
+
+template <int N>
+AMRFD_HD __int128 to_wide(const Limbs<N>& d) {
+  __int128 r = d.v[N - 1];
+#pragma unroll
+  for (int l = N - 2; l >= 0; l--) r = r * (1 << kLimb) + d.v[l];
+  return r;
+}
+
+// The double nearest to a, |a| < 2^125.
+AMRFD_HD double wide_double(__int128 a) {
+  double f = 1.0;
+  const __int128 h = a >> 96;
+  if (h != 0 && h != -1) {  // 72 or more bits remain, the rest in a sticky one
+    a = (a >> 24) | (__int128)((a & 0xffffff) != 0);
+    f = 16777216.0;
+  }
+  return f * fma((double)(long long)(a >> 44), 17592186044416.0, (double)((long long)a & ((1ll << 44) - 1)));
+}
+
+AMRFD_HD double scaled(double x, int adj) {  // x 2^(adj >> 20); normal results
+  int hi;
+  unsigned lo;
+  words(x, hi, lo);
+  return from_words(hi ? hi + adj : 0, lo);
+}
+
+// The double nearest to A - B (ties to even), units of 2^((lob >> 20) - 1075); limbs of the
+// difference below 2^31, the whole below 2^(22 N + 9).
+AMRFD_HD double to_double(const Limbs<3>& A, const Limbs<3>& B, int lob) {
+  const int d0 = A.v[0] - B.v[0], d1 = A.v[1] - B.v[1], d2 = A.v[2] - B.v[2];
+  const long long W = (long long)d1 * (1 << 22) + d0;
+  const int H = d2 + ((int)(W >> 32) >> 12);  // the sum >> 44
+  long long V = (long long)((unsigned long long)W + ((unsigned long long)(unsigned)d2 << 44));
+  int adj = lob - (1075 << 20);
+  if ((unsigned)(H + (1 << 18)) >= (1u << 19)) {
+    // over 62 bits: drop 6 or 13 into a sticky one; 55 or more remain
+    const long long r = W & ((1ll << 44) - 1);
+    const int sh = (unsigned)(H + (1 << 24)) < (1u << 25) ? 6 : 13;
+    V = (long long)((unsigned long long)(long long)H << (44 - sh)) + (r >> sh);
+    V |= (r & ((1ll << sh) - 1)) != 0;
+    adj += sh << 20;
+  }
+#ifdef __CUDACC__
+  const double x = __ll2double_rn(V);
+#else
+  const double x = (double)V;
+#endif
+  return scaled(x, adj);
+}
+AMRFD_HD double to_double(const Limbs<5>& A, const Limbs<5>& B, int lob) {
+  Limbs<5> d;
+#pragma unroll
+  for (int l = 0; l < 5; l++) d.v[l] = A.v[l] - B.v[l];
+  return scaled(wide_double(to_wide(d)), lob - (1075 << 20));
+}
+
+// ----------------------------------------------------------------------- MP5
+// MP5 (Suresh & Huynh 1997) at face i+1/2 from (f_{i-2}, ..., f_{i+2}), in the differences
+// dm = f_{i-1}-f_{i-2}, d0 = f_i-f_{i-1}, d1 = f_{i+1}-f_i, dp = f_{i+2}-f_{i+1} and the
+// curvature-limited second differences Mp (at i+1/2) and Mm (at i-1/2):
+//   f_or - f_i = (11 d0 - 2 dm + 24 d1 - 3 dp)/60,  f_mp - f_i = minmod(d1, 4 d0),
+//   f_ul - f_i = 4 d0,  f_md - f_i = d1/2 - Mp/2,  f_lc - f_i = d0/2 + 4 Mm/3,
+// with the acceptance test (f_or - f_i)(f_or - f_mp) <= 1e-10 (on F^{+-} = G^{+-}/2) and
+// otherwise median(f_or, f_min, f_max).
+// Per face and bias, with the differences of the five stencil cells (the right-biased
+// stencil reversed), every candidate of the limiter is a whole combination of
+// them after scaling by 30: 30 times the doubled value relative to the centre cell,
+//   X = -2 dm + 11 d0 + 24 d1 - 3 dp (unlimited),  0,  60 d1,  30 md = 30 (d1 - Mp),
+//   30 ul = 240 d0,  30 lc = 30 d0 + 80 Mm,
+// Mp, Mm one of 0, ka, kb, 4 ka - kb, 4 kb - ka of two neighbouring curvatures. The rows
+// give each combination less the unlimited one as coefficients of the five cells; a row is
+// the piece of the value and of Mp or Mm, as recorded for the adjoint: 0 X,
+// 1 zero, 2 d1, 3 md, 4 ul, 5 lc, and 0 zero, 1 ka, 2 kb, 3 4 ka - kb, 4 4 kb - ka.
+struct alignas(16) CoefRow { short v[8]; };
+AMRFD_TABLE CoefRow g_mp5_coef[14] = {
+    {{0, 0, 0, 0, 0, 0, 0, 0}},  // 0  unlimited: no correction
+    {{-2, 13, 13, -27, 3, 0, 0, 0}},  // 1  zero
+    {{-2, 13, -47, 33, 3, 0, 0, 0}},  // 2  2 d1
+    {{-2, 13, -17, 3, 3, 0, 0, 0}},  // 3  md, Mp = 0
+    {{-2, -17, 43, -27, 3, 0, 0, 0}},  // 4  md, Mp = kC = d1 - d0
+    {{-2, 13, -47, 63, -27, 0, 0, 0}},  // 5  md, Mp = kR = dp - d1
+    {{-2, -107, 253, -177, 33, 0, 0, 0}},  // 6  md, Mp = 4 kC - kR
+    {{-2, 43, -197, 273, -117, 0, 0, 0}},  // 7  md, Mp = 4 kR - kC
+    {{-2, -227, 253, -27, 3, 0, 0, 0}},  // 8  ul = 8 d0
+    {{-2, -17, 43, -27, 3, 0, 0, 0}},  // 9  lc, Mm = 0
+    {{78, -177, 123, -27, 3, 0, 0, 0}},  // 10  lc, Mm = kL = d0 - dm
+    {{-2, 63, -117, 53, 3, 0, 0, 0}},  // 11  lc, Mm = kC
+    {{318, -737, 523, -107, 3, 0, 0, 0}},  // 12  lc, Mm = 4 kL - kC
+    {{-82, 463, -677, 293, 3, 0, 0, 0}},  // 13  lc, Mm = 4 kC - kL
+};
+constexpr int kD0Code = 3 | (1 << 3);
+// Row of a recorded code (piece | Mp's piece << 3 | Mm's piece << 6).
+AMRFD_HD int mp5_row(int code) {
+  const int s = code & 7;
+  if (s == 3) return 3 + ((code >> 3) & 7);
+  if (s == 5) return 9 + ((code >> 6) & 7);
+  return s == 4 ? 8 : s;
+}
+
+// 30 X, the bound's sum 24|d1| + 11|d0| + 2|dm| + 3|dp|, and t = 30X (30X - 30mp) with a
+// bound B of its error: |t - exact| <= B. Inputs carry a relative error of 2^-23, so 30X
+// is off by at most 2^-21 S, 30 mp by 2^-22 |30 mp|, and t by less than 2^-19 S (S + |30 mp|).
+AMRFD_HD void mp5_test(float dm, float d0, float d1, float dp, float& X, float& t, float& B) {
+  X = fmaf(-3.0f, dp, fmaf(24.0f, d1, fmaf(11.0f, d0, -2.0f * dm)));
+  const float S = fmaf(3.0f, fabsf(dp), fmaf(24.0f, fabsf(d1), fmaf(11.0f, fabsf(d0), 2.0f * fabsf(dm))));
+  const float a = 4.0f * d0;
+  // minmod(d1, 4 d0) = median(0, d1, 4 d0)
+  const float m = fmaxf(fminf(a, 0.0f), fminf(fmaxf(a, 0.0f), d1));
+  t = X * fmaf(-60.0f, m, X);
+  B = (1.9073486328125e-06f * S) * fmaf(60.0f, fabsf(m), S);
+}
+// Whether the acceptance test surely holds, cheaper: with m between 0 and each of d1, 4 d0
+// or outside, t is at most the larger of 30X (30X - 60 d1) and 30X (30X - 240 d0), whose
+// FP32 error is below 0.0091 max|d|^2 (|30X| <= 40 max|d|).
+AMRFD_HD bool mp5_accepts(float dm, float d0, float d1, float dp, float thr_lo) {
+  const float X = fmaf(-3.0f, dp, fmaf(24.0f, d1, fmaf(11.0f, d0, -2.0f * dm)));
+  const float q = fmaxf(X * fmaf(-60.0f, d1, X), X * fmaf(-240.0f, d0, X));
+  const float mx = fmaxf(fmaxf(fabsf(dm), fabsf(d0)), fmaxf(fabsf(d1), fabsf(dp)));
+  return fmaf(0.01171875f * mx, mx, q) < thr_lo;
+}
+
+// minmod4(4 ka - kb, 4 kb - ka, ka, kb) in FP32 and its piece (0 zero, 1 ka, 2 kb,
+// 3 4 ka - kb, 4 4 kb - ka); piece -1 when two candidates lie within tau of the value.
+AMRFD_HD float m4_float(float ka, float kb, float tau, int& piece) {
+  const float c3 = fmaf(4.0f, ka, -kb), c4 = fmaf(4.0f, kb, -ka);
+  float v = 0.0f;
+  if (ka > 0.0f && kb > 0.0f) v = fmaxf(0.0f, fminf(fminf(ka, kb), fminf(c3, c4)));
+  if (ka < 0.0f && kb < 0.0f) v = fminf(0.0f, fmaxf(fmaxf(ka, kb), fmaxf(c3, c4)));
+  const bool n0 = fabsf(v) <= tau, n1 = fabsf(v - ka) <= tau, n2 = fabsf(v - kb) <= tau, n3 = fabsf(v - c3) <= tau,
+             n4 = fabsf(v - c4) <= tau;
+  const int n = n0 + n1 + n2 + n3 + n4;
+  piece = n != 1 ? -1 : (n0 ? 0 : (n1 ? 1 : (n2 ? 2 : (n3 ? 3 : 4))));
+  return v;
+}
+
+// The code of a face that mp5_accepts did not pass, from FP32; -1 when FP32 cannot tell.
+// With s = |dm| + |d0| + |d1| + |dp| every candidate's error is below 2^-18 s (curvatures
+// 2^-22.4 s, 4 ka - kb 2^-20.1 s, 8/3 of that 2^-18.7 s), and min, max and median are
+// 1-Lipschitz, so a piece whose value is the only one within 2^-17 s of the result is the
+// exact selection. Candidates that vanish exactly (equal cells: fronts into a uniform
+// state) count as one.
+AMRFD_HD int mp5_code_float(float dm, float d0, float d1, float dp, float thr_lo) {
+  float X, t, B;
+  mp5_test(dm, d0, d1, dp, X, t, B);
+  if (t + B < thr_lo) return 0;
+  // thr_lo lies below the threshold by 2^-20: its upper side is 2^-19 above that
+  if (!(t - B > fmaxf(thr_lo * 1.0000020f, kTiny))) return -1;
+  const float tau = 7.62939453125e-06f * (fabsf(dm) + fabsf(d0) + fabsf(d1) + fabsf(dp));
+  const float kL = d0 - dm, kC = d1 - d0, kR = dp - d1;
+  int cp, cm;
+  const float Mp = m4_float(kC, kR, tau, cp), Mm = m4_float(kL, kC, tau, cm);
+  const float x = X * (1.0f / 30.0f), c1 = 2.0f * d1, c2 = d1 - Mp, c3 = 8.0f * d0, c4 = fmaf(8.0f / 3.0f, Mm, d0);
+  const float lo = fmaxf(fminf(fminf(0.0f, c1), c2), fminf(fminf(0.0f, c3), c4));
+  const float hi = fminf(fmaxf(fmaxf(0.0f, c1), c2), fmaxf(fmaxf(0.0f, c3), c4));
+  const float r = fmaxf(fminf(x, lo), fminf(fmaxf(x, lo), hi));
+  // exact zeros: d1, and md where besides kC or kR vanishes; d0, and lc where kL or kC does
+  const bool z1 = d1 == 0.0f, z0 = d0 == 0.0f, z2 = z1 && (z0 || dp == 0.0f), z4 = z0 && (z1 || dm == 0.0f);
+  const bool nx = fabsf(x - r) <= tau, n0 = fabsf(r) <= tau, n1 = fabsf(c1 - r) <= tau && !z1,
+             n2 = fabsf(c2 - r) <= tau && !z2, n3 = fabsf(c3 - r) <= tau && !z0, n4 = fabsf(c4 - r) <= tau && !z4;
+  // md with Mp = kC and lc with Mm = 0 are the same combination, d0: recorded as the former
+  const bool same = n2 && n4 && cp == 1 && cm == 0;
+  if (nx + n0 + n1 + n2 + n3 + n4 - same != 1) return -1;
+  if (nx) return 0;
+  if (n0) return 1;
+  if (n1) return 2;
+  if (n3) return 4;
+  if (n2) return cp < 0 ? -1 : 3 | (cp << 3);
+  return cm < 0 ? -1 : (cm == 0 ? kD0Code : 5 | (cm << 6));
+}
+
+// minmod4 in FP32 from curvatures known to ea, eb, and its piece as m4_float's; e: the
+// value's error.
+AMRFD_HD float m4_bounded(float ka, float ea, float kb, float eb, int& piece, float& e) {
+  const float sg = ka < 0.0f ? -1.0f : 1.0f, a = ka * sg, b = kb * sg;
+  piece = 0;
+  e = 0.0f;
+  if (b < -eb || (ea == 0.0f && a == 0.0f) || (eb == 0.0f && b == 0.0f)) return 0.0f;
+  const float c3 = fmaf(4.0f, a, -b), c4 = fmaf(4.0f, b, -a), e3 = fmaf(4.0f, ea, eb), e4 = fmaf(4.0f, eb, ea);
+  if (a > ea && b > eb && (c3 < -1.01f * e3 || c4 < -1.01f * e4)) return 0.0f;
+  const float v = fmaxf(0.0f, fminf(fminf(a, b), fminf(c3, c4)));
+  // the candidate that gave v, if no other one's interval meets its own
+  const bool i1 = v == a, i2 = !i1 && v == b, i3 = !i1 && !i2 && v == c3, i4 = !i1 && !i2 && !i3 && v == c4;
+  const float es = i1 ? ea : (i2 ? eb : (i3 ? e3 : e4));
+  const bool clear = v > es && (i1 || a - v > 1.01f * (ea + es)) && (i2 || b - v > 1.01f * (eb + es)) &&
+                     (i3 || c3 - v > 1.01f * (e3 + es)) && (i4 || c4 - v > 1.01f * (e4 + es));
+  e = 1.01f * (clear ? es : fmaxf(e3, e4));
+  piece = clear ? (i1 ? 1 : (i2 ? 2 : (i3 ? 3 : 4))) : -1;
+  return v * sg;
+}
+
+// A second look at a face mp5_code_float could not settle, with an error for every candidate
+// (differences far smaller than the stencil's largest, as ahead of a front, keep their own
+// precision): the selection is exact when no other candidate's interval meets the selected
+// one's, for which candidates lie above and below it then does not depend on the errors.
+AMRFD_HD int mp5_code_bounded(float dm, float d0, float d1, float dp, float thr_lo) {
+  constexpr float u = 1.1920929e-07f;  // 2^-23, the differences' relative error
+  float X, t, B;
+  mp5_test(dm, d0, d1, dp, X, t, B);
+  if (t + B < thr_lo) return 0;
+  if (!(t - B > fmaxf(thr_lo * 1.0000020f, kTiny))) return -1;
+  const float am = fabsf(dm), a0 = fabsf(d0), a1 = fabsf(d1), ap = fabsf(dp);
+  const float kL = d0 - dm, kC = d1 - d0, kR = dp - d1;
+  int cp, cm;
+  float eP, eM;
+  const float Mp = m4_bounded(kC, 2.0f * u * (a1 + a0), kR, 2.0f * u * (ap + a1), cp, eP);
+  const float Mm = m4_bounded(kL, 2.0f * u * (a0 + am), kC, 2.0f * u * (a1 + a0), cm, eM);
+  float c[6], e[6];
+  c[0] = X * (1.0f / 30.0f);
+  e[0] = 0.15f * u * fmaf(3.0f, ap, fmaf(24.0f, a1, fmaf(11.0f, a0, 2.0f * am)));  // 4 u S / 30
+  c[1] = 0.0f;
+  e[1] = 0.0f;
+  c[2] = 2.0f * d1;
+  e[2] = 2.0f * u * a1;
+  c[3] = d1 - Mp;
+  e[3] = fmaf(2.0f * u, a1 + fabsf(Mp), eP);
+  c[4] = 8.0f * d0;
+  e[4] = 8.0f * u * a0;
+  c[5] = fmaf(8.0f / 3.0f, Mm, d0);
+  e[5] = fmaf(2.0f * u, fmaf(3.0f, fabsf(Mm), a0), 2.7f * eM);
+  const float lo = fmaxf(fminf(fminf(0.0f, c[2]), c[3]), fminf(fminf(0.0f, c[4]), c[5]));
+  const float hi = fminf(fmaxf(fmaxf(0.0f, c[2]), c[3]), fmaxf(fmaxf(0.0f, c[4]), c[5]));
+  const float r = fmaxf(fminf(c[0], lo), fminf(fmaxf(c[0], lo), hi));
+  int s = -1;
+  float es = 0.0f;
+#pragma unroll
+  for (int q = 5; q >= 0; q--)
+    if (c[q] == r) { s = q; es = e[q]; }  // an exact zero by its own name
+  if (r == 0.0f) { s = 1; es = 0.0f; }
+  // md with Mp = kC and lc with Mm = 0 are the same combination, d0
+  const bool same = cp == 1 && cm == 0 && (s == 3 || s == 5);
+  bool clear = s >= 0;
+#pragma unroll
+  for (int q = 0; q < 6; q++) {
+    const bool zero = s == 1 && c[q] == 0.0f && e[q] == 0.0f;  // also exactly zero
+    if (q != s && !zero && !(same && (q == 3 || q == 5))) clear = clear && fabsf(c[q] - r) > 1.01f * (e[q] + es);
+  }
+  if (!clear) return -1;
+  if (s == 3) return cp < 0 ? -1 : 3 | (cp << 3);
+  if (s == 5) return cm < 0 ? -1 : (cm == 0 ? kD0Code : 5 | (cm << 6));
+  return s;
+}
+
+AMRFD_HD __int128 absw(__int128 a) { return a < 0 ? -a : a; }
+
+// minmod4 and its piece, exactly.
+AMRFD_HD __int128 m4_exact(__int128 ka, __int128 kb, int& piece) {
+  piece = 0;
+  if (ka == 0 || kb == 0 || (ka < 0) != (kb < 0)) return 0;
+  const bool as = absw(ka) < absw(kb);
+  const __int128 s = as ? ka : kb, l = as ? kb : ka, t = 4 * s - l;
+  if (t == 0 || (t < 0) != (s < 0)) return 0;
+  if (absw(t) < absw(s)) { piece = as ? 3 : 4; return t; }
+  piece = as ? 1 : 2;
+  return s;
+}
+AMRFD_HD void minw(__int128 a, int ca, __int128 b, int cb, __int128& r, int& cr) {
+  const bool t = a < b;
+  r = t ? a : b;
+  cr = t ? ca : cb;
+}
+AMRFD_HD void maxw(__int128 a, int ca, __int128 b, int cb, __int128& r, int& cr) {
+  const bool t = a < b;
+  r = t ? b : a;
+  cr = t ? cb : ca;
+}
+
+// The code of a face in exact arithmetic. thr: the acceptance threshold on
+// 30X (30X - 30mp) in squared units; the product of the two exact factors, each rounded to
+// FP64, is compared with it.
+AMRFD_HD int mp5_code_exact(const Limbs<5>& em, const Limbs<5>& e0, const Limbs<5>& e1, const Limbs<5>& ep,
+                            double thr) {
+  const __int128 dm = to_wide(em), d0 = to_wide(e0), d1 = to_wide(e1), dp = to_wide(ep);
+  const __int128 X = 24 * d1 + 11 * d0 - 2 * dm - 3 * dp;
+  __int128 mp = 0;
+  if (d1 != 0 && d0 != 0 && (d1 < 0) == (d0 < 0)) mp = absw(d1) < absw(4 * d0) ? d1 : 4 * d0;
+  const __int128 Z = X - 60 * mp;
+  if (X == 0 || Z == 0 || (X < 0) != (Z < 0)) return 0;
+  if (wide_double(absw(X)) * wide_double(absw(Z)) <= thr) return 0;
+  const __int128 kL = d0 - dm, kC = d1 - d0, kR = dp - d1;
+  int cp, cm;
+  const __int128 Mp = m4_exact(kC, kR, cp), Mm = m4_exact(kL, kC, cm);
+  const __int128 md = 30 * (d1 - Mp), lc = 30 * d0 + 80 * Mm, d12 = 60 * d1, ul = 240 * d0;
+  __int128 a, b, lo, hi, t1, t2, t3, r;
+  int ca, cb, cl, ch, c1, c2, c3, code;
+  minw(0, 1, d12, 2, a, ca);
+  minw(a, ca, md, 3, a, ca);
+  minw(0, 1, ul, 4, b, cb);
+  minw(b, cb, lc, 5, b, cb);
+  maxw(a, ca, b, cb, lo, cl);
+  maxw(0, 1, d12, 2, a, ca);
+  maxw(a, ca, md, 3, a, ca);
+  maxw(0, 1, ul, 4, b, cb);
+  maxw(b, cb, lc, 5, b, cb);
+  minw(a, ca, b, cb, hi, ch);
+  minw(X, 0, lo, cl, t1, c1);
+  maxw(X, 0, lo, cl, t2, c2);
+  minw(t2, c2, hi, ch, t3, c3);
+  maxw(t1, c1, t3, c3, r, code);
+  if (r == 0) return 1;  // as the FP32 selection names an exact zero
+  if (code == 3) return 3 | (cp << 3);
+  if (code == 5) return cm == 0 ? kD0Code : 5 | (cm << 6);
+  return code;
+}
+
+// --------------------------------------------------------------------- LIMO3
+// With a, b the differences left and right of the centre cell, 30 times the value:
+// y3 10 a + 20 b, -a/2 -15 a, 2a 60 a, 1.6 b 48 b. Codes, as recorded for the adjoint:
+// piece (0 zero, 1 y3, 2 -a/2, 3 2a, 4 1.6 b) | mode << 3 (0 unlimited, 1 limited, 2 / 3 in
+// the blend band). From FP32, -1 when it cannot tell; thr = 4 (r dx)^2 in squared units.
+AMRFD_HD int limo3_code_float(float a, float b, float thr) {
+  const float s2 = fmaf(a, a, b * b);
+  if (s2 < thr * 0.99999809f) return 0;
+  if (!(s2 > fmaxf(thr * 1.00000191f, kTiny))) return -1;
+  const float sg = b < 0.0f ? -1.0f : 1.0f;
+  const float ap = a * sg, bp = b * sg, y3 = fmaf(2.0f, bp, ap) * (1.0f / 3.0f);
+  const float c2 = -0.5f * ap, c3 = 2.0f * ap, c4 = 1.6f * bp;
+  const float r = fmaxf(0.0f, fminf(y3, fmaxf(c2, fminf(fminf(c3, y3), c4))));
+  const float tau = 3.814697265625e-06f * (fabsf(a) + fabsf(b));  // 2^-18; candidate errors < 2^-20
+  const bool n0 = r <= tau, n1 = fabsf(y3 - r) <= tau, n2 = fabsf(c2 - r) <= tau, n3 = fabsf(c3 - r) <= tau,
+             n4 = fabsf(c4 - r) <= tau;
+  if (n0 + n1 + n2 + n3 + n4 != 1) return -1;
+  return (n0 ? 0 : (n1 ? 1 : (n2 ? 2 : (n3 ? 3 : 4)))) | (1 << 3);
+}
+
+// The code in exact arithmetic; inside the blend band also the value's difference from y3
+// (times 30, whole units). thr as above.
+AMRFD_HD int limo3_code_exact(const Limbs<5>& ea, const Limbs<5>& eb, double thr, __int128* blend) {
+  const __int128 a = to_wide(ea), b = to_wide(eb);
+  const double fa = wide_double(a), fb = wide_double(b), s2 = fma(fa, fa, fb * fb);
+  *blend = 0;
+  if (s2 <= thr * (1.0 - 1e-12)) return 0;
+  const bool neg = b < 0;
+  const __int128 ap = neg ? -a : a, bp = neg ? -b : b, y3 = 10 * ap + 20 * bp;
+  __int128 t;
+  int c;
+  minw(60 * ap, 3, y3, 1, t, c);
+  minw(t, c, 48 * bp, 4, t, c);
+  maxw(-15 * ap, 2, t, c, t, c);
+  minw(y3, 1, t, c, t, c);
+  maxw(0, 0, t, c, t, c);
+  if (s2 >= thr * (1.0 + 1e-12)) return c | (1 << 3);
+  const double z = (s2 / thr - 1.0) * 1e12;
+  const double x = wide_double(t - y3) * (0.5 * (1.0 + z));
+  const long long xh = (long long)(x * 8.470329472543003e-22);  // 2^-70
+  const double xl = x - (double)xh * 1.1805916207174113e+21;
+  const long long xm = (long long)(xl * 5.820766091346741e-11);  // 2^-34
+  const __int128 d = ((__int128)xh << 70) + ((__int128)xm << 34) + (long long)(xl - (double)xm * 17179869184.0);
+  *blend = neg ? -d : d;
+  return c | ((z < 0.0 ? 2 : 3) << 3);
+}
+
+// ------------------------------------------------------------------- sweeps
+// The scale (lob) for N limbs of nc cells of both lines from j on; false when some cell is
+// not a whole multiple of its unit. FINE looks at the mantissas' trailing zeros, else every
+// mantissa counts as 53 bits. bad: a value of 2^1008 or more.
+template <int N, bool FINE>
+AMRFD_HD bool window_scale(line_t gp, line_t gm, int j, int nc, int& lob, bool& bad) {
+  unsigned mx = 0u, mn = 0xffffffffu;  // mn: one less than the smallest key; zero wraps
+  for (int q = 0; q < nc; q++) {
+#pragma unroll
+    for (int s = 0; s < 2; s++) {
+      int hi;
+      unsigned lo = 0u;
+      if (FINE) cell_words(s ? gm : gp, j + q, hi, lo);
+      else hi = cell_hi(s ? gm : gp, j + q);
+      const unsigned a = (unsigned)hi & 0x7fffffffu;
+      mx = a > mx ? a : mx;
+      unsigned k = a;
+      if (FINE && a) {
+        const unsigned m = lo ? lo : ((a & 0xfffffu) | 0x100000u);
+#ifdef __CUDACC__
+        const int z = __ffs((int)m) - 1;
+#else
+        const int z = __builtin_ctz(m);
+#endif
+        k += (unsigned)(z + (lo ? 0 : 32)) << 20;
+      }
+      mn = k - 1u < mn ? k - 1u : mn;
+    }
+  }
+  int top = (int)(mx >> 20);
+  bad = top > kExpMax;
+  top = bad ? kExpMax : top;
+  lob = (top - room(N) < kExpUnit ? kExpUnit : top - room(N)) << 20;
+  const unsigned low = mn == 0xffffffffu ? mn : (mn + 1u) >> 20;
+  return low >= (unsigned)(lob >> 20) && !bad;
+}
+
+// The thresholds of the FP32 decisions in squared floats' units: MP5's acceptance threshold
+// on 30X (30X - 30mp), 2^-20 below; LIMO3's switch. Below kTiny, where products could meet
+// FP32's denormals, -kTiny: FP32 then settles only what lies farther from zero.
+template <bool LIMO, int N>
+AMRFD_HD float float_threshold(int lob, double limo_thr) {
+  const int e = -((lob >> 20) - 1075) - float_shift(N);
+  const float t = (float)(LIMO ? limo_thr * pow2d(e) * pow2d(e) : 1.43999863e-6 * pow2d(2 * e));  // 1.44e-6 (1 - 2^-20)
+  return t < kTiny ? -kTiny : t;
+}
+
+template <bool REC>
+AMRFD_HD void record(unsigned short* tp, unsigned short* tm, int f, int fend, int fmod, int cp, int cm) {
+  if (REC && f < fend) {
+    const int fi = f >= fmod ? f - fmod : f;
+    tp[fi] = (unsigned short)cp;
+    tm[fi] = (unsigned short)cm;
+  }
+}
+
+// The limiter's correction of one stencil as coefficients of its cells (5 with MP5, 3 with
+// LIMO3), from the left (G+) or from the right (G-): the selected combination less the
+// unlimited one.
+template <bool LIMO>
+AMRFD_HD void limited_coefs(int code, int e[5]) {
+  if constexpr (LIMO) {
+    const int piece = code & 7;
+    int ca = 0, cb = 0;  // of a and b
+    if (((code >> 3) & 3) == 1) {
+      ca = piece == 0 || piece == 4 ? -10 : (piece == 2 ? -25 : (piece == 3 ? 50 : 0));
+      cb = piece == 1 ? 0 : (piece == 4 ? 28 : -20);
+    }
+    e[0] = -ca; e[1] = ca - cb; e[2] = cb;
+  } else {
+#ifdef __CUDACC__
+    const uint4 t = *reinterpret_cast<const uint4*>(g_mp5_coef + mp5_row(code));
+    e[0] = (int)(short)t.x; e[1] = (int)t.x >> 16; e[2] = (int)(short)t.y; e[3] = (int)t.y >> 16; e[4] = (int)(short)t.z;
+#else
+    for (int q = 0; q < 5; q++) e[q] = g_mp5_coef[mp5_row(code)].v[q];
+#endif
+  }
+}
+
+// Adds a whole number given limb by limb to F.
+template <int N>
+AMRFD_HD void add_carried(Limbs<N>& F, const long long* s) {
+  long long carry = 0;
+#pragma unroll
+  for (int l = 0; l < N - 1; l++) {
+    const long long t = s[l] + carry;
+    F.v[l] += (int)t & kLimbMask;
+    carry = t >> kLimb;
+  }
+  F.v[N - 1] += (int)(s[N - 1] + carry);
+}
+
+// One cell by itself, its comparisons exact: the cells a sweep could not finish (a
+// comparison FP32 could not settle, a part over more than 110 bits, a value of 2^1008 or
+// more). i: the cell; its window starts at extended cell i + C0.
+template <bool LIMO, bool REC>
+AMRFD_HD void exact_cell(line_t gp, line_t gm, int i, double limo_thr, double* out, bool write, unsigned short* tp,
+                         unsigned short* tm, int f0, int fend, int fmod) {
+  constexpr int NC = LIMO ? 4 : 6;
+  constexpr int C0 = LIMO ? 1 : 0;
+  constexpr int ND = LIMO ? 2 : 4;
+  int lob;
+  bool bad;
+  window_scale<5, true>(gp, gm, i + C0, NC + 1, lob, bad);
+  const int qe = (lob >> 20) - 1075;
+  const float thr_lo = float_threshold<LIMO, 5>(lob, limo_thr);
+  Limbs<5> Fp;
+#pragma unroll 1
+  for (int face = 0; face < 2; face++) {
+    const int c0 = i + C0 + face;  // first cell of the face's window
+    Limbs<5> F = {{0, 0, 0, 0, 0}};
+    int code[2];
+#pragma unroll 1
+    for (int s = 0; s < 2; s++) {
+      // the stencil from the left (G+) or from the right (G-), as cells and differences
+      Limbs<5> D[ND], last;
+#pragma unroll
+      for (int q = 0; q <= ND; q++) {
+        int hi;
+        unsigned lo;
+        cell_words(s ? gm : gp, s ? c0 + NC - 1 - q : c0 + q, hi, lo);
+        const Limbs<5> u = limbs_wide(hi, lo, lob);
+        const int w = LIMO ? (q == 0 ? -10 : (q == 1 ? 50 : 20))
+                           : (q == 0 ? 2 : (q == 1 ? -13 : (q == 2 ? 47 : (q == 3 ? 27 : -3))));
+#pragma unroll
+        for (int l = 0; l < 5; l++) {
+          F.v[l] += w * u.v[l];
+          if (q) D[q - 1].v[l] = u.v[l] - last.v[l];
+        }
+        last = u;
+      }
+      if constexpr (LIMO) {
+        __int128 blend = 0;
+        code[s] = limo3_code_float(to_float(D[0]), to_float(D[1]), thr_lo);
+        if (code[s] < 0) code[s] = limo3_code_exact(D[0], D[1], limo_thr * pow2d(-qe) * pow2d(-qe), &blend);
+#pragma unroll
+        for (int l = 0; l < 5; l++) F.v[l] += l < 4 ? (int)(blend >> (22 * l)) & kLimbMask : (int)(blend >> 88);
+      } else {
+        const float dm = to_float(D[0]), d0 = to_float(D[1]), d1 = to_float(D[2]), dp = to_float(D[3]);
+        code[s] = mp5_code_float(dm, d0, d1, dp, thr_lo);
+        if (code[s] < 0) code[s] = mp5_code_bounded(dm, d0, d1, dp, thr_lo);
+        if (code[s] < 0) code[s] = mp5_code_exact(D[0], D[1], D[2], D[3], 1.44e-6 * pow2d(-2 * qe));
+      }
+      int e[5];
+      limited_coefs<LIMO>(code[s], e);
+      long long a[5] = {0, 0, 0, 0, 0};
+#pragma unroll
+      for (int q = 0; q <= ND; q++) {
+        int hi;
+        unsigned lo;
+        cell_words(s ? gm : gp, s ? c0 + NC - 1 - q : c0 + q, hi, lo);
+        const Limbs<5> u = limbs_wide(hi, lo, lob);
+#pragma unroll
+        for (int l = 0; l < 5; l++) a[l] += (long long)e[q] * u.v[l];
+      }
+      add_carried(F, a);
+    }
+    record<REC>(tp, tm, f0 + i + face, fend, fmod, code[0], code[1]);
+    if (face && write) {
+      const double r = to_double(Fp, F, lob);
+      *out = bad ? from_words(0x7ff80000, 0u) : r;
+    }
+    Fp = F;
+  }
+}
+
+// The faces k = 3..plen+3 of one (line, variable) at the scale lob of N limbs, and the
+// differences of its cells: see fixed_sweep. Returns the cells left to exact_cell; faces:
+// counts those at which the limiter was needed.
+template <bool LIMO, bool REC, int N>
+AMRFD_HD unsigned long long sweep_part(line_t gp, line_t gm, int plen, double limo_thr, double* out, int ostr,
+                                       unsigned long long wmask, unsigned short* tp, unsigned short* tm, int f0,
+                                       int fend, int fmod, int lob, int& limited) {
+  constexpr int NC = LIMO ? 4 : 6;        // cells of a face's window
+  constexpr int C0 = LIMO ? 1 : 0;        // first cell of face 3
+  constexpr int NA = NC - 1;
+  constexpr int ND = LIMO ? 2 : 4;        // differences of a stencil
+  Limbs<N> A[NA];                         // A[n]: the face that lacks n + 1 more cells
+  Limbs<N> gl, hl, Fp;                    // last cell's G+, G-; last face
+  float P[5], M[5];                       // differences of G+, G-, newest last
+  unsigned long long todo = 0ull;
+  const int cend = plen + 6 - C0;
+  const float thr_lo = float_threshold<LIMO, N>(lob, limo_thr);
+#pragma unroll
+  for (int l = 0; l < N; l++) {
+#pragma unroll
+    for (int q = 0; q < NA; q++) A[q].v[l] = 0;
+    gl.v[l] = hl.v[l] = Fp.v[l] = 0;
+  }
+#pragma unroll
+  for (int q = 0; q < 5; q++) P[q] = M[q] = 0.0f;
+#pragma unroll 1
+  for (int c = C0; c < cend; c++) {
+    int ph, mh;
+    unsigned pl, ml;
+    cell_words(gp, c, ph, pl);
+    cell_words(gm, c, mh, ml);
+    const Limbs<N> x = to_limbs<N>(ph, pl, lob), y = to_limbs<N>(mh, ml, lob);
+    Limbs<N> F, dg, dh;
+#pragma unroll
+    for (int l = 0; l < N; l++) {
+      const int g = x.v[l], h = y.v[l];
+      dg.v[l] = g - gl.v[l];
+      dh.v[l] = h - hl.v[l];
+      if constexpr (LIMO) {  // -10 g0 + 50 g1 + 20 g2 + 20 h1 + 50 h2 - 10 h3
+        F.v[l] = A[0].v[l] - 10 * h;
+        A[0].v[l] = A[1].v[l] + 20 * g + 50 * h;
+        A[1].v[l] = A[2].v[l] + 50 * g + 20 * h;
+        A[2].v[l] = -10 * g;
+      } else {  // 2 g0 - 13 g1 + 47 g2 + 27 g3 - 3 g4 - 3 h1 + 27 h2 + 47 h3 - 13 h4 + 2 h5
+        F.v[l] = A[0].v[l] + 2 * h;
+        A[0].v[l] = A[1].v[l] - 3 * g - 13 * h;
+        A[1].v[l] = A[2].v[l] + 27 * g + 47 * h;
+        A[2].v[l] = A[3].v[l] + 47 * g + 27 * h;
+        A[3].v[l] = A[4].v[l] - 13 * g - 3 * h;
+        A[4].v[l] = 2 * g;
+      }
+    }
+    gl = x;
+    hl = y;
+    P[0] = P[1]; P[1] = P[2]; P[2] = P[3]; P[3] = P[4]; P[4] = to_float(dg);
+    M[0] = M[1]; M[1] = M[2]; M[2] = M[3]; M[3] = M[4]; M[4] = to_float(dh);
+    const int i = c - NC - C0;  // the cell left of the face whose last cell is c
+    if (i < -1) continue;
+    // left-biased value of G+, right-biased of G-
+    int cp = 0, cm = 0;
+    bool np, nm;
+    if constexpr (LIMO) {
+      cp = limo3_code_float(P[2], P[3], thr_lo);
+      cm = limo3_code_float(M[4], M[3], thr_lo);
+      np = cp != 0 && cp != 9;  // not the unlimited value
+      nm = cm != 0 && cm != 9;
+    } else {
+      np = !mp5_accepts(P[0], P[1], P[2], P[3], thr_lo);
+      nm = !mp5_accepts(M[4], M[3], M[2], M[1], thr_lo);
+    }
+    if (np || nm) {
+      limited++;
+      // both biases together: the two chains of dependent operations overlap
+      if constexpr (!LIMO) {
+        cp = mp5_code_float(P[0], P[1], P[2], P[3], thr_lo);
+        cm = mp5_code_float(M[4], M[3], M[2], M[1], thr_lo);
+        if (cp < 0 || cm < 0) {
+#pragma unroll 1
+          for (int s = 0; s < 2; s++) {
+            if ((s ? cm : cp) >= 0) continue;
+            const int cd = mp5_code_bounded(s ? M[4] : P[0], s ? M[3] : P[1], s ? M[2] : P[2], s ? M[1] : P[3], thr_lo);
+            if (s) cm = cd;
+            else cp = cd;
+          }
+        }
+      }
+      if (cp < 0 || cm < 0) todo |= i < 0 ? 1ull : 3ull << i;
+      // the stencils again, from the left (G+) and from the right (G-)
+      int e[5], k[5];
+      limited_coefs<LIMO>(cp < 0 ? 0 : cp, e);
+      limited_coefs<LIMO>(cm < 0 ? 0 : cm, k);
+      long long a[N];
+#pragma unroll
+      for (int l = 0; l < N; l++) a[l] = 0;
+#pragma unroll
+      for (int q = 0; q <= ND; q++) {
+        int hi;
+        unsigned lo;
+        cell_words(gp, c - NC + 1 + q, hi, lo);
+        const Limbs<N> u = to_limbs<N>(hi, lo, lob);
+        cell_words(gm, c - q, hi, lo);
+        const Limbs<N> v = to_limbs<N>(hi, lo, lob);
+#pragma unroll
+        for (int l = 0; l < N; l++) a[l] += (long long)e[q] * u.v[l] + (long long)k[q] * v.v[l];
+      }
+      add_carried(F, a);
+    }
+    record<REC>(tp, tm, f0 + i + 1, fend, fmod, cp, cm);
+    if (i >= 0) {
+      if (wmask & 1ull) *out = to_double(Fp, F, lob);
+      out += ostr;
+      wmask >>= 1;
+    }
+    Fp = F;
+  }
+  return todo;
+}
+
+// One (line, variable): the faces k = 3..plen+3 of the line's extended index (cell j = k-1
+// left of face k) and 60 (Fsum_{k-1} - Fsum_k) of its plen <= 64 cells, Fsum = G+_{k-1} +
+// G-_k + (Y+_k + Y-_k)/2, stored to out[i ostr] where wmask has its bit (the factor
+// 1/(120 dx) is applied by the stage combination). Every lane in `lanes` must call this
+// with the same plen. REC records per face and bias the code of the piece the limiter took:
+// face k at index f0 + k - 3 if below fend (face fmod as face 0). Returns the number of
+// faces at which the lane's limiter was needed.
+// A cell enters the partial sums of the faces it belongs to when it is read (a transposed
+// filter), so that only those sums and the last cell stay in registers; the limiter's
+// correction of a face reads its stencil again. What FP32 cannot decide is left to
+// exact_cell after the loop, which keeps that code's registers out of it.
+template <bool LIMO, bool REC>
+AMRFD_HD int fixed_sweep(line_t gp, line_t gm, int plen, double limo_thr, double* out, int ostr,
+                         unsigned long long wmask, unsigned short* tp, unsigned short* tm, int f0, int fend, int fmod,
+                         unsigned lanes) {
+  constexpr int C0 = LIMO ? 1 : 0;
+  const int nc = plen + 6 - 2 * C0;
+  int lob, limited = 0;
+  bool bad;
+  const bool narrow = window_scale<3, false>(gp, gm, C0, nc, lob, bad);
+  unsigned long long todo;
+  if (!AMRFD_ANY(lanes, !narrow)) {
+    todo = sweep_part<LIMO, REC, 3>(gp, gm, plen, limo_thr, out, ostr, wmask, tp, tm, f0, fend, fmod, lob, limited);
+  } else {
+    const bool whole = window_scale<5, true>(gp, gm, C0, nc, lob, bad);
+    todo = sweep_part<LIMO, REC, 5>(gp, gm, plen, limo_thr, out, ostr, wmask, tp, tm, f0, fend, fmod, lob, limited);
+    if (!whole) todo = ~0ull;
+  }
+  if (plen < 64) todo &= (1ull << plen) - 1ull;
+  while (todo) {
+#ifdef __CUDACC__
+    const int i = __ffsll((long long)todo) - 1;
+#else
+    const int i = __builtin_ctzll(todo);
+#endif
+    todo &= todo - 1ull;
+    exact_cell<LIMO, REC>(gp, gm, i, limo_thr, out + (long long)i * ostr, (wmask >> i) & 1ull, tp, tm, f0, fend, fmod);
+  }
+  return limited;
+}
+
+}  // namespace amrfd
