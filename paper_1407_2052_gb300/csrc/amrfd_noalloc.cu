@@ -17,6 +17,7 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "../../include/amrfd.h"
 #include "amrfd_device.cuh"
@@ -42,6 +43,7 @@ struct NaLayout {
   NaDesc dom[kNaMaxDomains];
   int nchunks;                              // chunks of all domains
   unsigned bad[kNaMaxDomains];              // a non-physical cell was met
+  unsigned tlow[kNaMaxDomains][4];          // largest FP32 lower bounds of the speeds (bits)
   unsigned long long slot[kNaMaxDomains][4];
 };
 
@@ -67,7 +69,10 @@ __global__ void __launch_bounds__(256) na_upload_kernel(const __grid_constant__ 
     u.lay->dom[k] = u.d[i];
     u.lay->bad[k] = 0u;
 #pragma unroll
-    for (int q = 0; q < 4; q++) u.lay->slot[k][q] = 0ull;
+    for (int q = 0; q < 4; q++) {
+      u.lay->slot[k][q] = 0ull;
+      u.lay->tlow[k][q] = 0u;
+    }
   }
   if (threadIdx.x == 0) u.lay->nchunks = u.nchunks;
 }
@@ -81,12 +86,20 @@ struct NaParams {
   int ndim;
 };
 
-template <int PHYS, int NV>
+// The exact speed maxima in two launches, as the handle's speeds pass takes them: FP32
+// bounds of every active cell first (EXACT = false), whose largest lower bounds T go to the
+// scratch, then the exact IEEE speeds of only the cells whose upper bound reaches T or that
+// carry no bound (non-physical ones among them, which the exact evaluation flags). A cell
+// costs about 60 FP64 operations exactly, square roots and divisions among them: FP64-bound in
+// one launch (256^3 MHD: 6.89 ms the call, 0.67 in two; 900 blocks of 8^3 to 32^3: 3.78 and
+// 0.48 ms). Now both launches stream the state.
+template <int PHYS, int NV, bool EXACT>
 __global__ void __launch_bounds__(256) na_speeds_kernel(NaParams p) {
   __shared__ unsigned long long red[4][32];
   __shared__ int s_dom;
   __shared__ int s_bad;
   const int nchunks = p.lay->nchunks;
+  const float gam = (float)p.gamma;
   for (int it = blockIdx.x; it < nchunks; it += gridDim.x) {
     if (threadIdx.x == 0) {
       int lo = 0, hi = p.ndom - 1;  // last domain whose first chunk is <= it
@@ -99,23 +112,43 @@ __global__ void __launch_bounds__(256) na_speeds_kernel(NaParams p) {
     }
     __syncthreads();
     const int dmi = s_dom;
-    const NaDesc dm = p.lay->dom[dmi];
+    const NaDesc& dm = p.lay->dom[dmi];
+    const int n0 = dm.n[0], n01 = dm.n[0] * dm.n[1], ncell = dm.ncell;
+    const float rdx[3] = {(float)(1.0 / dm.dx[0]), (float)(1.0 / dm.dx[1]), (float)(1.0 / dm.dx[2])};
+    const double dx[3] = {dm.dx[0], dm.dx[1], dm.dx[2]};
+    float T[4] = {0.f, 0.f, 0.f, 0.f}, lom[4] = {0.f, 0.f, 0.f, 0.f};
+    if (EXACT) {
+#pragma unroll
+      for (int q = 0; q < 4; q++) T[q] = __uint_as_float(p.lay->tlow[dmi][q]);
+    }
     const long long c0 = (long long)(it - dm.chunk0) * kNaChunk;
     unsigned long long mx[4] = {0ull, 0ull, 0ull, 0ull};
     for (int c = threadIdx.x; c < kNaChunk; c += blockDim.x) {
       const long long idx = c0 + c;
-      if (idx >= dm.ncell) break;
-      const int x = (int)(idx % dm.n[0]);
-      const int y = (int)((idx / dm.n[0]) % dm.n[1]);
-      const int z = (int)(idx / ((long long)dm.n[0] * dm.n[1]));
+      if (idx >= ncell) break;
       if (p.active) {
+        const int i = (int)idx, z = i / n01, y = (i - z * n01) / n0, x = i - z * n01 - y * n0;
         const int b = dm.block0 + ((z / dm.be[2]) * dm.nb[1] + y / dm.be[1]) * dm.nb[0] + x / dm.be[0];
         if (!p.active[b]) continue;
       }
       const double* src = p.U + dm.off + idx;
       double u[NV];
 #pragma unroll
-      for (int v = 0; v < NV; v++) u[v] = src[(long long)v * dm.ncell];
+      for (int v = 0; v < NV; v++) u[v] = src[(long long)v * ncell];
+      float up[4], lo[4];
+      bool force;
+      speed_bounds<PHYS, NV>(u, gam, p.ndim, rdx, true, up, lo, force);
+      if (!EXACT) {
+        if (!force) {
+#pragma unroll
+          for (int q = 0; q < 4; q++) lom[q] = fmaxf(lom[q], lo[q]);
+        }
+        continue;
+      }
+      bool cand = force;
+#pragma unroll
+      for (int q = 0; q < 4; q++) cand |= (q == 3 || q < p.ndim) && up[q] >= T[q];
+      if (!cand) continue;
       Prim w;
       if (!cons2prim_exact<PHYS, NV>(u, p.gamma, p.ndim, w)) {
         s_bad = 1;  // benign race: every writer stores 1
@@ -128,11 +161,15 @@ __global__ void __launch_bounds__(256) na_speeds_kernel(NaParams p) {
           const double cd = char_speed_exact<PHYS>(w, p.gamma, d);
           const unsigned long long bb = (unsigned long long)dbits(cd);
           mx[d] = bb > mx[d] ? bb : mx[d];
-          rate = __dadd_rn(rate, __ddiv_rn(cd, dm.dx[d]));
+          rate = __dadd_rn(rate, __ddiv_rn(cd, dx[d]));
         }
       }
       const unsigned long long br = (unsigned long long)dbits(rate);
       mx[3] = br > mx[3] ? br : mx[3];
+    }
+    if (!EXACT) {  // non-negative floats order like their bits
+#pragma unroll
+      for (int q = 0; q < 4; q++) mx[q] = __float_as_uint(lom[q]);
     }
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
 #pragma unroll
@@ -145,7 +182,10 @@ __global__ void __launch_bounds__(256) na_speeds_kernel(NaParams p) {
 #pragma unroll
       for (int q = 0; q < 4; q++) {
         const unsigned long long xw = warp_max_u64(lane < nw ? red[q][lane] : 0ull);
-        if (lane == 0 && xw) atomicMax(&p.lay->slot[dmi][q], xw);
+        if (lane == 0 && xw) {
+          if (EXACT) atomicMax(&p.lay->slot[dmi][q], xw);
+          else atomicMax(&p.lay->tlow[dmi][q], (unsigned)xw);
+        }
       }
       if (lane == 0 && s_bad) atomicOr(&p.lay->bad[dmi], 1u);
     }
@@ -233,7 +273,7 @@ extern "C" int amrfd_dt_noalloc(const amrfd_config* cfg, const amrfd_domain* dom
   if (cfg->dt_scope != AMRFD_DT_PER_DOMAIN && cfg->dt_scope != AMRFD_DT_GLOBAL) return na_fail("bad dt_scope");
   if (!(cfg->gamma > 1.0) || !(cfg->cfl > 0.0)) return na_fail("gamma must exceed 1 and cfl be positive");
   // every descriptor is checked before anything is enqueued
-  long long nch = 0;
+  long long nch = 0, most = 0;
   for (int i = 0; i < ndomain; i++) {
     const amrfd_domain& d = domains[i];
     for (int k = 0; k < 3; k++) {
@@ -245,6 +285,7 @@ extern "C" int amrfd_dt_noalloc(const amrfd_config* cfg, const amrfd_domain* dom
     const long long nc = (long long)d.n[0] * d.n[1] * d.n[2];
     if (nc > 0x7fffffffLL) return na_fail("domain too large");
     nch += (nc + kNaChunk - 1) / kNaChunk;
+    most = nc > most ? nc : most;
     if (nch > 0x7fffffffLL) return na_fail("too many cells");
   }
   const int nv = cfg->physics == AMRFD_EULER ? 2 + cfg->ndim : 9;
@@ -303,11 +344,19 @@ extern "C" int amrfd_dt_noalloc(const amrfd_config* cfg, const amrfd_domain* dom
   int nsm = 0;
   if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return AMRFD_ERR_CUDA;
   const int grid = nch < 8 * nsm ? (nch > 0 ? (int)nch : 1) : 8 * nsm;
-  if (cfg->physics == AMRFD_MHD_GLM) na_speeds_kernel<PH_MHD, 9><<<grid, 256, 0, s>>>(p);
-  else if (nv == 3) na_speeds_kernel<PH_EULER, 3><<<grid, 256, 0, s>>>(p);
-  else if (nv == 4) na_speeds_kernel<PH_EULER, 4><<<grid, 256, 0, s>>>(p);
-  else na_speeds_kernel<PH_EULER, 5><<<grid, 256, 0, s>>>(p);
-  if (cudaGetLastError() != cudaSuccess) return AMRFD_ERR_CUDA;
+  auto speeds = [&](auto exact) {
+    constexpr bool E = decltype(exact)::value;
+    if (cfg->physics == AMRFD_MHD_GLM) na_speeds_kernel<PH_MHD, 9, E><<<grid, 256, 0, s>>>(p);
+    else if (nv == 3) na_speeds_kernel<PH_EULER, 3, E><<<grid, 256, 0, s>>>(p);
+    else if (nv == 4) na_speeds_kernel<PH_EULER, 4, E><<<grid, 256, 0, s>>>(p);
+    else na_speeds_kernel<PH_EULER, 5, E><<<grid, 256, 0, s>>>(p);
+    return cudaGetLastError();
+  };
+  // without the bounds T stays zero and every cell is evaluated exactly: faster where that is
+  // at most two cells a thread of one wave (512-cell tube: 23 us, 27 with the bounds)
+  const bool bounds = most > 512 || nch > nsm;
+  if (bounds && speeds(std::false_type{}) != cudaSuccess) return AMRFD_ERR_CUDA;
+  if (speeds(std::true_type{}) != cudaSuccess) return AMRFD_ERR_CUDA;
   NaDtParams q{};
   q.lay = lay;
   q.dt_out = dt_dev;
