@@ -16,6 +16,7 @@
 
 #include "amrfd_device.cuh"
 #include "amrfd_kernels.cuh"
+#include "amrfd_sweep.cuh"
 
 namespace amrfd {
 
@@ -127,52 +128,6 @@ __device__ __forceinline__ void split_flux_adj(const double* u, double gm1, doub
   }
 }
 
-// Backward of one reconstruction at face k for one variable, from the recorded
-// pieces: rec = (piece of the MP5 value) | (piece of Mp) << 3 | (piece of Mm) << 6.
-// The stencil occupies positions q0..q0+4 of the line window; NEG is the mirrored
-// (right-biased) reconstruction. Accumulates d(value)/dG * gY into gG.
-// The weights of the unlimited value as register operands: 4, 6, 26, 54 (/60).
-struct FaceW {
-  double a4, a6, a26, a54;
-};
-
-template <bool NEG>
-__device__ __forceinline__ void face_adj(double* gG, int q0, double gY, unsigned rec, const FaceW& fw) {
-  if ((rec & 7) == SEL_X) {
-    // the unlimited value f_or (the common case): fixed weights on the five G values,
-    // the differences' coefficients (-4, 22, 48, -6)/60 telescoped (mirrored for NEG)
-    gG[q0] = fma(NEG ? -fw.a6 : fw.a4, gY, gG[q0]);
-    gG[q0 + 1] = fma(NEG ? fw.a54 : -fw.a26, gY, gG[q0 + 1]);
-    gG[q0 + 2] = fma(-fw.a26, gY, gG[q0 + 2]);
-    gG[q0 + 3] = fma(NEG ? -fw.a26 : fw.a54, gY, gG[q0 + 3]);
-    gG[q0 + 4] = fma(NEG ? fw.a4 : -fw.a6, gY, gG[q0 + 4]);
-    return;
-  }
-  double gDm, gD0, gD1, gDp, gMp, gMm;
-  if (!NEG) mp5_rel2_grad<false>(rec & 7, gY, gDm, gD0, gD1, gDp, gMp, gMm);
-  else mp5_rel2_grad<true>(rec & 7, gY, gDm, gD0, gD1, gDp, gMp, gMm);
-  // curvatures kL, kC, kR at q0+1, q0+2, q0+3 (line order)
-  double gkL = 0.0, gkC = 0.0, gkR = 0.0, t1, t2;
-  if (!NEG) {
-    dm4_grad((rec >> 6) & 7, gMm, t1, t2); gkL += t1; gkC += t2;  // Mm from (kL, kC)
-    dm4_grad((rec >> 3) & 7, gMp, t1, t2); gkC += t1; gkR += t2;  // Mp from (kC, kR)
-  } else {
-    dm4_grad((rec >> 3) & 7, gMp, t1, t2); gkC += t1; gkL += t2;  // mirrored: Mp from (kC, kL)
-    dm4_grad((rec >> 6) & 7, gMm, t1, t2); gkR += t1; gkC += t2;  // Mm from (kR, kC)
-  }
-  // gradients of the line differences h_j = G[q0+j] - G[q0+j-1], j = 1..4
-  double gh1, gh2, gh3, gh4;
-  if (!NEG) { gh1 = gDm; gh2 = gD0; gh3 = gD1; gh4 = gDp; }
-  else { gh1 = gDp; gh2 = gD1; gh3 = gD0; gh4 = gDm; }
-  // kL = h2 - h1, kC = h3 - h2, kR = h4 - h3
-  gh1 -= gkL; gh2 += gkL - gkC; gh3 += gkC - gkR; gh4 += gkR;
-  gG[q0] -= gh1;
-  gG[q0 + 1] += gh1 - gh2;
-  gG[q0 + 2] += gh2 - gh3;
-  gG[q0 + 3] += gh3 - gh4;
-  gG[q0 + 4] += gh4;
-}
-
 // Whether the block next to block `blk` along d (side -1 or +1) exists and is active
 // (wrapping across periodic faces).
 __device__ __forceinline__ bool nb_active(const DomDev& dm, const unsigned char* active, int blk, int d, int side) {
@@ -193,23 +148,7 @@ __device__ __forceinline__ bool passive_fed(const DomDev& dm, const unsigned cha
   return !active[dm.block0 + blk] && (nb_active(dm, active, blk, d, -1) || nb_active(dm, active, blk, d, 1));
 }
 
-// Backward of one LIMO3 value Y(a, b) at a face from its recorded piece:
-// dY/da, dY/db of the piece. Inside the 2e-12-wide blend band of the switch the exact
-// derivative carries a factor 1e12 through the blend weight; there the piece of the
-// nearer half (unlimited or limited) is taken.
-__device__ __forceinline__ void limo3_piece_grad(unsigned rec, double& ca, double& cb) {
-  const unsigned mode = (rec >> 3) & 3u;
-  if (mode == 0u || mode == 2u) { ca = 1.0 / 3.0; cb = 2.0 / 3.0; return; }
-  switch (rec & 7u) {
-    case 1: ca = 1.0 / 3.0; cb = 2.0 / 3.0; break;  // y3
-    case 2: ca = -0.5; cb = 0.0; break;               // -a/2
-    case 3: ca = 2.0; cb = 0.0; break;                // 2a
-    case 4: ca = 0.0; cb = 1.6; break;                // 1.6 b
-    default: ca = 0.0; cb = 0.0; break;               // zero
-  }
-}
-
-template <int PHYS, int NV, int D>
+template <int PHYS, int NV, int D, bool LIMO>
 __device__ __forceinline__ void adj_item(const AdjFluxParams& p, const FluxItem& it, double* sm) {
   constexpr int od1 = D == 0 ? 1 : 0;
   constexpr int od2 = D == 2 ? 1 : 2;
@@ -226,12 +165,16 @@ __device__ __forceinline__ void adj_item(const AdjFluxParams& p, const FluxItem&
     for (int d = 0; d < p.ndim; d++) ch = imax(ch, bitsd((long long)s0p[d]));
   const double alpha = imax(bitsd((long long)sk[D]), ch);
   const double ch2 = ch * ch;
-  const double w = p.dt[it.dom] * p.b * (0.5 / dm.dx[D]);
+  // the transposed sweeps give 60 times the gradient: w + wl = dt b / (120 dx) to twice the
+  // precision, since the weight's rounding would bias every cell alike
+  const double den = 120.0 * dm.dx[D], rden = 1.0 / den, num = p.dt[it.dom] * p.b;
+  const double w = num * rden;
+  const double wl = (fma(-w, den, num) + (fma(p.dt[it.dom], p.b, -num) - w * fma(120.0, dm.dx[D], -den))) * rden;
   const double pfac = p.psi_fac ? p.psi_fac[it.dom] : 1.0;
   const int nl = it.nl, slen = it.slen, P = p.P, SA = p.SSa, SG = p.SSg;
   const int n = dm.n[D];
   const int s0 = o[D] + it.s0;               // first cell of the segment (domain coordinate)
-  const int WA = slen + 10, WG = slen + 6;
+  const int WG = slen + 6;
   double* gGp = sm;                           // [NV][P][SA] gradient w.r.t. G+ at positions s0-5 ..
   double* gGm = gGp + NV * P * SA;
   double* gh = gGm + NV * P * SA;             // [NV][P][SG] scaled upstream gradient at s0-3 ..
@@ -241,17 +184,10 @@ __device__ __forceinline__ void adj_item(const AdjFluxParams& p, const FluxItem&
   const int bo = it.blk - (o[D] / dm.be[D]) * bstride;  // block index with coordinate D = 0
   // ---- phase A: upstream gradient at s0-3 .. s0+slen+2 (zero beyond an outflow face and
   // at passive cells, whose residual the step does not use)
-  for (int c = threadIdx.x; c < nl * WA; c += blockDim.x) {
-    int pl, q;
-    if (D == 0) { pl = c / WA; q = c - pl * WA; }
-    else { q = c / nl; pl = c - q * nl; }
-#pragma unroll
-    for (int v = 0; v < NV; v++) {
-      gGp[(v * P + pl) * SA + q] = 0.0;
-      gGm[(v * P + pl) * SA + q] = 0.0;
-    }
-    const int r = q - 2;
-    if (r < 0 || r >= WG) continue;
+  for (int c = threadIdx.x; c < nl * WG; c += blockDim.x) {
+    int pl, r;
+    if (D == 0) { pl = c / WG; r = c - pl * WG; }
+    else { r = c / nl; pl = c - r * nl; }
     const int line = it.l0 + pl;
     const int a1 = line % dm.be[od1], a2 = line / dm.be[od1];
     int x[3];
@@ -268,7 +204,8 @@ __device__ __forceinline__ void adj_item(const AdjFluxParams& p, const FluxItem&
     for (int v = 0; v < NV; v++) {
       double gv = 0.0;
       if (live) {
-        gv = p.G[dm.off + idx + (long long)v * dm.ncell] * w;
+        gv = p.G[dm.off + idx + (long long)v * dm.ncell];
+        gv = fma(gv, w, gv * wl);
         if (PHYS == PH_MHD && v == 8) gv *= pfac;
       }
       gh[(v * P + pl) * SG + r] = gv;
@@ -279,45 +216,25 @@ __device__ __forceinline__ void adj_item(const AdjFluxParams& p, const FluxItem&
   int kb = s0 - 2, ke = s0 + slen + 2;
   if (dm.bc[D][0] != 0 && kb < 0) kb = 0;
   if (dm.bc[D][1] != 0 && ke > n) ke = n;
+  // cells whose gradient is used: the segment's and, at a face with ghosts, those
+  const int lo = dm.bc[D][0] != 0 && s0 == 0 ? -3 : 0;
+  const int hi = dm.bc[D][1] != 0 && s0 + slen == n ? slen + 2 : slen - 1;
   const long long nlines = (long long)dm.n[od1] * dm.n[od2];
-  const double one = ldk(K_ONE), half = ldk(K_HALF), mz = ldk(K_MZ);
-  const FaceW fw = {ldk(K_C4), ldk(K_C6), ldk(K_C26), ldk(K_C54)};
-  for (int t = threadIdx.x; t < nl * NV; t += blockDim.x) {
+  const int total = nl * NV, lane = threadIdx.x & 31;
+  for (int t0 = threadIdx.x - lane; t0 < total; t0 += blockDim.x) {
+    const int t = t0 + lane;
+    const unsigned vm = __ballot_sync(0xffffffffu, t < total);
+    if (t >= total) continue;
     const int v = t / nl, pl = t - v * nl;
     double* ggp = gGp + (v * P + pl) * SA;
     double* ggm = gGm + (v * P + pl) * SA;
-    const double* ghl = gh + (v * P + pl) * SG;
     const int line = it.l0 + pl;
     const int a1 = line % dm.be[od1], a2 = line / dm.be[od1];
     const long long ld = (long long)(o[od2] + a2) * dm.n[od1] + (o[od1] + a1);
     const unsigned short* tp = p.tape + dm.tape_off[D] + ((long long)(v * 2 + 0) * nlines + ld) * (n + 1);
-    const unsigned short* tm = p.tape + dm.tape_off[D] + ((long long)(v * 2 + 1) * nlines + ld) * (n + 1);
-    for (int k = kb; k <= ke; k++) {
-      const int qk = k - (s0 - 5);        // position of cell k in the G window
-      const int rk = k - (s0 - 3);        // position of cell k in the gradient window
-      const double gF = rsub(ghl[rk], ghl[rk - 1], one);
-      if (abits(gF) == 0) continue;
-      const int f = (k < 0) ? k + n : (k >= n && dm.bc[D][1] == 0 ? k - n : k);  // periodic faces wrap
-      ggp[qk - 1] = radd(ggp[qk - 1], gF, one);
-      ggm[qk] = radd(ggm[qk], gF, one);
-      const double gY = rmul(half, gF, mz);
-      if (p.limo3) {
-        // F = G+_{k-1} + G-_k + (Y+ - Y-)/2: Y+ of a = G+_{k-1} - G+_{k-2}, b = G+_k - G+_{k-1};
-        // Y- of a = G-_{k+1} - G-_k, b = G-_k - G-_{k-1}
-        double ca, cb;
-        limo3_piece_grad(tp[f], ca, cb);
-        ggp[qk - 2] -= ca * gY;
-        ggp[qk - 1] += (ca - cb) * gY;
-        ggp[qk] += cb * gY;
-        limo3_piece_grad(tm[f], ca, cb);
-        ggm[qk + 1] -= ca * gY;
-        ggm[qk] += (ca - cb) * gY;
-        ggm[qk - 1] += cb * gY;
-      } else {
-        face_adj<false>(ggp, qk - 3, gY, tp[f], fw);  // + stencil: cells k-3 .. k+1, centre k-1
-        face_adj<true>(ggm, qk - 2, gY, tm[f], fw);   // - stencil: cells k-2 .. k+2, centre k
-      }
-    }
+    const TapeLine tape = {tp, tp + nlines * (n + 1), s0, n, dm.bc[D][1] == 0};
+    adjoint_sweep<LIMO>((line_t)__cvta_generic_to_shared(gh + (v * P + pl) * SG), slen, tape, kb - s0, ke - s0, lo, hi,
+                        ggp, ggm, vm);
     // outflow: ghost copies of an edge cell fold back into it
     if (dm.bc[D][0] == 1 && s0 == 0) {
       const int q0 = 5;  // position of cell 0
@@ -376,7 +293,7 @@ __device__ __forceinline__ void adj_item(const AdjFluxParams& p, const FluxItem&
   __syncthreads();
 }
 
-template <int PHYS, int NV>
+template <int PHYS, int NV, bool LIMO>
 __global__ void __launch_bounds__(256) adj_flux_kernel(AdjFluxParams p) {
   extern __shared__ double sm[];
   constexpr int maxd = PHYS == PH_EULER ? NV - 2 : 3;
@@ -387,9 +304,9 @@ __global__ void __launch_bounds__(256) adj_flux_kernel(AdjFluxParams p) {
       const DomDev& dm = p.doms[item.dom];
       if (!p.active[dm.block0 + item.blk] && !passive_fed(dm, p.active, item.blk, item.d)) continue;
     }
-    if (item.d == 0) adj_item<PHYS, NV, 0>(p, item, sm);
-    if constexpr (maxd > 1) { if (item.d == 1) adj_item<PHYS, NV, 1>(p, item, sm); }
-    if constexpr (maxd > 2) { if (item.d == 2) adj_item<PHYS, NV, 2>(p, item, sm); }
+    if (item.d == 0) adj_item<PHYS, NV, 0, LIMO>(p, item, sm);
+    if constexpr (maxd > 1) { if (item.d == 1) adj_item<PHYS, NV, 1, LIMO>(p, item, sm); }
+    if constexpr (maxd > 2) { if (item.d == 2) adj_item<PHYS, NV, 2, LIMO>(p, item, sm); }
   }
 }
 
@@ -498,15 +415,19 @@ __global__ void psi_fac_kernel(const unsigned long long* araw0, const double* dt
     else return cudaErrorInvalidValue;                                      \
   } while (0)
 
+cudaError_t adj_flux_allow_smem(int physics, int nv, int limo3) {
+#define CALL(PH, NVV)                                                                   \
+  return allow_smem(limo3 ? (const void*)adj_flux_kernel<PH, NVV, true> : (const void*)adj_flux_kernel<PH, NVV, false>)
+  AMRFD_DISPATCH_ADJ(physics, nv, CALL);
+#undef CALL
+  return cudaSuccess;
+}
+
 cudaError_t launch_adj_flux(int physics, int nv, const AdjFluxParams& p, int grid, int block, size_t smem,
                             cudaStream_t s) {
-#define CALL(PH, NVV)                                                                                      \
-  {                                                                                                        \
-    cudaError_t e = cudaFuncSetAttribute(adj_flux_kernel<PH, NVV>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                         (int)smem);                                                       \
-    if (e != cudaSuccess) return e;                                                                        \
-    adj_flux_kernel<PH, NVV><<<grid, block, smem, s>>>(p);                                                 \
-  }
+#define CALL(PH, NVV)                                                          \
+  if (p.limo3) adj_flux_kernel<PH, NVV, true><<<grid, block, smem, s>>>(p);    \
+  else adj_flux_kernel<PH, NVV, false><<<grid, block, smem, s>>>(p)
   AMRFD_DISPATCH_ADJ(physics, nv, CALL);
 #undef CALL
   return cudaGetLastError();

@@ -555,7 +555,7 @@ int enqueue_step(amrfd_handle* h, double* U, const double* dt, cudaStream_t s, b
   CK(cudaMemsetAsync(h->d_tlow, 0, sizeof(unsigned) * h->ns * h->ndom * 4, s));
   const std::vector<int> live = batched ? std::vector<int>() : live_domains(h);
   // Items differ in cost (limiters): taken from a counter, where blocks take more than one
-  // and one launch covers the pass (96x80x64 Euler blast, 5 stages: 3.85 ms with a fixed
+  // and one launch covers the pass (123x95x78 Euler blast, 4 stages: 3.85 ms with a fixed
   // share per block, 3.10 ms from the counter).
   const bool counted =
       batched || (live.size() == 1 && h->dom_fend[live[0]] - h->dom_fbeg[live[0]] > h->flux_grid);
@@ -943,6 +943,7 @@ int adjoint_prepare(amrfd_handle* h, cudaStream_t s) {
     }
   }
   if (!h->d_adj_items) {
+    CK(adj_flux_allow_smem(h->cfg.physics, h->nv, h->cfg.recon == AMRFD_LIMO3));
     for (int k = 1; k < h->ns; k++) CK(cudaMalloc(&h->d_gstage[k], sizeof(double) * h->nelem));
     CK(cudaMalloc(&h->d_psifac, sizeof(double) * h->ndom));
     CK(cudaMalloc(&h->d_tape, sizeof(unsigned short) * std::max<long long>(1, h->tape_len) * h->ns));

@@ -116,8 +116,8 @@ __device__ __forceinline__ float f32_trunc_abs(long long ax) {
 // constants are read from a mutable device array through an opaque load, so the
 // compiler can neither fold them back into immediates nor read them from the constant
 // bank.
-enum { K_ONE, K_MZ, K_HALF, K_C4, K_C6, K_ZERO, K_C26, K_C54, K_COUNT };
-static __device__ double g_regk[K_COUNT] = {1.0, -0.0, 0.5, 4.0 / 60.0, 6.0 / 60.0, 0.0, 26.0 / 60.0, 54.0 / 60.0};
+enum { K_ONE, K_MZ, K_HALF, K_ZERO, K_COUNT };
+static __device__ double g_regk[K_COUNT] = {1.0, -0.0, 0.5, 0.0};
 
 // Constant K_* as a register value (an opaque load at this point of the code).
 __device__ __forceinline__ double ldk(int i) {
@@ -129,49 +129,6 @@ __device__ __forceinline__ double ldk(int i) {
 __device__ __forceinline__ double radd(double x, double y, double one) { return fma(x, one, y); }
 __device__ __forceinline__ double rsub(double x, double y, double one) { return fma(x, one, -y); }
 __device__ __forceinline__ double rmul(double c, double x, double mz) { return fma(c, x, mz); }
-
-// ------------------------------------------------ MP5's pieces, for the discrete adjoint
-// MP5 (Suresh & Huynh 1997) at face i+1/2 from (f_{i-2}, ..., f_{i+2}), written in
-// differences Dm = f_{i-1}-f_{i-2}, D0 = f_i-f_{i-1}, D1 = f_{i+1}-f_i, Dp = f_{i+2}-f_{i+1}
-// and the curvature-limited second differences Mp (at i+1/2) and Mm (at i-1/2):
-//   f_or - f_i = (11 D0 - 2 Dm + 24 D1 - 3 Dp)/60,  f_mp - f_i = minmod(D1, 4 D0),
-//   f_ul - f_i = 4 D0,  f_md - f_i = D1/2 - Mp/2,  f_lc - f_i = D0/2 + 4 Mm/3,
-// with the acceptance test (f_or - f_i)(f_or - f_mp) <= eps and otherwise
-// median(f_or, f_min, f_max). The sweeps (amrfd_sweep.cuh) record which piece they took; the
-// adjoint works on twice the value, 2 (f_face - f_i), of the splitting G = 2 F^{+-}. NEG is
-// the mirror-image stencil, whose differences are the negatives of the ones used.
-enum { SEL_X = 0, SEL_ZERO = 1, SEL_D1 = 2, SEL_MD = 3, SEL_UL = 4, SEL_LC = 5 };
-
-// Gradient of the MP5 value w.r.t. (Dm, D0, D1, Dp, Mp, Mm) for the piece `code`, times g.
-template <bool NEG>
-__device__ __forceinline__ void mp5_rel2_grad(int code, double g, double& gDm, double& gD0, double& gD1,
-                                              double& gDp, double& gMp, double& gMm) {
-  constexpr double sg = NEG ? -1.0 : 1.0;
-  gDm = gD0 = gD1 = gDp = gMp = gMm = 0.0;
-  switch (code) {
-    case SEL_X:
-      gDm = (-sg * (4.0 / 60.0)) * g;
-      gD0 = (sg * (22.0 / 60.0)) * g;
-      gD1 = (sg * (48.0 / 60.0)) * g;
-      gDp = (-sg * (6.0 / 60.0)) * g;
-      break;
-    case SEL_D1: gD1 = (2.0 * sg) * g; break;
-    case SEL_MD: gD1 = sg * g; gMp = -g; break;
-    case SEL_UL: gD0 = (8.0 * sg) * g; break;
-    case SEL_LC: gD0 = sg * g; gMm = (8.0 / 3.0) * g; break;
-    default: break;
-  }
-}
-
-// Gradient of minmod4(4 ka - kb, 4 kb - ka, ka, kb) for its piece: 0 zero, 1 ka, 2 kb,
-// 3 4 ka - kb, 4 4 kb - ka.
-__device__ __forceinline__ void dm4_grad(int code, double g, double& gka, double& gkb) {
-  gka = gkb = 0.0;
-  if (code == 1) gka = g;
-  else if (code == 2) gkb = g;
-  else if (code == 3) { gka = 4.0 * g; gkb = -g; }
-  else if (code == 4) { gkb = 4.0 * g; gka = -g; }
-}
 
 // Reciprocal of a positive normal double: FP32 seed from the leading bits (integer
 // conversion, MUFU reciprocal) and two Newton steps y <- y + y (1 - x y) in FP64.

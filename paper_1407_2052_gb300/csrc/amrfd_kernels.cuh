@@ -202,6 +202,7 @@ cudaError_t launch_dt(const DtParams& p, cudaStream_t s);
 cudaError_t launch_compact(const CompactParams& p, cudaStream_t s);
 cudaError_t allow_smem(const void* fn);
 cudaError_t flux_allow_smem(int physics, int nv);
+cudaError_t adj_flux_allow_smem(int physics, int nv, int limo3);
 cudaError_t flux_occupancy(int physics, int nv, int limo3, int block, size_t smem, int* per_sm);
 
 }  // namespace amrfd

@@ -170,9 +170,26 @@ AMRFD_HD Limbs<5> limbs_wide(int hi, unsigned lo, int lob) {
   }
   return r;
 }
+// The same as limbs with four limbs: exponents in [lob >> 20, (lob >> 20) + 35].
+AMRFD_HD Limbs<4> limbs4(int hi, unsigned lo, int lob) {
+  const int x = hi & 0x7fffffff;
+  const int L = (x - lob) >> 20;
+  const unsigned m = ((unsigned)hi & 0xfffffu) | 0x100000u;
+  const int sg = x ? ((hi >> 31) | 1) : 0;
+  const unsigned a0 = shf_l(0u, lo, L), a1 = shf_l(lo, m, L), a2 = shf_l(m, 0u, L);  // by L & 31
+  const bool up = L >= 32;
+  const unsigned w0 = up ? 0u : a0, w1 = up ? a0 : a1, w2 = up ? a1 : a2;
+  Limbs<4> r;
+  r.v[0] = (int)(w0 & (unsigned)kLimbMask) * sg;
+  r.v[1] = (int)(shf_r(w0, w1, 22) & (unsigned)kLimbMask) * sg;
+  r.v[2] = (int)(shf_r(w1, w2, 12) & (unsigned)kLimbMask) * sg;
+  r.v[3] = (int)(w2 >> 2) * sg;
+  return r;
+}
 template <int N>
 AMRFD_HD Limbs<N> to_limbs(int hi, unsigned lo, int lob) {
   if constexpr (N == 3) return limbs(hi, lo, lob);
+  else if constexpr (N == 4) return limbs4(hi, lo, lob);
   else return limbs_wide(hi, lo, lob);
 }
 
@@ -238,6 +255,27 @@ AMRFD_HD double to_double(const Limbs<3>& A, const Limbs<3>& B, int lob) {
   const double x = (double)V;
 #endif
   return scaled(x, adj);
+}
+// The same for one number of four limbs, each below 2^31.
+AMRFD_HD double to_double(const Limbs<4>& d, int lob) {
+  const long long W = (long long)d.v[1] * (1 << 22) + d.v[0];
+  const long long X = (long long)d.v[3] * (1 << 22) + d.v[2] + (W >> 44);  // the sum >> 44
+  const unsigned long long r = (unsigned long long)W & ((1ull << 44) - 1);
+  const long long a = X ^ (X >> 63);
+#ifdef __CUDACC__
+  const int nb = 64 - __clzll(a);
+#else
+  const int nb = a ? 64 - __builtin_clzll((unsigned long long)a) : 0;
+#endif
+  const int sh = nb > 18 ? nb - 18 : 0;  // over 62 bits: the rest into a sticky one
+  long long V = (long long)((unsigned long long)X << (44 - sh)) + (long long)(r >> sh);
+  V |= (r & ((1ull << sh) - 1)) != 0;
+#ifdef __CUDACC__
+  const double x = __ll2double_rn(V);
+#else
+  const double x = (double)V;
+#endif
+  return scaled(x, lob - (1075 << 20) + (sh << 20));
 }
 AMRFD_HD double to_double(const Limbs<5>& A, const Limbs<5>& B, int lob) {
   Limbs<5> d;
@@ -544,8 +582,9 @@ AMRFD_HD int limo3_code_exact(const Limbs<5>& ea, const Limbs<5>& eb, double thr
 // ------------------------------------------------------------------- sweeps
 // The scale (lob) for N limbs of nc cells of both lines from j on; false when some cell is
 // not a whole multiple of its unit. FINE looks at the mantissas' trailing zeros, else every
-// mantissa counts as 53 bits. bad: a value of 2^1008 or more.
-template <int N, bool FINE>
+// mantissa counts as 53 bits. bad: a value of 2^1008 or more. HEAD: bits left free above
+// the largest value.
+template <int N, bool FINE, int HEAD = 0>
 AMRFD_HD bool window_scale(line_t gp, line_t gm, int j, int nc, int& lob, bool& bad) {
   unsigned mx = 0u, mn = 0xffffffffu;  // mn: one less than the smallest key; zero wraps
   for (int q = 0; q < nc; q++) {
@@ -573,7 +612,8 @@ AMRFD_HD bool window_scale(line_t gp, line_t gm, int j, int nc, int& lob, bool& 
   int top = (int)(mx >> 20);
   bad = top > kExpMax;
   top = bad ? kExpMax : top;
-  lob = (top - room(N) < kExpUnit ? kExpUnit : top - room(N)) << 20;
+  constexpr int span = room(N) - HEAD;
+  lob = (top - span < kExpUnit ? kExpUnit : top - span) << 20;
   const unsigned low = mn == 0xffffffffu ? mn : (mn + 1u) >> 20;
   return low >= (unsigned)(lob >> 20) && !bad;
 }
@@ -864,6 +904,184 @@ AMRFD_HD int fixed_sweep(line_t gp, line_t gm, int plen, double limo_thr, double
     exact_cell<LIMO, REC>(gp, gm, i, limo_thr, out + (long long)i * ostr, (wmask >> i) & 1ull, tp, tm, f0, fend, fmod);
   }
   return limited;
+}
+
+// ------------------------------------------------------------------- adjoint
+// Transposed sweep of one (line, variable), in the same arithmetic: with the pieces of the
+// forward pass fixed, 60 Fsum_k is a whole combination of the G+- cells, so 60 times the
+// gradient with respect to a cell is a whole combination of the differences gF_k of the
+// upstream gradient over the faces within reach. g: the upstream gradient, g[r] at cell
+// s0 - 3 + r for r = 0..slen+5; faces kb..ke (relative to s0, -2 <= kb, ke <= slen + 2);
+// tp, tm: the recorded codes of face k at index k + fofs, wrapped into [0, n) on a periodic
+// line (wrap). The gradients of cells lo..hi (relative to s0) go to gp, gm[cell + 5], those
+// that no face reaches as zeros.
+// LIMO3's codes inside the blend band stand for the nearer half.
+// A cell's gradient sums up to five faces' differences (twice the largest value) with
+// coefficients of magnitude 2140 together (the largest of each stencil cell over the
+// limiter's pieces: 320, 750, 630, 320, 120), less than 2^13 times the largest value.
+constexpr int kAdjHead = 4;
+
+template <bool LIMO>
+AMRFD_HD int adjoint_code(int code) {
+  if (!LIMO) return code;
+  const int mode = (code >> 3) & 3;
+  return mode == 0 || mode == 2 ? 0 : (code & 7) | (1 << 3);
+}
+
+struct TapeLine {
+  const unsigned short *tp, *tm;
+  int fofs, n;
+  bool wrap;
+};
+AMRFD_HD int tape_index(const TapeLine& t, int k) {
+  const int f = k + t.fofs;
+  return t.wrap ? (f < 0 ? f + t.n : (f >= t.n ? f - t.n : f)) : f;
+}
+
+// One cell by itself (relative to s0), at the scale of the seven values that reach it.
+template <bool LIMO>
+AMRFD_HD void adjoint_cell(line_t g, const TapeLine& t, int kb, int ke, int cell, double* gp, double* gm) {
+  constexpr int NS = LIMO ? 3 : 5;         // cells of a stencil
+  constexpr int off = LIMO ? 2 : 3;        // G+ stencil of face k: cells k - off ..
+  int lob;
+  bool bad;
+  const int r0 = cell < 0 ? 0 : cell, r1 = cell + 6;  // g[r] of cells cell-3 .. cell+3, those there are
+  const int last = ke + 3;
+  window_scale<5, true, kAdjHead>(g, g, r0, (r1 < last ? r1 : last) - r0 + 1, lob, bad);
+  Limbs<5> F[2] = {{{0, 0, 0, 0, 0}}, {{0, 0, 0, 0, 0}}};
+#pragma unroll 1
+  for (int s = 0; s < 2; s++) {
+#pragma unroll 1
+    for (int q = 0; q < NS; q++) {
+      // G+: face whose stencil cell q is this one; G-: counted from the right, cell k + off - 1 - q
+      const int k = s ? cell + q - (off - 1) : cell + off - q;
+      if (k < kb || k > ke) continue;
+      int ah, bh;
+      unsigned al, bl;
+      cell_words(g, k + 3, ah, al);
+      cell_words(g, k + 2, bh, bl);
+      if (((ah ^ bh) | (int)(al ^ bl)) == 0) continue;  // no code where the gradient does not reach
+      const Limbs<5> a = limbs_wide(ah, al, lob), b = limbs_wide(bh, bl, lob);
+      const int f = tape_index(t, k);
+      int e[5];
+      limited_coefs<LIMO>(adjoint_code<LIMO>(s ? t.tm[f] : t.tp[f]), e);
+      const int w = LIMO ? (q == 0 ? -10 : (q == 1 ? 50 : 20))
+                         : (q == 0 ? 2 : (q == 1 ? -13 : (q == 2 ? 47 : (q == 3 ? 27 : -3))));
+      const int c = w + (q == 0 ? e[0] : (q == 1 ? e[1] : (q == 2 ? e[2] : (q == 3 ? e[3] : e[4]))));
+      long long x[5];
+#pragma unroll
+      for (int l = 0; l < 5; l++) x[l] = (long long)c * (a.v[l] - b.v[l]);
+      add_carried(F[s], x);
+    }
+  }
+  const Limbs<5> zero = {{0, 0, 0, 0, 0}};
+  const double nan = from_words(0x7ff80000, 0u);
+  gp[cell + 5] = bad ? nan : to_double(F[0], zero, lob);
+  gm[cell + 5] = bad ? nan : to_double(F[1], zero, lob);
+}
+
+template <int N>
+AMRFD_HD double gradient(const Limbs<N>& d, int lob) {
+  if constexpr (N == 4) return to_double(d, lob);
+  else return to_double(d, Limbs<N>{}, lob);
+}
+
+template <bool LIMO, int N>
+AMRFD_HD void adjoint_part(line_t g, const TapeLine& t, int kb, int ke, int lo, int hi, int lob, double* gp,
+                           double* gm) {
+  constexpr int NS = LIMO ? 3 : 5;
+  constexpr int off = LIMO ? 2 : 3;
+  Limbs<N> P[NS], M[NS], last;             // partial sums of the stencils' cells, leftmost first
+  const Limbs<N> zero = {};
+#pragma unroll
+  for (int q = 0; q < NS; q++) P[q] = M[q] = zero;
+  int h;
+  unsigned w;
+  cell_words(g, kb + 2, h, w);
+  last = to_limbs<N>(h, w, lob);
+  for (int c = lo; c <= kb - off; c++) {   // ghosts that no face reaches
+    gm[c + 5] = 0.0;
+    if (c < kb - off) gp[c + 5] = 0.0;
+  }
+  const int kend = hi + off;               // the face that completes cell hi's G+
+#pragma unroll 1
+  for (int k = kb; k <= kend; k++) {
+    if (k <= ke) {
+      cell_words(g, k + 3, h, w);
+      const Limbs<N> x = to_limbs<N>(h, w, lob);
+      Limbs<N> d;
+#pragma unroll
+      for (int l = 0; l < N; l++) d.v[l] = x.v[l] - last.v[l];
+      last = x;
+      int any = 0;
+#pragma unroll
+      for (int l = 0; l < N; l++) any |= d.v[l];
+      int cp = 0, cm = 0;
+      if (any) {  // a face the gradient does not reach may hold no code (passive blocks)
+        const int f = tape_index(t, k);
+        cp = adjoint_code<LIMO>(t.tp[f]);
+        cm = adjoint_code<LIMO>(t.tm[f]);
+      }
+#pragma unroll
+      for (int l = 0; l < N; l++) {
+        const int x0 = d.v[l];
+        if constexpr (LIMO) {
+          P[0].v[l] -= 10 * x0; P[1].v[l] += 50 * x0; P[2].v[l] += 20 * x0;
+          M[0].v[l] += 20 * x0; M[1].v[l] += 50 * x0; M[2].v[l] -= 10 * x0;
+        } else {
+          P[0].v[l] += 2 * x0; P[1].v[l] -= 13 * x0; P[2].v[l] += 47 * x0; P[3].v[l] += 27 * x0; P[4].v[l] -= 3 * x0;
+          M[0].v[l] -= 3 * x0; M[1].v[l] += 27 * x0; M[2].v[l] += 47 * x0; M[3].v[l] -= 13 * x0; M[4].v[l] += 2 * x0;
+        }
+      }
+      if ((cp | cm) > 0) {
+        int e[5], m[5];
+        limited_coefs<LIMO>(cp, e);
+        limited_coefs<LIMO>(cm, m);
+#pragma unroll
+        for (int q = 0; q < NS; q++) {
+          long long x0[N], x1[N];
+#pragma unroll
+          for (int l = 0; l < N; l++) {
+            x0[l] = (long long)e[q] * d.v[l];
+            x1[l] = (long long)m[NS - 1 - q] * d.v[l];
+          }
+          add_carried(P[q], x0);
+          add_carried(M[q], x1);
+        }
+      }
+    }
+    // G+ of cell k - off and G- of the cell after it are complete
+    const int c = k - off;
+    if (c >= lo) gp[c + 5] = gradient(P[0], lob);
+    if (c + 1 >= lo && c + 1 <= hi) gm[c + 6] = gradient(M[0], lob);
+#pragma unroll
+    for (int q = 0; q < NS - 1; q++) {
+      P[q] = P[q + 1];
+      M[q] = M[q + 1];
+    }
+    P[NS - 1] = M[NS - 1] = zero;
+  }
+}
+
+// Four limbs first (31 binades): an upstream gradient of random numbers spans more than the 9
+// that three would leave in nearly every warp, and the fallback's five limbs and two
+// conversions of 128 bits a cell then cost what the integers save (512^2 MHD, adjoint of one
+// step: 1.68 ms with three limbs, 1.48 with four, 1.77 with the FP64 transposition).
+template <bool LIMO>
+AMRFD_HD void adjoint_sweep(line_t g, int slen, const TapeLine& t, int kb, int ke, int lo, int hi, double* gp,
+                            double* gm, unsigned lanes) {
+  int lob;
+  bool bad;
+  const bool narrow = window_scale<4, false, kAdjHead>(g, g, 0, slen + 6, lob, bad);
+  if (!AMRFD_ANY(lanes, !narrow)) {
+    adjoint_part<LIMO, 4>(g, t, kb, ke, lo, hi, lob, gp, gm);
+    return;
+  }
+  if (window_scale<5, true, kAdjHead>(g, g, 0, slen + 6, lob, bad)) {
+    adjoint_part<LIMO, 5>(g, t, kb, ke, lo, hi, lob, gp, gm);
+  } else {
+    for (int c = lo; c <= hi; c++) adjoint_cell<LIMO>(g, t, kb, ke, c, gp, gm);
+  }
 }
 
 }  // namespace amrfd
