@@ -33,28 +33,13 @@ BYTES_PER_CELL_UPDATE = 64 * NV
 # the three per-direction residuals (3 nv doubles). The kernel also reads five
 # derived quantities per cell (40 B), traffic spent to save FP64 work.
 FLUX_BYTES_PER_CELL = 4 * NV * 8
-# FP64 work of the flux pass per cell and direction (flop = DADD + DMUL + 2 DFMA thread
-# instructions, counted by ncu on the 128^3 blast's first step, 32 lines per tile, with a
-# build whose sums and products were still DADD and DMUL; the kernels now issue them as
-# FMAs by 1 and with -0, the same instruction count, which 2 x DFMA no longer reads as flop):
-# 291.96 at 16-cell segments, 273.17 at 32-cell segments. A segment of S cells computes
-# the split flux of its S + 6 cells and starts its sweeps afresh, so the count is
-# a + b/S; the method's own work (one split flux per cell, one reconstruction per face,
-# no segment overheads) is the limit a = 254.4 of the two measurements. Of b = 601.3,
-# 6 x 57 flop is the halo's split flux (the MHD+GLM flux along one direction, 21 flop,
-# and its split, 18 FMAs) and 259.3 the sweep restart (the extra face and the opening
-# differences), which a segment swept in parts pays per part.
+# FP64 work of the method per cell and direction in the flux pass (flop = DADD + DMUL + 2 DFMA
+# thread instructions; one split flux per cell, one reconstruction per face and bias, no
+# segment overheads), counted by ncu on a build that did all of it in FP64: a + b/S at
+# segments of S cells, a = 254.4. The kernel now does the reconstructions in exact fixed
+# point on the integer units, so this is the work delivered, not the FP64 instructions
+# executed (split flux, conversions).
 FLUX_FLOPS_PER_CELL_DIR = 254.4
-FLUX_FLOP_HALO = 6 * 57.0
-FLUX_FLOP_SWEEP_START = 259.3
-
-
-def flux_flop_executed(seg, part):
-    """FP64 flop per cell and direction the flux pass executes with segments of seg cells
-    swept in parts of part cells."""
-    return FLUX_FLOPS_PER_CELL_DIR + FLUX_FLOP_HALO / seg + FLUX_FLOP_SWEEP_START / part
-
-
 FP64_PEAK_TFLOPS_NOMINAL = 1.25   # GB300 FP64, nominal (context only)
 # DRAM bytes per cell of one flux launch (ncu dram__bytes_read + write of the 128^3 blast's
 # first flux pass, tile 64 x 8 lines x 320 threads, scaled by cells): traffic grows with
@@ -625,16 +610,13 @@ def run_ours(args, rank, world, local_rank):
     hbm_peak = peaks.get("hbm_gbs", 6800.0)
     # the FP64 rate this GPU sustains, measured here (the flux pass runs inside a long step)
     fp64 = A.fp64_peak(seconds=2.0)
-    seg_eff = min(int(s.get_tile()[0]), nside)
-    part_eff = seg_eff // (seg_eff // 16) if seg_eff >= 32 else seg_eff
     achieved = FLUX_FLOPS_PER_CELL_DIR * 3 * ncell / flux_avg_s / 1e12
-    executed = flux_flop_executed(seg_eff, part_eff) * 3 * ncell / flux_avg_s / 1e12
     roof = {"bound": "alu", "unit": "TFLOP/s", "achieved": achieved, "peak": fp64["sustained_tflops"],
             "frac": achieved / fp64["sustained_tflops"], "traffic": FLUX_TRAFFIC_BYTES_PER_CELL * ncell,
             "kernel": "flux_kernel", "launch_ms": flux_avg_s * 1e3,
             "flop_per_cell_dir": FLUX_FLOPS_PER_CELL_DIR,
-            "flop_per_cell_dir_executed": flux_flop_executed(seg_eff, part_eff),
-            "executed_tflops": executed, "executed_frac": executed / fp64["sustained_tflops"],
+            "note": "achieved: the method's FP64 work over the launch time; the reconstructions run in exact fixed "
+                    "point on the integer units, so the FP64 pipe executes less",
             "peak_source": "measured: amrfd_fp64_peak, independent FP64 FMAs on every SM, back to back for 2 s "
                            "(sustained); burst %.3f TFLOP/s" % fp64["burst_tflops"],
             "peak_nominal": FP64_PEAK_TFLOPS_NOMINAL}
