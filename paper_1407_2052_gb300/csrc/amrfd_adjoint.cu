@@ -214,7 +214,7 @@ __device__ __forceinline__ void adj_item(const AdjFluxParams& p, const FluxItem&
   __syncthreads();
   // ---- phase B: one thread per (line, variable) walks the faces within reach, in fixed point
   // on the integer units (512^2 MHD: the launch went from 344 us, bound by FP64 replay of the
-  // pieces, to about 250); phase C's FP64 and the 12 warps an SM holds bound the kernel now
+  // pieces, to about 255); phase C's FP64 and the 12 warps an SM holds bound the kernel now
   int kb = s0 - 2, ke = s0 + slen + 2;
   if (dm.bc[D][0] != 0 && kb < 0) kb = 0;
   if (dm.bc[D][1] != 0 && ke > n) ke = n;

@@ -1066,7 +1066,7 @@ AMRFD_HD void adjoint_part(line_t g, const TapeLine& t, int kb, int ke, int lo, 
 // Four limbs first (31 binades): an upstream gradient of random numbers spans more than the 9
 // that three would leave in nearly every warp, and the fallback's five limbs and two
 // conversions of 128 bits a cell then cost what the integers save (512^2 MHD, adjoint of one
-// step: 1.68 ms with three limbs, 1.48 with four, 1.77 with the FP64 transposition).
+// step: 1.68 ms with three limbs, 1.48 with four, about 1.75 with the FP64 transposition).
 template <bool LIMO>
 AMRFD_HD void adjoint_sweep(line_t g, int slen, const TapeLine& t, int kb, int ke, int lo, int hi, double* gp,
                             double* gm, unsigned lanes) {
