@@ -316,12 +316,13 @@ int configure_tile(amrfd_handle* h, int seg, int lines, int threads) {
 // that fills the GPU with 20 warps per SM; shorter parts, hence shorter chains of dependent
 // faces and more warps, where it does not: a launch then lasts as long as one sweep (128^2
 // Euler blast: 43 us with 4 cells, 95 with whole segments of 16 in FP64; on the 256^3 MHD
-// blast parts of 8 to 12 measured 5 to 15 % slower than 16).
+// blast parts of 8 to 12 measured 5 to 15 % slower than 16). The line for 16 lies at two waves:
+// just above one, 42x36x42 MHD took 1.03 ms a step with parts of 16 and 0.96 with 8.
 int choose_part(const amrfd_handle* h) {
   long long cells = 0;
   for (auto& dm : h->hdom) cells += dm.ncell;
   const long long faces = cells * h->cfg.ndim * h->nv / 32, room = 20LL * h->nsm;
-  return faces >= 16 * room ? 16 : (faces >= 8 * room ? 8 : 4);
+  return faces >= 32 * room ? 16 : (faces >= 8 * room ? 8 : 4);
 }
 
 // Sweeps per line of the longest segment of a dimension, as build_items cuts it.
@@ -356,15 +357,16 @@ int tile_lines(const amrfd_handle* h, int seg, int threads) {
 }
 
 // The default tile. Segments of 32 cells, 16 where the domains are too small to fill the GPU
-// otherwise. 320 threads from sixteen tiles per CTA on (3D blast of 128^3: 1.19 against
-// 1.25 ms per launch with 160; 3D Euler in ragged blocks 0.65 against 0.77), 160 below
-// (512^2: 0.111 against 0.119 ms, the last wave of tiles shorter).
+// otherwise. 320 threads in 3D, where lines abound (whole steps, 320 and 160 threads:
+// 123x95x78 Euler 2.79 and 3.11 ms, 21x168x112 Euler 1.71 and 2.14, 75x62x96 MHD 2.40 and
+// 2.53), and from sixteen tiles per CTA on; 160 below (512^2: 0.111 against 0.119 ms per
+// launch, the last wave of tiles shorter).
 void default_tile(const amrfd_handle* h, int& seg, int& lines, int& threads) {
   seg = h->part == 16 ? 32 : 16;
   lines = tile_lines(h, seg, kFluxMaxThreads);
   long long cells = 0;
   for (auto& dm : h->hdom) cells += dm.ncell;
-  if (cells * h->cfg.ndim / ((long long)seg * lines) >= 32LL * h->nsm) {
+  if ((h->cfg.ndim == 3 && h->part >= 8) || cells * h->cfg.ndim / ((long long)seg * lines) >= 32LL * h->nsm) {
     threads = kFluxMaxThreads;
   } else {
     lines = tile_lines(h, seg, 160);
