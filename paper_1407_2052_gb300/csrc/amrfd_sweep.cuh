@@ -219,9 +219,9 @@ AMRFD_HD __int128 to_wide(const Limbs<N>& d) {
 AMRFD_HD double wide_double(__int128 a) {
   double f = 1.0;
   const __int128 h = a >> 96;
-  if (h != 0 && h != -1) {  // 72 or more bits remain, the rest in a sticky one
-    a = (a >> 24) | (__int128)((a & 0xffffff) != 0);
-    f = 16777216.0;
+  if (h != 0 && h != -1) {  // 64 to 93 bits remain, the rest in a sticky one: a >> 44 is exact
+    a = (a >> 32) | (__int128)((a & 0xffffffffll) != 0);
+    f = 4294967296.0;
   }
   return f * fma((double)(long long)(a >> 44), 17592186044416.0, (double)((long long)a & ((1ll << 44) - 1)));
 }
