@@ -241,47 +241,6 @@ __device__ __forceinline__ int halo_cell(const DomDev& dm, int d, int g, unsigne
   return g;
 }
 
-__device__ __forceinline__ int exponent(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) - 1023; }
-
-// Rounds the G^{+-} that are tiny on their cell's own flux scale to whole multiples of
-// 2^-96 of it: rho a^2 for momentum, sqrt(rho) a^2 and a^3 for B and psi (a the splitting
-// speed, exponents only). Ahead of a front such components fall off by binades per cell
-// down to underflow; whole multiples of one unit keep the sweeps' exact sums within 110
-// bits there. The change is 2^-43 of the scale's FP64 rounding, and components above 2^-43
-// of the scale keep all their bits.
-template <int PHYS, int NV>
-__device__ __forceinline__ void round_tiny(double rho, int ea, double* gp, double* gm) {
-  const int er = exponent(rho);
-  constexpr int m0 = 1, m1 = PHYS == PH_EULER ? NV - 1 : 4;
-  // exponents (biased) below which the last mantissa bit lies under the unit
-  const int tm = min(er + 2 * ea + (1023 + 52 - 96), 2046), tb = min((er >> 1) + 2 * ea + (1023 + 52 - 96), 2046),
-            tp = min((er >> 1) + 3 * ea + (1023 + 52 - 96), 2046);
-  bool any = false;
-#pragma unroll
-  for (int v = m0; v < NV; v++) {
-    if (PHYS == PH_EULER ? v >= m1 : v == 4) continue;
-    const int t = (v < m1 ? tm : (v < 8 ? tb : tp)) << 20;
-    const int a = __double2hiint(gp[v]) & 0x7fffffff, b = __double2hiint(gm[v]) & 0x7fffffff;
-    any |= (unsigned)(a - 1) < (unsigned)(t - 1) || (unsigned)(b - 1) < (unsigned)(t - 1);
-  }
-  if (!any) return;
-#pragma unroll
-  for (int v = m0; v < NV; v++) {
-    if (PHYS == PH_EULER ? v >= m1 : v == 4) continue;
-    const int t = v < m1 ? tm : (v < 8 ? tb : tp);
-#pragma unroll
-    for (int s = 0; s < 2; s++) {
-      double& g = s ? gm[v] : gp[v];
-      const long long x = dbits(g);
-      const int r = t - (int)((x >> 52) & 0x7ff);  // mantissa bits under the unit
-      if (r <= 0) continue;
-      const int k = r < 53 ? r : 53;
-      const long long y = (x + (1ll << (k - 1))) & ~((1ll << (k < 52 ? k : 52)) - 1);
-      g = bitsd(r > 53 ? 0ll : y);
-    }
-  }
-}
-
 // Phase A of a flux item along D: the tile's G^{+-} (lines x segment + halo) into shared
 // memory. FP64-bound: 33 of its ~150 instructions per cell, one per 64 cycles; the index
 // arithmetic keeps no division and no block lookup in the loop (on the 1024^2 vortex the
@@ -296,7 +255,6 @@ __device__ __forceinline__ void flux_phase_a(const FluxParams& p, const DomDev& 
   double ch2;
   const double alpha = item_alpha<D>(p, it, ch2);
   const double gm1 = p.gm1, one = ldk(K_ONE), mz = ldk(K_MZ);
-  const int ea = exponent(alpha);
   const int sx[3] = {1, dm.n[0], dm.n[0] * dm.n[1]};
   int o[3];
   block_coords(dm, it.blk, o);
@@ -347,7 +305,6 @@ __device__ __forceinline__ void flux_phase_a(const FluxParams& p, const DomDev& 
       prim_w<PHYS, NV>(u, gm1, w);
     }
     split_flux_w<PHYS, NV, D>(u, w, alpha, ch2, one, mz, gp, gmn);
-    round_tiny<PHYS, NV>(u[0], ea, gp, gmn);
 #pragma unroll
     for (int v = 0; v < NV; v++) {
       sm[((0 * NV + v) * P + pl) * SS + j] = gp[v];

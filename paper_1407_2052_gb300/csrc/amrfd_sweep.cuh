@@ -20,11 +20,13 @@
 // Scale. A sweep works at one power-of-two scale at which every cell of its part is a whole
 // number: of 66 bits (three limbs) where the cells' exponents span at most 13 binades, else
 // of 110 bits (five limbs, about 1.8 times the work). Nothing is rounded then, so the
-// results do not depend on the scale, hence not on where a sweep starts. A part that spans
-// more than 110 bits is left to exact_cell, which takes every cell by itself and rounds a
-// seven-cell window to the 110-bit unit of its largest value only where the window itself
-// spans more. Values below 2^-988 count as zero, and a window holding a value of 2^1008 or
-// more gives NaN.
+// results do not depend on the scale, hence not on where a sweep starts. Where a part spans
+// more than 110 bits, the cells whose window holds a value that is no whole number are left
+// to exact_cell, which takes each by itself at its own window's scale; where a seven-cell
+// window spans more, it carries what the units of 2^-110 of the largest value leave over as
+// doubles besides (Wide), so that a component that is weak next to a strong one keeps its
+// FP64 precision where the limiter drops the strong one. Values below 2^-1042 count as zero,
+// and a window holding a value that is not finite gives NaN.
 #pragma once
 #include <math.h>
 #include <stdint.h>
@@ -50,7 +52,7 @@ namespace amrfd {
 
 constexpr int kLimb = 22;                    // bits per limb
 constexpr int kLimbMask = (1 << kLimb) - 1;
-constexpr int kExpMax = 2030;                // largest biased exponent of a scale's top
+constexpr int kExpMax = 2030;                // largest biased exponent of a sweep's top
 constexpr int kExpUnit = 87;                 // smallest biased exponent of a scale's lob
 
 constexpr float kTiny = 1e-27f;
@@ -470,63 +472,177 @@ AMRFD_HD int mp5_code_bounded(float dm, float d0, float d1, float dp, float thr_
   return s;
 }
 
-AMRFD_HD __int128 absw(__int128 a) { return a < 0 ? -a : a; }
+// ------------------------------------------------------------- wide numbers
+// h units + r. With RES (a window that spans more than the units reach) r carries what the
+// whole units of each cell left over, as a double of its own: a value far below the unit is
+// then all remainder and keeps its FP64 precision where the limiter drops the large ones.
+// Without RES every cell is a whole number of units and r is not used.
+template <bool RES>
+struct Wide {
+  __int128 h;
+  double r;
+};
+struct Unit {  // of a scale lob: the unit as a double, its reciprocal
+  double u, inv;
+};
+AMRFD_HD Unit unit_of(int lob) { return {pow2d((lob >> 20) - 1075), pow2d(1075 - (lob >> 20))}; }
+
+AMRFD_HD bool any_bits(double x) {  // no FP64 comparison
+  int hi;
+  unsigned lo;
+  words(x, hi, lo);
+  return (hi | (int)lo) != 0;
+}
+// |r| <= unit/2 (or a little more) again, so that h and then r order the numbers.
+template <bool RES>
+AMRFD_HD void carry_units(Wide<RES>& c, const Unit& un) {
+  int hr, hu;
+  unsigned lr, lu;
+  words(c.r, hr, lr);
+  words(un.u, hu, lu);
+  if ((hr & 0x7fffffff) < hu - (1 << 20)) return;
+  const double q = rint(c.r * un.inv);
+  c.h += (long long)q;
+  c.r = fma(-q, un.u, c.r);
+}
+// ca a + cb b
+template <bool RES>
+AMRFD_HD Wide<RES> lin(int ca, const Wide<RES>& a, int cb, const Wide<RES>& b, const Unit& un) {
+  Wide<RES> c;
+  c.h = a.h * ca + b.h * cb;
+  c.r = 0.0;
+  if (RES && (any_bits(a.r) || any_bits(b.r))) {
+    c.r = fma((double)ca, a.r, (double)cb * b.r);
+    carry_units(c, un);
+  }
+  return c;
+}
+template <bool RES>
+AMRFD_HD bool less(const Wide<RES>& a, const Wide<RES>& b) {
+  return a.h < b.h || (RES && a.h == b.h && a.r < b.r);
+}
+template <bool RES>
+AMRFD_HD int sign(const Wide<RES>& a) {
+  if (a.h != 0) return a.h < 0 ? -1 : 1;
+  return RES ? (a.r > 0.0) - (a.r < 0.0) : 0;
+}
+template <bool RES>
+AMRFD_HD Wide<RES> absw(const Wide<RES>& a) {
+  return sign(a) < 0 ? Wide<RES>{-a.h, RES ? -a.r : 0.0} : a;
+}
+// The number as a float in units of 2^float_shift(5): relative error <= 2^-23. small: not zero,
+// but too small for FP32's comparisons.
+template <bool RES>
+AMRFD_HD float wide_float(const Wide<RES>& a, const Unit& un, bool& small) {
+  const __int128 m = a.h < 0 ? -a.h : a.h;
+  float f;
+  if (RES && any_bits(a.r) && m < (1 << 26)) {
+    const double x = (double)(int)m + (a.h < 0 ? -a.r : a.r) * un.inv;
+    f = (float)(x * 0x1p-64);
+    small |= fabsf(f) < 1e-30f;
+  } else {
+    f = (float)(int)(m >> 96) * 0x1p32f;
+    f = fmaf((float)(int)((m >> 72) & 0xffffff), 0x1p8f, f);
+    f = fmaf((float)(int)((m >> 48) & 0xffffff), 0x1p-16f, f);
+    f = fmaf((float)(int)((m >> 24) & 0xffffff), 0x1p-40f, f);
+    f = fmaf((float)(int)(m & 0xffffff), 0x1p-64f, f);
+  }
+  return a.h < 0 ? -f : f;
+}
+template <bool RES>  // in units
+AMRFD_HD double in_units(const Wide<RES>& a, const Unit& un) {
+  return RES ? fma(a.r, un.inv, wide_double(a.h)) : wide_double(a.h);
+}
+// The double nearest to the number, |h| < 2^122; infinity beyond the largest.
+template <bool RES>
+AMRFD_HD double nearest(const Wide<RES>& a, const Unit& un, int lob) {
+  const int e = (lob >> 20) - 1075;
+  if (RES && a.r != 0.0) {
+    if (absw(Wide<false>{a.h, 0.0}).h < (1ll << 53)) return fma((double)(long long)a.h, un.u, a.r);
+    return ldexp(wide_double(4 * a.h + (a.r > 0.0 ? 1 : -1)), e - 2);  // r decides a tie
+  }
+  return ldexp(wide_double(a.h), e);
+}
+// Element j of a line. Cells whose units round: half away from zero.
+template <bool RES>
+AMRFD_HD Wide<RES> wide_cell(line_t l, int j, int lob, const Unit& un) {
+  int hi;
+  unsigned lo;
+  cell_words(l, j, hi, lo);
+  const int L = ((hi & 0x7fffffff) - lob) >> 20;
+  const unsigned long long m = ((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32) | lo;
+  Wide<RES> a = {0, 0.0};
+  if (L >= 0) a.h = (__int128)m << L;
+  else if (L >= -54) a.h = (__int128)((m + (1ull << (-L - 1))) >> -L);
+  if (hi < 0) a.h = -a.h;
+  if (RES && L < 0) a.r = fma(-(double)(long long)a.h, un.u, from_words(hi, lo));
+  return a;
+}
 
 // minmod4 and its piece, exactly.
-AMRFD_HD __int128 m4_exact(__int128 ka, __int128 kb, int& piece) {
+template <bool RES>
+AMRFD_HD Wide<RES> m4_exact(const Wide<RES>& ka, const Wide<RES>& kb, const Unit& un, int& piece) {
+  const Wide<RES> zero = {0, 0.0};
   piece = 0;
-  if (ka == 0 || kb == 0 || (ka < 0) != (kb < 0)) return 0;
-  const bool as = absw(ka) < absw(kb);
-  const __int128 s = as ? ka : kb, l = as ? kb : ka, t = 4 * s - l;
-  if (t == 0 || (t < 0) != (s < 0)) return 0;
-  if (absw(t) < absw(s)) { piece = as ? 3 : 4; return t; }
-  piece = as ? 1 : 2;
-  return s;
+  const int sg = sign(ka);
+  if (sg == 0 || sg != sign(kb)) return zero;
+  const bool as = less(absw(ka), absw(kb));
+  const Wide<RES> s = as ? ka : kb, t = lin(4, s, -1, as ? kb : ka, un);
+  if (sign(t) != sg) return zero;
+  const bool four = less(absw(t), absw(s));
+  piece = four ? (as ? 3 : 4) : (as ? 1 : 2);
+  return four ? t : s;
 }
-AMRFD_HD void minw(__int128 a, int ca, __int128 b, int cb, __int128& r, int& cr) {
-  const bool t = a < b;
+template <bool RES>
+AMRFD_HD void minw(const Wide<RES>& a, int ca, const Wide<RES>& b, int cb, Wide<RES>& r, int& cr) {
+  const bool t = less(a, b);
   r = t ? a : b;
   cr = t ? ca : cb;
 }
-AMRFD_HD void maxw(__int128 a, int ca, __int128 b, int cb, __int128& r, int& cr) {
-  const bool t = a < b;
+template <bool RES>
+AMRFD_HD void maxw(const Wide<RES>& a, int ca, const Wide<RES>& b, int cb, Wide<RES>& r, int& cr) {
+  const bool t = less(a, b);
   r = t ? b : a;
   cr = t ? cb : ca;
 }
 
-// The code of a face in exact arithmetic. thr: the acceptance threshold on
-// 30X (30X - 30mp) in squared units; the product of the two exact factors, each rounded to
-// FP64, is compared with it.
-AMRFD_HD int mp5_code_exact(const Limbs<5>& em, const Limbs<5>& e0, const Limbs<5>& e1, const Limbs<5>& ep,
-                            double thr) {
-  const __int128 dm = to_wide(em), d0 = to_wide(e0), d1 = to_wide(e1), dp = to_wide(ep);
-  const __int128 X = 24 * d1 + 11 * d0 - 2 * dm - 3 * dp;
-  __int128 mp = 0;
-  if (d1 != 0 && d0 != 0 && (d1 < 0) == (d0 < 0)) mp = absw(d1) < absw(4 * d0) ? d1 : 4 * d0;
-  const __int128 Z = X - 60 * mp;
-  if (X == 0 || Z == 0 || (X < 0) != (Z < 0)) return 0;
-  if (wide_double(absw(X)) * wide_double(absw(Z)) <= thr) return 0;
-  const __int128 kL = d0 - dm, kC = d1 - d0, kR = dp - d1;
+// The code of a face and 30 times its doubled value y relative to the centre cell, in exact
+// arithmetic. thr: the acceptance threshold on 30X (30X - 30mp) in squared units; the
+// product of the two exact factors, each rounded to FP64, is compared with it.
+template <bool RES>
+AMRFD_HD int mp5_exact(const Wide<RES>& dm, const Wide<RES>& d0, const Wide<RES>& d1, const Wide<RES>& dp, double thr,
+                       const Unit& un, Wide<RES>& y) {
+  const Wide<RES> zero = {0, 0.0};
+  const Wide<RES> X = lin(1, lin(24, d1, 11, d0, un), -1, lin(2, dm, 3, dp, un), un);
+  Wide<RES> mp = zero;
+  const Wide<RES> d04 = lin(4, d0, 0, zero, un);
+  if (sign(d1) == sign(d0)) mp = less(absw(d1), absw(d04)) ? d1 : d04;
+  const Wide<RES> Z = lin(1, X, -60, mp, un);
+  y = X;
+  if (sign(X) * sign(Z) <= 0) return 0;
+  if (in_units(absw(X), un) * in_units(absw(Z), un) <= thr) return 0;
+  const Wide<RES> kL = lin(1, d0, -1, dm, un), kC = lin(1, d1, -1, d0, un), kR = lin(1, dp, -1, d1, un);
   int cp, cm;
-  const __int128 Mp = m4_exact(kC, kR, cp), Mm = m4_exact(kL, kC, cm);
-  const __int128 md = 30 * (d1 - Mp), lc = 30 * d0 + 80 * Mm, d12 = 60 * d1, ul = 240 * d0;
-  __int128 a, b, lo, hi, t1, t2, t3, r;
+  const Wide<RES> Mp = m4_exact(kC, kR, un, cp), Mm = m4_exact(kL, kC, un, cm);
+  const Wide<RES> md = lin(30, d1, -30, Mp, un), lc = lin(30, d0, 80, Mm, un), d12 = lin(60, d1, 0, zero, un),
+                  ul = lin(60, d04, 0, zero, un);
+  Wide<RES> a, b, lo, hi, t1, t2, t3;
   int ca, cb, cl, ch, c1, c2, c3, code;
-  minw(0, 1, d12, 2, a, ca);
+  minw(zero, 1, d12, 2, a, ca);
   minw(a, ca, md, 3, a, ca);
-  minw(0, 1, ul, 4, b, cb);
+  minw(zero, 1, ul, 4, b, cb);
   minw(b, cb, lc, 5, b, cb);
   maxw(a, ca, b, cb, lo, cl);
-  maxw(0, 1, d12, 2, a, ca);
+  maxw(zero, 1, d12, 2, a, ca);
   maxw(a, ca, md, 3, a, ca);
-  maxw(0, 1, ul, 4, b, cb);
+  maxw(zero, 1, ul, 4, b, cb);
   maxw(b, cb, lc, 5, b, cb);
   minw(a, ca, b, cb, hi, ch);
   minw(X, 0, lo, cl, t1, c1);
   maxw(X, 0, lo, cl, t2, c2);
   minw(t2, c2, hi, ch, t3, c3);
-  maxw(t1, c1, t3, c3, r, code);
-  if (r == 0) return 1;  // as the FP32 selection names an exact zero
+  maxw(t1, c1, t3, c3, y, code);
+  if (sign(y) == 0) return 1;  // as the FP32 selection names an exact zero
   if (code == 3) return 3 | (cp << 3);
   if (code == 5) return cm == 0 ? kD0Code : 5 | (cm << 6);
   return code;
@@ -552,70 +668,96 @@ AMRFD_HD int limo3_code_float(float a, float b, float thr) {
   return (n0 ? 0 : (n1 ? 1 : (n2 ? 2 : (n3 ? 3 : 4)))) | (1 << 3);
 }
 
-// The code in exact arithmetic; inside the blend band also the value's difference from y3
-// (times 30, whole units). thr as above.
-AMRFD_HD int limo3_code_exact(const Limbs<5>& ea, const Limbs<5>& eb, double thr, __int128* blend) {
-  const __int128 a = to_wide(ea), b = to_wide(eb);
-  const double fa = wide_double(a), fb = wide_double(b), s2 = fma(fa, fa, fb * fb);
-  *blend = 0;
+// The code and 30 times the value in exact arithmetic; inside the blend band the value's
+// difference from y3 is formed in FP64. thr as above.
+template <bool RES>
+AMRFD_HD int limo3_exact(const Wide<RES>& a, const Wide<RES>& b, double thr, const Unit& un, Wide<RES>& y) {
+  const Wide<RES> zero = {0, 0.0};
+  const double fa = in_units(a, un), fb = in_units(b, un), s2 = fma(fa, fa, fb * fb);
+  const Wide<RES> y3 = lin(10, a, 20, b, un);
+  y = y3;
   if (s2 <= thr * (1.0 - 1e-12)) return 0;
-  const bool neg = b < 0;
-  const __int128 ap = neg ? -a : a, bp = neg ? -b : b, y3 = 10 * ap + 20 * bp;
-  __int128 t;
+  const int sg = sign(b) < 0 ? -1 : 1;
+  const Wide<RES> yp = lin(sg, y3, 0, zero, un);
+  Wide<RES> t;
   int c;
-  minw(60 * ap, 3, y3, 1, t, c);
-  minw(t, c, 48 * bp, 4, t, c);
-  maxw(-15 * ap, 2, t, c, t, c);
-  minw(y3, 1, t, c, t, c);
-  maxw(0, 0, t, c, t, c);
-  if (s2 >= thr * (1.0 + 1e-12)) return c | (1 << 3);
+  minw(lin(60 * sg, a, 0, zero, un), 3, yp, 1, t, c);
+  minw(t, c, lin(48 * sg, b, 0, zero, un), 4, t, c);
+  maxw(lin(-15 * sg, a, 0, zero, un), 2, t, c, t, c);
+  minw(yp, 1, t, c, t, c);
+  maxw(zero, 0, t, c, t, c);
+  if (s2 >= thr * (1.0 + 1e-12)) {
+    y = lin(sg, t, 0, zero, un);
+    return c | (1 << 3);
+  }
   const double z = (s2 / thr - 1.0) * 1e12;
-  const double x = wide_double(t - y3) * (0.5 * (1.0 + z));
+  const double x = in_units(lin(sg, t, -1, y3, un), un) * (0.5 * (1.0 + z));
   const long long xh = (long long)(x * 8.470329472543003e-22);  // 2^-70
   const double xl = x - (double)xh * 1.1805916207174113e+21;
   const long long xm = (long long)(xl * 5.820766091346741e-11);  // 2^-34
-  const __int128 d = ((__int128)xh << 70) + ((__int128)xm << 34) + (long long)(xl - (double)xm * 17179869184.0);
-  *blend = neg ? -d : d;
+  const double xr = xl - (double)xm * 17179869184.0;
+  const Wide<RES> d = {((__int128)xh << 70) + ((__int128)xm << 34) + (long long)xr,
+                       RES ? (xr - (double)(long long)xr) * un.u : 0.0};
+  y = lin(1, y3, 1, d, un);
   return c | ((z < 0.0 ? 2 : 3) << 3);
 }
 
 // ------------------------------------------------------------------- sweeps
-// The scale (lob) for N limbs of nc cells of both lines from j on; false when some cell is
-// not a whole multiple of its unit. FINE looks at the mantissas' trailing zeros, else every
-// mantissa counts as 53 bits. bad: a value of 2^1008 or more. HEAD: bits left free above
-// the largest value.
-template <int N, bool FINE, int HEAD = 0>
-AMRFD_HD bool window_scale(line_t gp, line_t gm, int j, int nc, int& lob, bool& bad) {
-  unsigned mx = 0u, mn = 0xffffffffu;  // mn: one less than the smallest key; zero wraps
+// A cell's exponent word, with FINE raised by its mantissa's trailing zeros (that of a value
+// with the same last bit and a full mantissa); 0 for a zero.
+template <bool FINE>
+AMRFD_HD unsigned cell_key(line_t l, int j, unsigned& a) {
+  int hi;
+  unsigned lo = 0u;
+  if (FINE) cell_words(l, j, hi, lo);
+  else hi = cell_hi(l, j);
+  a = (unsigned)hi & 0x7fffffffu;
+  unsigned k = a;
+  if (FINE && a) {
+    const unsigned m = lo ? lo : ((a & 0xfffffu) | 0x100000u);
+#ifdef __CUDACC__
+    const int z = __ffs((int)m) - 1;
+#else
+    const int z = __builtin_ctz(m);
+#endif
+    k += (unsigned)(z + (lo ? 0 : 32)) << 20;
+  }
+  return k;
+}
+
+// Largest exponent word and smallest key, less one (a zero wraps), of nc cells of both lines
+// from j on.
+struct Span { unsigned mx, mn; };
+template <bool FINE>
+AMRFD_HD Span window_span(line_t gp, line_t gm, int j, int nc) {
+  Span w = {0u, 0xffffffffu};
   for (int q = 0; q < nc; q++) {
 #pragma unroll
     for (int s = 0; s < 2; s++) {
-      int hi;
-      unsigned lo = 0u;
-      if (FINE) cell_words(s ? gm : gp, j + q, hi, lo);
-      else hi = cell_hi(s ? gm : gp, j + q);
-      const unsigned a = (unsigned)hi & 0x7fffffffu;
-      mx = a > mx ? a : mx;
-      unsigned k = a;
-      if (FINE && a) {
-        const unsigned m = lo ? lo : ((a & 0xfffffu) | 0x100000u);
-#ifdef __CUDACC__
-        const int z = __ffs((int)m) - 1;
-#else
-        const int z = __builtin_ctz(m);
-#endif
-        k += (unsigned)(z + (lo ? 0 : 32)) << 20;
-      }
-      mn = k - 1u < mn ? k - 1u : mn;
+      unsigned a;
+      const unsigned k = cell_key<FINE>(s ? gm : gp, j + q, a);
+      w.mx = a > w.mx ? a : w.mx;
+      w.mn = k - 1u < w.mn ? k - 1u : w.mn;
     }
   }
-  int top = (int)(mx >> 20);
-  bad = top > kExpMax;
-  top = bad ? kExpMax : top;
+  return w;
+}
+// The scale (lob) for N limbs; false when some cell is not a whole multiple of its unit or is
+// 2^1008 or more. bad: a value that is not finite. HEAD: bits left free above the largest.
+template <int N, int HEAD = 0>
+AMRFD_HD bool span_scale(const Span& w, int& lob, bool& bad) {
+  int top = (int)(w.mx >> 20);
+  bad = top == 2047;
+  top = bad ? 2046 : top;
   constexpr int span = room(N) - HEAD;
   lob = (top - span < kExpUnit ? kExpUnit : top - span) << 20;
-  const unsigned low = mn == 0xffffffffu ? mn : (mn + 1u) >> 20;
-  return low >= (unsigned)(lob >> 20) && !bad;
+  const unsigned low = w.mn == 0xffffffffu ? w.mn : (w.mn + 1u) >> 20;
+  return low >= (unsigned)(lob >> 20) && top <= kExpMax;
+}
+// Both. FINE looks at the mantissas' trailing zeros, else every mantissa counts as 53 bits.
+template <int N, bool FINE, int HEAD = 0>
+AMRFD_HD bool window_scale(line_t gp, line_t gm, int j, int nc, int& lob, bool& bad) {
+  return span_scale<N, HEAD>(window_span<FINE>(gp, gm, j, nc), lob, bad);
 }
 
 // The thresholds of the FP32 decisions in squared floats' units: MP5's acceptance threshold
@@ -673,78 +815,147 @@ AMRFD_HD void add_carried(Limbs<N>& F, const long long* s) {
   F.v[N - 1] += (int)(s[N - 1] + carry);
 }
 
+// A face's code from its differences in FP32, -1 when that cannot tell: numbers with
+// remainders are costly to compare (28x78x45 MHD step: 733 us without, 663 with), whole ones
+// cheaper exactly.
+template <bool LIMO, bool RES>
+AMRFD_HD int float_code(const Wide<RES>* D, float thr_lo, const Unit& un) {
+  bool small = false;
+  float f[4];
+#pragma unroll
+  for (int q = 0; q < (LIMO ? 2 : 4); q++) f[q] = wide_float(D[q], un, small);
+  if (small) return -1;
+  if constexpr (LIMO) return limo3_code_float(f[0], f[1], thr_lo);
+  const int c = mp5_code_float(f[0], f[1], f[2], f[3], thr_lo);
+  return c < 0 ? mp5_code_bounded(f[0], f[1], f[2], f[3], thr_lo) : c;
+}
+
 // One cell by itself, its comparisons exact: the cells a sweep could not finish (a
-// comparison FP32 could not settle, a part over more than 110 bits, a value of 2^1008 or
-// more). i: the cell; its window starts at extended cell i + C0.
-template <bool LIMO, bool REC>
-AMRFD_HD void exact_cell(line_t gp, line_t gm, int i, double limo_thr, double* out, bool write, unsigned short* tp,
-                         unsigned short* tm, int f0, int fend, int fmod) {
+// comparison FP32 could not settle, a window over more than 110 bits, values of 2^1008 or
+// more). i: the cell; its window starts at extended cell i + C0. RES: some value is no whole
+// number of units.
+template <bool LIMO, bool REC, bool RES>
+AMRFD_HD double exact_value(line_t gp, line_t gm, int i, double limo_thr, int lob, unsigned short* tp,
+                            unsigned short* tm, int f0, int fend, int fmod) {
   constexpr int NC = LIMO ? 4 : 6;
   constexpr int C0 = LIMO ? 1 : 0;
   constexpr int ND = LIMO ? 2 : 4;
-  int lob;
-  bool bad;
-  window_scale<5, true>(gp, gm, i + C0, NC + 1, lob, bad);
+  const Unit un = unit_of(lob);
   const int qe = (lob >> 20) - 1075;
+  const double thr = (LIMO ? limo_thr : 1.44e-6) * pow2d(-qe) * pow2d(-qe);
   const float thr_lo = float_threshold<LIMO, 5>(lob, limo_thr);
-  Limbs<5> Fp;
+  // 60 (Fsum_{k-1} - Fsum_k) as 30 times the doubled values and 60 times the differences of the
+  // two faces' centre cells
+  Wide<RES> F = {0, 0.0};
 #pragma unroll 1
   for (int face = 0; face < 2; face++) {
     const int c0 = i + C0 + face;  // first cell of the face's window
-    Limbs<5> F = {{0, 0, 0, 0, 0}};
     int code[2];
 #pragma unroll 1
     for (int s = 0; s < 2; s++) {
-      // the stencil from the left (G+) or from the right (G-), as cells and differences
-      Limbs<5> D[ND], last;
+      // the stencil from the left (G+) or from the right (G-), as differences
+      Wide<RES> D[ND], last;
 #pragma unroll
       for (int q = 0; q <= ND; q++) {
-        int hi;
-        unsigned lo;
-        cell_words(s ? gm : gp, s ? c0 + NC - 1 - q : c0 + q, hi, lo);
-        const Limbs<5> u = limbs_wide(hi, lo, lob);
-        const int w = LIMO ? (q == 0 ? -10 : (q == 1 ? 50 : 20))
-                           : (q == 0 ? 2 : (q == 1 ? -13 : (q == 2 ? 47 : (q == 3 ? 27 : -3))));
-#pragma unroll
-        for (int l = 0; l < 5; l++) {
-          F.v[l] += w * u.v[l];
-          if (q) D[q - 1].v[l] = u.v[l] - last.v[l];
-        }
+        const Wide<RES> u = wide_cell<RES>(s ? gm : gp, s ? c0 + NC - 1 - q : c0 + q, lob, un);
+        if (q) D[q - 1] = lin(1, u, -1, last, un);
         last = u;
       }
-      if constexpr (LIMO) {
-        __int128 blend = 0;
-        code[s] = limo3_code_float(to_float(D[0]), to_float(D[1]), thr_lo);
-        if (code[s] < 0) code[s] = limo3_code_exact(D[0], D[1], limo_thr * pow2d(-qe) * pow2d(-qe), &blend);
+      Wide<RES> y;
+      code[s] = RES ? float_code<LIMO>(D, thr_lo, un) : -1;
+      if (code[s] >= 0) {
+        y = {0, 0.0};
+        int e[5], sum = 0;
+        limited_coefs<LIMO>(code[s], e);
 #pragma unroll
-        for (int l = 0; l < 5; l++) F.v[l] += l < 4 ? (int)(blend >> (22 * l)) & kLimbMask : (int)(blend >> 88);
+        for (int q = 0; q < ND; q++) {  // the cells' coefficients add up to zero
+          sum += e[q];
+          y = lin(1, y, (LIMO ? (q == 0 ? 10 : 20) : (q == 0 ? -2 : (q == 1 ? 11 : (q == 2 ? 24 : -3)))) - sum, D[q], un);
+        }
+      } else if constexpr (LIMO) {
+        code[s] = limo3_exact(D[0], D[1], thr, un, y);
       } else {
-        const float dm = to_float(D[0]), d0 = to_float(D[1]), d1 = to_float(D[2]), dp = to_float(D[3]);
-        code[s] = mp5_code_float(dm, d0, d1, dp, thr_lo);
-        if (code[s] < 0) code[s] = mp5_code_bounded(dm, d0, d1, dp, thr_lo);
-        if (code[s] < 0) code[s] = mp5_code_exact(D[0], D[1], D[2], D[3], 1.44e-6 * pow2d(-2 * qe));
+        code[s] = mp5_exact(D[0], D[1], D[2], D[3], thr, un, y);
       }
-      int e[5];
-      limited_coefs<LIMO>(code[s], e);
-      long long a[5] = {0, 0, 0, 0, 0};
-#pragma unroll
-      for (int q = 0; q <= ND; q++) {
-        int hi;
-        unsigned lo;
-        cell_words(s ? gm : gp, s ? c0 + NC - 1 - q : c0 + q, hi, lo);
-        const Limbs<5> u = limbs_wide(hi, lo, lob);
-#pragma unroll
-        for (int l = 0; l < 5; l++) a[l] += (long long)e[q] * u.v[l];
-      }
-      add_carried(F, a);
+      F = lin(1, F, face ? -1 : 1, y, un);
+      if (face) F = lin(1, F, s ? 60 : -60, D[LIMO ? s : 1 + s], un);
     }
     record<REC>(tp, tm, f0 + i + face, fend, fmod, code[0], code[1]);
-    if (face && write) {
-      const double r = to_double(Fp, F, lob);
-      *out = bad ? from_words(0x7ff80000, 0u) : r;
-    }
-    Fp = F;
   }
+  return nearest(F, un, lob);
+}
+
+// A cell both of whose faces are surely unlimited: a fixed filter of its cells, their largest
+// value (with a weight of at least 2) at 110 bits. What rounds, below 2^-110 of that, is far
+// below the rounding of any sum the large values are in. The tails ahead of a front, which
+// fall off by binades per cell down to underflow, go this way.
+template <bool LIMO>
+AMRFD_HD double linear_value(line_t gp, line_t gm, int j, int top) {
+  constexpr int NC = LIMO ? 4 : 6;
+  const int lob = (top - room(5) < kExpUnit ? kExpUnit : top - room(5)) << 20;
+  const Unit un = unit_of(lob);
+  Wide<true> F = {0, 0.0};
+#pragma unroll
+  for (int q = 0; q < NC; q++) {
+    const int w = LIMO ? (q == 0 ? -10 : (q == 1 ? 60 : (q == 2 ? -30 : -20)))
+                       : (q == 0 ? 2 : (q == 1 ? -15 : (q == 2 ? 60 : (q == 3 ? -20 : (q == 4 ? -30 : 3)))));
+    const Wide<true> a = wide_cell<true>(gp, j + q, lob, un), b = wide_cell<true>(gm, j + NC - q, lob, un);
+    F.h += (a.h - b.h) * w;
+    if (lob == kExpUnit << 20) F.r = fma((double)w, a.r - b.r, F.r);  // no large value
+  }
+  return nearest(lin(1, F, 0, F, un), un, lob);
+}
+
+// Out of line: its registers stay out of the sweeps'.
+template <bool LIMO, bool REC>
+AMRFD_HD_CALL void exact_cell(line_t gp, line_t gm, int i, double limo_thr, double* out, bool write, unsigned short* tp,
+                              unsigned short* tm, int f0, int fend, int fmod) {
+  constexpr int NC = LIMO ? 4 : 6;
+  const int j = i + (LIMO ? 1 : 0);
+  // largest exponents of the window and of the cells in it that the faces' stencils hold
+  int most = 0, top = 0;
+#pragma unroll
+  for (int q = 0; q <= NC; q++) {
+    const int a = (cell_hi(gp, j + q) >> 20) & 0x7ff, b = (cell_hi(gm, j + NC - q) >> 20) & 0x7ff, m = a > b ? a : b;
+    most = m > most ? m : most;
+    if (q < NC) top = m > top ? m : top;
+  }
+  const double x = pow2d(most - 1022);
+  double r;
+  // differences below 2 x: 30X (30X - 30mp) below 16000 x^2, LIMO3's a^2 + b^2 below 8 x^2
+  if (LIMO ? 8.01 * x * x < limo_thr : x < 0x1p-17) {
+    r = linear_value<LIMO>(gp, gm, j, top);
+    record<REC>(tp, tm, f0 + i, fend, fmod, 0, 0);
+    record<REC>(tp, tm, f0 + i + 1, fend, fmod, 0, 0);
+  } else {
+    int lob;
+    bool bad;
+    const bool whole = window_scale<5, true>(gp, gm, j, NC + 1, lob, bad);
+    r = whole ? exact_value<LIMO, REC, false>(gp, gm, i, limo_thr, lob, tp, tm, f0, fend, fmod)
+              : exact_value<LIMO, REC, true>(gp, gm, i, limo_thr, lob, tp, tm, f0, fend, fmod);
+    if (bad) r = from_words(0x7ff80000, 0u);
+  }
+  if (write) *out = r;
+}
+
+// The cells of a part whose window holds a value that is no whole number of units at the
+// scale lob, or is beyond a sweep's range.
+template <bool LIMO>
+AMRFD_HD unsigned long long partial_cells(line_t gp, line_t gm, int nc, int lob) {
+  constexpr int NC = LIMO ? 4 : 6;
+  constexpr unsigned long long hit = (2ull << NC) - 1ull;  // the cells i with q in [i, i + NC]
+  unsigned long long m = 0ull;
+  for (int q = 0; q < nc; q++) {
+    bool part = false;
+#pragma unroll
+    for (int s = 0; s < 2; s++) {
+      unsigned a;
+      const unsigned k = cell_key<true>(s ? gm : gp, q + (LIMO ? 1 : 0), a);
+      part |= (k && k < (unsigned)lob) || (int)(a >> 20) > kExpMax;
+    }
+    if (part) m |= q < NC ? hit >> (NC - q) : hit << (q - NC);
+  }
+  return m;
 }
 
 // The faces k = 3..plen+3 of one (line, variable) at the scale lob of N limbs, and the
@@ -884,16 +1095,18 @@ AMRFD_HD int fixed_sweep(line_t gp, line_t gm, int plen, double limo_thr, double
   const int nc = plen + 6 - 2 * C0;
   int lob, limited = 0;
   bool bad;
-  const bool narrow = window_scale<3, false>(gp, gm, C0, nc, lob, bad);
+  const Span span = window_span<false>(gp, gm, C0, nc);
+  const unsigned long long all = plen < 64 ? (1ull << plen) - 1ull : ~0ull;
   unsigned long long todo;
-  if (!AMRFD_ANY(lanes, !narrow)) {
+  if (!AMRFD_ANY(lanes, !span_scale<3>(span, lob, bad))) {
     todo = sweep_part<LIMO, REC, 3>(gp, gm, plen, limo_thr, out, ostr, wmask, tp, tm, f0, fend, fmod, lob, limited);
   } else {
     const bool whole = window_scale<5, true>(gp, gm, C0, nc, lob, bad);
-    todo = sweep_part<LIMO, REC, 5>(gp, gm, plen, limo_thr, out, ostr, wmask, tp, tm, f0, fend, fmod, lob, limited);
-    if (!whole) todo = ~0ull;
+    todo = whole ? 0ull : partial_cells<LIMO>(gp, gm, nc, lob);
+    if (AMRFD_ANY(lanes, (~todo & all) != 0ull))
+      todo |= sweep_part<LIMO, REC, 5>(gp, gm, plen, limo_thr, out, ostr, wmask, tp, tm, f0, fend, fmod, lob, limited);
   }
-  if (plen < 64) todo &= (1ull << plen) - 1ull;
+  todo &= all;
   while (todo) {
 #ifdef __CUDACC__
     const int i = __ffsll((long long)todo) - 1;

@@ -9,6 +9,8 @@ from fractions import Fraction
 import numpy as np
 import pytest
 
+from test_sweep_host import _reference
+
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1407_2052_gb300", "csrc")
 
 HARNESS = """
@@ -16,6 +18,11 @@ HARNESS = """
 using namespace amrfd;
 extern "C" double wide(long long hi, unsigned long long lo) {
   return wide_double((__int128)(((unsigned __int128)(unsigned long long)hi << 64) | lo));
+}
+extern "C" void sweep(int limo, const double* gp, const double* gm, int plen, double thr, double* out,
+                      unsigned short* tp, unsigned short* tm) {
+  if (limo) fixed_sweep<true, true>(gp, gm, plen, thr, out, 1, ~0ull, tp, tm, 0, plen + 1, 1 << 30, 1);
+  else fixed_sweep<false, true>(gp, gm, plen, 0.0, out, 1, ~0ull, tp, tm, 0, plen + 1, 1 << 30, 1);
 }
 """
 
@@ -32,7 +39,15 @@ def lib(tmp_path_factory):
                     "-o", str(so)], check=True)
     L = ctypes.CDLL(str(so))
     L.wide.restype, L.wide.argtypes = ctypes.c_double, [ctypes.c_longlong, ctypes.c_ulonglong]
+    L.sweep.argtypes = [ctypes.c_int] + [ctypes.c_void_p] * 2 + [ctypes.c_int, ctypes.c_double] + [ctypes.c_void_p] * 3
     return L
+
+
+def _sweep(lib, limo, g, h, thr=0.0):
+    n = len(g) - 6
+    out, tp, tm = np.full(n, np.nan), np.zeros(n + 1, np.uint16), np.zeros(n + 1, np.uint16)
+    lib.sweep(limo, g.ctypes.data, h.ctypes.data, n, thr, out.ctypes.data, tp.ctypes.data, tm.ctypes.data)
+    return out, tp, tm
 
 
 @pytest.mark.parametrize("bits", [53, 54, 95, 96, 97, 120, 121, 122, 123, 124, 125])
@@ -44,3 +59,39 @@ def test_wide_sums_round_once(lib, bits):
         a += (1 << max(0, bits - 54)) + int(rng.integers(-2, 3))  # half a unit in the last place, about
         a = min(a, (1 << bits) - 1) * int(rng.choice((-1, 1)))
         assert lib.wide(a >> 64, a & (2 ** 64 - 1)) == float(Fraction(a)), a
+
+
+@pytest.mark.parametrize("limo", [0, 1], ids=["mp5", "limo3"])
+@pytest.mark.parametrize("weak", [1e-20, 1e-34, 1e-60, 1e-200, 1e-300])
+def test_weak_cells_beside_strong_ones_keep_their_precision(lib, weak, limo):
+    """Where the limiter drops the strong cells of a window, the difference is one of the weak
+    cells alone, and off by no more than FP64 sums of them are: fewer than 40 roundings of
+    terms below 2000 weak cells."""
+    rng, dropped = np.random.default_rng(7), 0
+    for _ in range(60):
+        n = 24
+        s = rng.integers(3, 12)
+        g = np.where(np.arange(n) < s, 1 + 0.1 * rng.random(n), weak * rng.uniform(0.5, 2.0, n))
+        h = np.where(np.arange(n) >= n - s, 1 + 0.1 * rng.random(n), weak * rng.uniform(-1, 1, n))
+        out, _, _ = _sweep(lib, limo, g, h, 1e-30)
+        for i, want in enumerate(_reference(limo, g, h, 1e-30)):
+            strong = any(abs(x) > 0.5 for x in (*g[i:i + 7], *h[i:i + 7]))
+            if abs(want) < 2000 * 2 * weak:
+                dropped += strong
+                err = abs(Fraction(float(out[i])) - want)
+                assert err <= Fraction(40 * 2000 * 2 * weak) * Fraction(2) ** -53 + Fraction(2) ** -1060, i
+    assert dropped > 50
+
+
+@pytest.mark.parametrize("limo", [0, 1], ids=["mp5", "limo3"])
+def test_finite_values_of_any_size_give_the_rounded_difference(lib, limo):
+    rng = np.random.default_rng(8)
+    for top in (1005, 1012, 1018, 1023):
+        g, h = (np.ldexp(rng.uniform(-1, 1, 30), top) for _ in range(2))
+        out, _, _ = _sweep(lib, limo, g, h, 1e-30)
+        for i, want in enumerate(_reference(limo, g, h, 1e-30)):
+            try:
+                w = float(want)
+            except OverflowError:
+                w = np.inf if want > 0 else -np.inf
+            assert out[i] == w, (top, i)
