@@ -95,3 +95,16 @@ def test_finite_values_of_any_size_give_the_rounded_difference(lib, limo):
             except OverflowError:
                 w = np.inf if want > 0 else -np.inf
             assert out[i] == w, (top, i)
+
+
+@pytest.mark.parametrize("limo", [0, 1], ids=["mp5", "limo3"])
+@pytest.mark.parametrize("binades", [12, 13, 14, 34, 35, 36, 56, 57])
+def test_every_width_of_the_sums_rounds_correctly(lib, binades, limo):
+    """One limb more or less: the cells' exponents span exactly `binades`, full mantissas."""
+    rng = np.random.default_rng(binades)
+    for _ in range(20):
+        e = rng.integers(-binades, 1, (2, 38))
+        e[0, 5], e[1, 6] = 0, -binades
+        g, h = (np.ldexp(rng.uniform(1, 2, 38) * rng.choice((-1, 1), 38), x) for x in e)
+        out, _, _ = _sweep(lib, limo, g, h, 0.1)
+        assert out.tolist() == [float(x) for x in _reference(limo, g, h, 0.1)]
