@@ -492,11 +492,11 @@ struct Unit {  // of a scale lob: the unit as a double, its reciprocal
 };
 AMRFD_HD Unit unit_of(int lob) { return {pow2d((lob >> 20) - 1075), pow2d(1075 - (lob >> 20))}; }
 
-AMRFD_HD bool any_bits(double x) {  // no FP64 comparison
+AMRFD_HD bool any_bits(double x) {  // not +-0, without an FP64 comparison
   int hi;
   unsigned lo;
   words(x, hi, lo);
-  return (hi | (int)lo) != 0;
+  return ((hi << 1) | (int)lo) != 0;
 }
 // |r| <= unit/2 (or a little more) again, so that h and then r order the numbers.
 template <bool RES>
@@ -580,7 +580,7 @@ AMRFD_HD Wide<RES> wide_cell(line_t l, int j, int lob, const Unit& un) {
   if (L >= 0) a.h = (__int128)m << L;
   else if (L >= -54) a.h = (__int128)((m + (1ull << (-L - 1))) >> -L);
   if (hi < 0) a.h = -a.h;
-  if (RES && L < 0) a.r = fma(-(double)(long long)a.h, un.u, from_words(hi, lo));
+  if (RES && L < 0) a.r = a.h == 0 ? from_words(hi, lo) : fma(-(double)(long long)a.h, un.u, from_words(hi, lo));
   return a;
 }
 
@@ -1158,46 +1158,56 @@ AMRFD_HD int tape_index(const TapeLine& t, int k) {
   return t.wrap ? (f < 0 ? f + t.n : (f >= t.n ? f - t.n : f)) : f;
 }
 
-// One cell by itself (relative to s0), at the scale of the seven values that reach it.
-template <bool LIMO>
-AMRFD_HD void adjoint_cell(line_t g, const TapeLine& t, int kb, int ke, int cell, double* gp, double* gm) {
+// One cell by itself (relative to s0), at the scale of the seven values that reach it; what
+// its units leave over (RES) is carried as in exact_value.
+template <bool LIMO, bool RES>
+AMRFD_HD void adjoint_values(line_t g, const TapeLine& t, int kb, int ke, int cell, int lob, double v[2]) {
   constexpr int NS = LIMO ? 3 : 5;         // cells of a stencil
   constexpr int off = LIMO ? 2 : 3;        // G+ stencil of face k: cells k - off ..
-  int lob;
-  bool bad;
-  const int r0 = cell < 0 ? 0 : cell, r1 = cell + 6;  // g[r] of cells cell-3 .. cell+3, those there are
-  const int last = ke + 3;
-  window_scale<5, true, kAdjHead>(g, g, r0, (r1 < last ? r1 : last) - r0 + 1, lob, bad);
-  Limbs<5> F[2] = {{{0, 0, 0, 0, 0}}, {{0, 0, 0, 0, 0}}};
+  const Unit un = unit_of(lob);
+  const int k0 = cell - off + 1 > kb ? cell - off + 1 : kb, k1 = cell + off < ke ? cell + off : ke;
+  Wide<RES> F[2] = {{0, 0.0}, {0, 0.0}}, b = wide_cell<RES>(g, k0 + 2, lob, un);
 #pragma unroll 1
-  for (int s = 0; s < 2; s++) {
-#pragma unroll 1
-    for (int q = 0; q < NS; q++) {
-      // G+: face whose stencil cell q is this one; G-: counted from the right, cell k + off - 1 - q
-      const int k = s ? cell + q - (off - 1) : cell + off - q;
-      if (k < kb || k > ke) continue;
-      int ah, bh;
-      unsigned al, bl;
-      cell_words(g, k + 3, ah, al);
-      cell_words(g, k + 2, bh, bl);
-      if (((ah ^ bh) | (int)(al ^ bl)) == 0) continue;  // no code where the gradient does not reach
-      const Limbs<5> a = limbs_wide(ah, al, lob), b = limbs_wide(bh, bl, lob);
-      const int f = tape_index(t, k);
+  for (int k = k0; k <= k1; k++) {
+    const Wide<RES> a = wide_cell<RES>(g, k + 3, lob, un);
+    const __int128 h = a.h - b.h;
+    const double r = RES && (any_bits(a.r) || any_bits(b.r)) ? a.r - b.r : 0.0;
+    b = a;
+    if (h == 0 && !any_bits(r)) continue;  // no code where the gradient does not reach
+    const int f = tape_index(t, k);
+#pragma unroll
+    for (int s = 0; s < 2; s++) {
+      // the face's stencil cell this one is: G+ cells k - off .., G- counted from the right
+      const int q = s ? k + off - 1 - cell : cell + off - k;
+      if (q < 0 || q >= NS) continue;
       int e[5];
       limited_coefs<LIMO>(adjoint_code<LIMO>(s ? t.tm[f] : t.tp[f]), e);
       const int w = LIMO ? (q == 0 ? -10 : (q == 1 ? 50 : 20))
                          : (q == 0 ? 2 : (q == 1 ? -13 : (q == 2 ? 47 : (q == 3 ? 27 : -3))));
       const int c = w + (q == 0 ? e[0] : (q == 1 ? e[1] : (q == 2 ? e[2] : (q == 3 ? e[3] : e[4]))));
-      long long x[5];
-#pragma unroll
-      for (int l = 0; l < 5; l++) x[l] = (long long)c * (a.v[l] - b.v[l]);
-      add_carried(F[s], x);
+      F[s].h += h * c;
+      if (RES && any_bits(r)) F[s].r = fma((double)c, r, F[s].r);
     }
   }
-  const Limbs<5> zero = {{0, 0, 0, 0, 0}};
+#pragma unroll
+  for (int s = 0; s < 2; s++) {
+    if (RES) carry_units(F[s], un);
+    v[s] = nearest(F[s], un, lob);
+  }
+}
+template <bool LIMO>
+AMRFD_HD_CALL void adjoint_cell(line_t g, TapeLine t, int kb, int ke, int cell, double* gp, double* gm) {
+  int lob;
+  bool bad;
+  const int r0 = cell < 0 ? 0 : cell, r1 = cell + 6;  // g[r] of cells cell-3 .. cell+3, those there are
+  const int last = ke + 3;
+  double v[2];
+  if (window_scale<5, true, kAdjHead>(g, g, r0, (r1 < last ? r1 : last) - r0 + 1, lob, bad))
+    adjoint_values<LIMO, false>(g, t, kb, ke, cell, lob, v);
+  else adjoint_values<LIMO, true>(g, t, kb, ke, cell, lob, v);
   const double nan = from_words(0x7ff80000, 0u);
-  gp[cell + 5] = bad ? nan : to_double(F[0], zero, lob);
-  gm[cell + 5] = bad ? nan : to_double(F[1], zero, lob);
+  gp[cell + 5] = bad ? nan : v[0];
+  gm[cell + 5] = bad ? nan : v[1];
 }
 
 template <int N>

@@ -24,6 +24,11 @@ extern "C" void sweep(int limo, const double* gp, const double* gm, int plen, do
   if (limo) fixed_sweep<true, true>(gp, gm, plen, thr, out, 1, ~0ull, tp, tm, 0, plen + 1, 1 << 30, 1);
   else fixed_sweep<false, true>(gp, gm, plen, 0.0, out, 1, ~0ull, tp, tm, 0, plen + 1, 1 << 30, 1);
 }
+extern "C" void adjoint(int limo, const double* g, int slen, const unsigned short* codes, double* gp, double* gm) {
+  const TapeLine t = {codes, codes, 1, slen + 20, true};
+  if (limo) adjoint_sweep<true>(g, slen, t, -2, slen + 2, 0, slen - 1, gp, gm, 1);
+  else adjoint_sweep<false>(g, slen, t, -2, slen + 2, 0, slen - 1, gp, gm, 1);
+}
 """
 
 
@@ -40,6 +45,7 @@ def lib(tmp_path_factory):
     L = ctypes.CDLL(str(so))
     L.wide.restype, L.wide.argtypes = ctypes.c_double, [ctypes.c_longlong, ctypes.c_ulonglong]
     L.sweep.argtypes = [ctypes.c_int] + [ctypes.c_void_p] * 2 + [ctypes.c_int, ctypes.c_double] + [ctypes.c_void_p] * 3
+    L.adjoint.argtypes = [ctypes.c_int, ctypes.c_void_p, ctypes.c_int] + [ctypes.c_void_p] * 3
     return L
 
 
@@ -108,3 +114,20 @@ def test_every_width_of_the_sums_rounds_correctly(lib, binades, limo):
         g, h = (np.ldexp(rng.uniform(1, 2, 38) * rng.choice((-1, 1), 38), x) for x in e)
         out, _, _ = _sweep(lib, limo, g, h, 0.1)
         assert out.tolist() == [float(x) for x in _reference(limo, g, h, 0.1)]
+
+
+@pytest.mark.parametrize("limo", [0, 1], ids=["mp5", "limo3"])
+@pytest.mark.parametrize("weak", [1e-20, 1e-40, 1e-290])
+def test_weak_gradients_beside_strong_ones_keep_their_precision(lib, weak, limo):
+    """With every face on the piece "zero" a cell's gradient is 60 times one difference of the
+    upstream gradient: of two weak ones wherever it is, whatever else lies within reach."""
+    rng, n = np.random.default_rng(11), 16
+    codes = np.full(n + 21, 8 if limo else 1, np.uint16)
+    for _ in range(20):
+        g = np.where(rng.random(n + 6) < 0.3, 1.0, weak) * rng.uniform(0.5, 2.0, n + 6)
+        gp, gm = np.zeros(n + 10), np.zeros(n + 10)
+        lib.adjoint(limo, g.ctypes.data, n, codes.ctypes.data, gp.ctypes.data, gm.ctypes.data)
+        G = [Fraction(float(x)) for x in g]
+        for c in range(n):  # G+ of cell c is the centre of face c + 1, G- of face c
+            for got, want in ((gp[c + 5], 60 * (G[c + 4] - G[c + 3])), (gm[c + 5], 60 * (G[c + 3] - G[c + 2]))):
+                assert abs(Fraction(float(got)) - want) <= abs(want) * Fraction(2) ** -51, c
