@@ -627,9 +627,9 @@ __global__ void __launch_bounds__(256) combine_kernel(CombParams p) {
     const double dtb = dt * p.co.b;
     // L = sum_d (Fsum_{i-1/2} - Fsum_{i+1/2}) / (2 dx_d), Fsum in units of 2 F^; the flux pass
     // stores 60 times the differences
-    const double w0 = dtb * (1.0 / (120.0 * dm.dx[0]));
-    const double w1 = p.ndim > 1 ? dtb * (1.0 / (120.0 * dm.dx[1])) : 0.0;
-    const double w2 = p.ndim > 2 ? dtb * (1.0 / (120.0 * dm.dx[2])) : 0.0;
+    const double w0 = stage_weight(dtb, dm.dx[0]);
+    const double w1 = p.ndim > 1 ? stage_weight(dtb, dm.dx[1]) : 0.0;
+    const double w2 = p.ndim > 2 ? stage_weight(dtb, dm.dx[2]) : 0.0;
     const bool damp = PHYS == PH_MHD && p.final_stage && p.glm_cr > 0.0;
     if (damp) {
       if (threadIdx.x == 0) {

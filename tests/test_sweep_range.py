@@ -29,6 +29,7 @@ extern "C" void adjoint(int limo, const double* g, int slen, const unsigned shor
   if (limo) adjoint_sweep<true>(g, slen, t, -2, slen + 2, 0, slen - 1, gp, gm, 1);
   else adjoint_sweep<false>(g, slen, t, -2, slen + 2, 0, slen - 1, gp, gm, 1);
 }
+extern "C" double weight(double dtb, double dx) { return stage_weight(dtb, dx); }
 """
 
 
@@ -44,6 +45,7 @@ def lib(tmp_path_factory):
                     "-o", str(so)], check=True)
     L = ctypes.CDLL(str(so))
     L.wide.restype, L.wide.argtypes = ctypes.c_double, [ctypes.c_longlong, ctypes.c_ulonglong]
+    L.weight.restype, L.weight.argtypes = ctypes.c_double, [ctypes.c_double] * 2
     L.sweep.argtypes = [ctypes.c_int] + [ctypes.c_void_p] * 2 + [ctypes.c_int, ctypes.c_double] + [ctypes.c_void_p] * 3
     L.adjoint.argtypes = [ctypes.c_int, ctypes.c_void_p, ctypes.c_int] + [ctypes.c_void_p] * 3
     return L
@@ -131,3 +133,10 @@ def test_weak_gradients_beside_strong_ones_keep_their_precision(lib, weak, limo)
         for c in range(n):  # G+ of cell c is the centre of face c + 1, G- of face c
             for got, want in ((gp[c + 5], 60 * (G[c + 4] - G[c + 3])), (gm[c + 5], 60 * (G[c + 3] - G[c + 2]))):
                 assert abs(Fraction(float(got)) - want) <= abs(want) * Fraction(2) ** -51, c
+
+
+def test_stage_weight_rounds_once_on_power_of_two_grids(lib):
+    rng = np.random.default_rng(5)
+    for _ in range(3000):
+        dtb, k = float(rng.uniform(1e-6, 1.0)), int(rng.integers(0, 14))
+        assert lib.weight(dtb, 2.0 ** -k) == float(Fraction(dtb) * 2 ** k / 120)
