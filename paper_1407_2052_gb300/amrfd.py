@@ -146,7 +146,7 @@ def _ints(v):
 def _spacings(values):
     try:
         a = np.array(values, dtype=np.float64)  # mostly distinct: converted at once
-        if a.ndim == 2 and a.shape[1] == 3:
+        if a.ndim == 2 and a.shape[1] == 3 and not np.isnan(a).any():  # numpy reads None as NaN
             return a
     except (TypeError, ValueError):
         pass
@@ -159,22 +159,26 @@ def _faces(v):
 
 def _domain_table(domains):
     """The domains as an array of _DOMAIN records, filled field by field (900 blocks: four
-    times faster than one assignment per number)."""
+    times faster than one assignment per number), and their numbers of cells and blocks and
+    their offsets before they narrow to the records' types, in FP64 (no overflow)."""
     t = np.zeros(len(domains), _DOMAIN)
+    cells = blocks = offsets = np.zeros(0)
     if len(domains):
         none = ((0, 0),) * 3
         asym = [getattr(d, "asym", None) for d in domains]
-        t["n"] = _column([d.n for d in domains], _ints)
-        t["nb"] = _column([d.nb for d in domains], _ints)
+        n, nb = _column([d.n for d in domains], _ints), _column([d.nb for d in domains], _ints)
+        cells, blocks = (a.astype(np.float64).prod(axis=1) for a in (n, nb))
+        t["n"], t["nb"] = n, nb
         t["dx"] = _spacings([d.dx for d in domains])
         t["bc"] = _column([d.bc for d in domains], _faces)
         t["asym"] = _column([none if a is None else a for a in asym], _faces)
         t["offset"] = [int(d.offset) for d in domains]
-    return t
+        offsets = t["offset"].astype(np.float64)
+    return t, cells, blocks, offsets
 
 
 def domains_c(domains):
-    return (DomainC * len(domains)).from_buffer_copy(_domain_table(domains))
+    return (DomainC * len(domains)).from_buffer_copy(_domain_table(domains)[0])
 
 
 def dt_noalloc(physics, ndim, gamma, cfl, domains, U, out, active=None, t=0.0, t_end=float("inf"),
@@ -186,9 +190,9 @@ def dt_noalloc(physics, ndim, gamma, cfl, domains, U, out, active=None, t=0.0, t
     tensor of at least len(domains) values, `U` large enough for every domain."""
     import torch
     nv = 2 + ndim if physics == EULER else 9
-    table = _domain_table(domains)
-    nblocks = table["nb"].prod(axis=1, dtype=np.float64).sum()  # whole numbers; no overflow
-    need = (table["offset"] + nv * table["n"].prod(axis=1, dtype=np.float64)).max(initial=0.0)
+    table, cells, blocks, offsets = _domain_table(domains)
+    nblocks = blocks.sum()
+    need = (offsets + nv * cells).max(initial=0.0)
     if active is not None:
         if not isinstance(active, torch.Tensor) or active.dtype != torch.uint8 or not active.is_contiguous():
             raise TypeError("active: expected a contiguous uint8 tensor")

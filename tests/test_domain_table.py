@@ -48,3 +48,24 @@ def test_short_fields_stay_refused(field):
     d[field] = d[field][:1]
     with pytest.raises(IndexError):
         A.domains_c([D(**d), D(**d)])
+
+
+@pytest.mark.parametrize("field,value", [("n", (2 ** 32 + 16, 16, 1)), ("nb", (2 ** 32 + 1, 1, 1)),
+                                         ("n", (2 ** 31 + 8, 2 ** 31, 2 ** 31))])
+def test_sizes_beyond_the_records_types_are_not_taken_for_small_ones(field, value):
+    """The time step of many blocks sizes its tensors from the numbers given, not from what a
+    record of 32-bit sizes holds of them."""
+    torch = pytest.importorskip("torch")
+    d = dict(n=(16, 16, 1), nb=(1, 1, 1), dx=(1.0, 1.0, 1.0), bc=((0, 0),) * 3, offset=0)
+    d[field] = value
+    U, out, act = torch.zeros(9 * 256, dtype=torch.float64), torch.zeros(1, dtype=torch.float64), torch.ones(1, dtype=torch.uint8)
+    with pytest.raises(ValueError):
+        A.dt_noalloc(A.MHD_GLM, 2, 1.4, 0.4, [D(**d)], U, out, active=act if field == "nb" else None)
+
+
+def test_a_missing_spacing_stays_refused():
+    d = D(n=(5, 6, 7), nb=(1, 1, 1), dx=(0.1, None, 0.3), bc=BC, offset=0)
+    with pytest.raises(TypeError):
+        A.domains_c([d])
+    d.dx = (0.1, float("nan"), 0.3)
+    assert np.isnan(A.domains_c([d])[0].dx[1])
