@@ -190,6 +190,7 @@ int build_items(amrfd_handle* h) {
   for (int g = 0; g < h->nblocks; g++) total_cells += bsize[g];
   const long long want = (total_cells + 8LL * h->nsm - 1) / (8LL * h->nsm);
   const int cell_chunk = (int)std::max<long long>(256, std::min<long long>(4096, (want + 255) / 256 * 256));
+  fi.reserve((size_t)(total_cells * nd / ((long long)h->seg * h->lines) * 5 / 4 + 64));
   for (int pos = 0; pos < h->nblocks; pos++) {
     const int g = ord[pos], d = bdom[g], b = bloc[g];
     const DomDev& dm = h->hdom[d];

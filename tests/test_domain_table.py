@@ -69,3 +69,21 @@ def test_a_missing_spacing_stays_refused():
         A.domains_c([d])
     d.dx = (0.1, float("nan"), 0.3)
     assert np.isnan(A.domains_c([d])[0].dx[1])
+
+
+@pytest.mark.parametrize("name", [c for c in CASES if CASES[c]])
+@pytest.mark.parametrize("few", [0, 100], ids=["table", "one_by_one"])
+def test_both_ways_of_filling_give_the_same_records(few, name, monkeypatch):
+    monkeypatch.setattr(A, "_FEW", few)
+    doms = CASES[name]
+    arr, nblocks, need = A._domain_records(doms, 9)
+    assert bytes(arr) == bytes(_plain(doms))
+    assert nblocks == sum(int(d.nb[0]) * int(d.nb[1]) * int(d.nb[2]) for d in doms)
+    assert need == max(int(d.offset) + 9 * int(d.n[0]) * int(d.n[1]) * int(d.n[2]) for d in doms)
+
+
+@pytest.mark.parametrize("few", [0, 100], ids=["table", "one_by_one"])
+@pytest.mark.parametrize("field,value", [("n", (2 ** 32 + 16, 16, 1)), ("nb", (2 ** 32 + 1, 1, 1))])
+def test_both_ways_refuse_sizes_beyond_the_records_types(few, field, value, monkeypatch):
+    monkeypatch.setattr(A, "_FEW", few)
+    test_sizes_beyond_the_records_types_are_not_taken_for_small_ones(field, value)
