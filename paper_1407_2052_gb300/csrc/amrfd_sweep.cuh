@@ -346,14 +346,20 @@ AMRFD_HD void mp5_test(float dm, float d0, float d1, float dp, float& X, float& 
   t = X * fmaf(-60.0f, m, X);
   B = (1.9073486328125e-06f * S) * fmaf(60.0f, fabsf(m), S);
 }
+// Floats of differences are zero exactly where the differences are.
+AMRFD_HD bool equal_cells(float dm, float d0, float d1, float dp) {
+  return fmaxf(fmaxf(fabsf(dm), fabsf(d0)), fmaxf(fabsf(d1), fabsf(dp))) == 0.0f;
+}
 // Whether the acceptance test surely holds, cheaper: with m between 0 and each of d1, 4 d0
 // or outside, t is at most the larger of 30X (30X - 60 d1) and 30X (30X - 240 d0), whose
-// FP32 error is below 0.0091 max|d|^2 (|30X| <= 40 max|d|).
+// FP32 error is below 0.0091 max|d|^2 (|30X| <= 40 max|d|). Equal cells need no threshold: in
+// large units it is below what FP32's products can tell from zero (thr_lo is -kTiny then), and
+// uniform lines of 1e25 or more would all be limited and taken cell by cell.
 AMRFD_HD bool mp5_accepts(float dm, float d0, float d1, float dp, float thr_lo) {
   const float X = fmaf(-3.0f, dp, fmaf(24.0f, d1, fmaf(11.0f, d0, -2.0f * dm)));
   const float q = fmaxf(X * fmaf(-60.0f, d1, X), X * fmaf(-240.0f, d0, X));
   const float mx = fmaxf(fmaxf(fabsf(dm), fabsf(d0)), fmaxf(fabsf(d1), fabsf(dp)));
-  return fmaf(0.01171875f * mx, mx, q) < thr_lo;
+  return fmaf(0.01171875f * mx, mx, q) < thr_lo || mx == 0.0f;
 }
 
 // minmod4(4 ka - kb, 4 kb - ka, ka, kb) in FP32 and its piece (0 zero, 1 ka, 2 kb,
@@ -379,7 +385,7 @@ AMRFD_HD float m4_float(float ka, float kb, float tau, int& piece) {
 AMRFD_HD int mp5_code_float(float dm, float d0, float d1, float dp, float thr_lo) {
   float X, t, B;
   mp5_test(dm, d0, d1, dp, X, t, B);
-  if (t + B < thr_lo) return 0;
+  if (t + B < thr_lo || equal_cells(dm, d0, d1, dp)) return 0;
   // thr_lo lies below the threshold by 2^-20: its upper side is 2^-19 above that
   if (!(t - B > fmaxf(thr_lo * 1.0000020f, kTiny))) return -1;
   const float tau = 7.62939453125e-06f * (fabsf(dm) + fabsf(d0) + fabsf(d1) + fabsf(dp));
@@ -433,7 +439,7 @@ AMRFD_HD int mp5_code_bounded(float dm, float d0, float d1, float dp, float thr_
   constexpr float u = 1.1920929e-07f;  // 2^-23, the differences' relative error
   float X, t, B;
   mp5_test(dm, d0, d1, dp, X, t, B);
-  if (t + B < thr_lo) return 0;
+  if (t + B < thr_lo || equal_cells(dm, d0, d1, dp)) return 0;
   if (!(t - B > fmaxf(thr_lo * 1.0000020f, kTiny))) return -1;
   const float am = fabsf(dm), a0 = fabsf(d0), a1 = fabsf(d1), ap = fabsf(dp);
   const float kL = d0 - dm, kC = d1 - d0, kR = dp - d1;
@@ -660,7 +666,7 @@ AMRFD_HD int mp5_exact(const Wide<RES>& dm, const Wide<RES>& d0, const Wide<RES>
 // the blend band). From FP32, -1 when it cannot tell; thr = 4 (r dx)^2 in squared units.
 AMRFD_HD int limo3_code_float(float a, float b, float thr) {
   const float s2 = fmaf(a, a, b * b);
-  if (s2 < thr * 0.99999809f) return 0;
+  if (s2 < thr * 0.99999809f || (a == 0.0f && b == 0.0f)) return 0;
   if (!(s2 > fmaxf(thr * 1.00000191f, kTiny))) return -1;
   const float sg = b < 0.0f ? -1.0f : 1.0f;
   const float ap = a * sg, bp = b * sg, y3 = fmaf(2.0f, bp, ap) * (1.0f / 3.0f);

@@ -29,6 +29,17 @@ extern "C" void adjoint(int limo, const double* g, int slen, const unsigned shor
   if (limo) adjoint_sweep<true>(g, slen, t, -2, slen + 2, 0, slen - 1, gp, gm, 1);
   else adjoint_sweep<false>(g, slen, t, -2, slen + 2, 0, slen - 1, gp, gm, 1);
 }
+// The cells a three-limb sweep leaves to the exact arithmetic.
+extern "C" int left(int limo, const double* gp, const double* gm, int plen, double thr) {
+  double out[64];
+  int lob, limited = 0;
+  bool bad;
+  if (!window_scale<3, false>(gp, gm, 0, plen + 6, lob, bad)) return -1;
+  const unsigned long long todo =
+      limo ? sweep_part<true, false, 3>(gp, gm, plen, thr, out, 1, ~0ull, 0, 0, 0, 0, 0, lob, limited)
+           : sweep_part<false, false, 3>(gp, gm, plen, 0.0, out, 1, ~0ull, 0, 0, 0, 0, 0, lob, limited);
+  return __builtin_popcountll(todo & ((1ull << plen) - 1ull));
+}
 extern "C" double weight(double dtb, double dx) { return stage_weight(dtb, dx); }
 """
 
@@ -45,6 +56,7 @@ def lib(tmp_path_factory):
                     "-o", str(so)], check=True)
     L = ctypes.CDLL(str(so))
     L.wide.restype, L.wide.argtypes = ctypes.c_double, [ctypes.c_longlong, ctypes.c_ulonglong]
+    L.left.argtypes = [ctypes.c_int] + [ctypes.c_void_p] * 2 + [ctypes.c_int, ctypes.c_double]
     L.weight.restype, L.weight.argtypes = ctypes.c_double, [ctypes.c_double] * 2
     L.sweep.argtypes = [ctypes.c_int] + [ctypes.c_void_p] * 2 + [ctypes.c_int, ctypes.c_double] + [ctypes.c_void_p] * 3
     L.adjoint.argtypes = [ctypes.c_int, ctypes.c_void_p, ctypes.c_int] + [ctypes.c_void_p] * 3
@@ -140,3 +152,12 @@ def test_stage_weight_rounds_once_on_power_of_two_grids(lib):
     for _ in range(3000):
         dtb, k = float(rng.uniform(1e-6, 1.0)), int(rng.integers(0, 14))
         assert lib.weight(dtb, 2.0 ** -k) == float(Fraction(dtb) * 2 ** k / 120)
+
+
+@pytest.mark.parametrize("limo", [0, 1], ids=["mp5", "limo3"])
+@pytest.mark.parametrize("size", [1.0, 1e20, 1e25, 1e30, 1e100, 1e290])
+def test_uniform_lines_in_any_units_leave_no_cell(lib, size, limo):
+    g, h = np.full(38, size), np.full(38, -0.3 * size)
+    assert lib.left(limo, g.ctypes.data, h.ctypes.data, 32, 1e-4) == 0
+    g[:10] *= 1.5  # and the cells whose stencils are uniform, beside a jump
+    assert lib.left(limo, g.ctypes.data, h.ctypes.data, 32, 1e-4) <= 10
