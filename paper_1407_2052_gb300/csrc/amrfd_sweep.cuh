@@ -668,6 +668,7 @@ AMRFD_HD int limo3_code_float(float a, float b, float thr) {
   const float s2 = fmaf(a, a, b * b);
   if (s2 < thr * 0.99999809f || (a == 0.0f && b == 0.0f)) return 0;
   if (!(s2 > fmaxf(thr * 1.00000191f, kTiny))) return -1;
+  if (a == 0.0f || b == 0.0f) return 1 << 3;  // exactly zero, as the exact selection names it
   const float sg = b < 0.0f ? -1.0f : 1.0f;
   const float ap = a * sg, bp = b * sg, y3 = fmaf(2.0f, bp, ap) * (1.0f / 3.0f);
   const float c2 = -0.5f * ap, c3 = 2.0f * ap, c4 = 1.6f * bp;

@@ -161,3 +161,19 @@ def test_uniform_lines_in_any_units_leave_no_cell(lib, size, limo):
     assert lib.left(limo, g.ctypes.data, h.ctypes.data, 32, 1e-4) == 0
     g[:10] *= 1.5  # and the cells whose stencils are uniform, beside a jump
     assert lib.left(limo, g.ctypes.data, h.ctypes.data, 32, 1e-4) <= 10
+
+
+@pytest.mark.parametrize("step", [1, 2, 3, 5, 9])
+def test_steps_between_flat_states_leave_no_cell_with_limo3(lib, step):
+    """A difference of exactly zero beside another one gives a face value of zero by several of
+    LIMO3's pieces; FP32 and the exact selection give it the same name."""
+    rng, thr = np.random.default_rng(step), 1e-14
+    for _ in range(20):
+        g, h = (np.repeat(rng.uniform(0.5, 1.5, 60 // step + 1), step)[:60] for _ in range(2))
+        left = lib.left(1, g.ctypes.data, h.ctypes.data, 54, thr)
+        assert left == 0 if step > 1 else left <= 2
+        out, tp, tm = _sweep(lib, 1, g, h, thr)
+        assert out.tolist() == [float(x) for x in _reference(1, g, h, thr)]
+        for k in range(3, 58):
+            a, b = g[k - 1] - g[k - 2], g[k] - g[k - 1]
+            assert a * b != 0 or tp[k - 3] == (0 if a == b else 8)
