@@ -362,11 +362,29 @@ int tile_lines(const amrfd_handle* h, int seg, int threads) {
 // 123x95x78 Euler 2.79 and 3.11 ms, 21x168x112 Euler 1.71 and 2.14, 75x62x96 MHD 2.40 and
 // 2.53), and from sixteen tiles per CTA on; 160 below (512^2: 0.111 against 0.119 ms per
 // launch, the last wave of tiles shorter).
+// In 1D a tile is one line: few sweeps, and threads beyond them only wait at the barriers
+// (320 threads from 8e4 cells on: 4797 us for 1e6 cells of Euler, 4355 of MHD; with the FP64
+// sweeps 1809 and 2623). From two segments of 64 per SM on it takes those, the longest, and as
+// many threads as 20 warps per SM leave to each, down to one warp: 3e4, 2e5 and 1e6 cells of
+// Euler 138, 245 and 530 us (segments of 16 with 64 threads 147 at 3e4), of MHD 217, 536 and
+// 1510. Below, shorter segments give more CTAs (level at 2e4 cells).
 void default_tile(const amrfd_handle* h, int& seg, int& lines, int& threads) {
-  seg = h->part == 16 ? 32 : 16;
-  lines = tile_lines(h, seg, kFluxMaxThreads);
   long long cells = 0;
   for (auto& dm : h->hdom) cells += dm.ncell;
+  seg = h->part == 16 ? 32 : 16;
+  if (h->cfg.ndim == 1) {
+    const long long tiles = cells / 64;
+    lines = 1;
+    if (tiles >= 2LL * h->nsm) {
+      seg = 64;
+      const int fair = (int)(20LL * h->nsm / tiles + 1) * 32;
+      threads = std::min(fair, std::max(96, tile_threads(h, seg, lines, 1)));
+    } else {
+      threads = tile_threads(h, seg, lines, 1);
+    }
+    return;
+  }
+  lines = tile_lines(h, seg, kFluxMaxThreads);
   if ((h->cfg.ndim == 3 && h->part >= 8) || cells * h->cfg.ndim / ((long long)seg * lines) >= 32LL * h->nsm) {
     threads = kFluxMaxThreads;
   } else {
@@ -1180,13 +1198,32 @@ int amrfd_autotune(amrfd_handle* h, double* U, const double* dt_dev, void* strea
     int rc = speeds_from_scratch(h, U, 0, 0, true, std::vector<int>(), s);
     if (rc) return rc;
   }
-  const int segs[] = {16, 32, 64};
   int best_seg = h->seg, best_lines = h->lines, best_thr = h->threads;
   float best = 1e30f;
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
-  for (int sg : segs) {
+  auto time_tile = [&](int sg, int ln, int thr) {
+    if (configure_tile(h, sg, ln, thr)) return;
+    if (compact(h, s)) return;
+    FluxParams fp = flux_params(h, U, U, 0);
+    fp.items = h->d_fact; fp.nitems_dev = h->d_counts; fp.counter = h->d_counters;
+    float tot = 1e30f;
+    bool ok = true;
+    for (int rep = 0; rep < 5 && ok; rep++) {
+      if (cudaMemsetAsync(h->d_counters, 0, sizeof(int), s) != cudaSuccess) ok = false;
+      cudaEventRecord(e0, s);
+      if (launch_flux(h->cfg.physics, h->nv, fp, h->flux_grid, h->launch_threads, h->flux_smem, s) != cudaSuccess) ok = false;
+      cudaEventRecord(e1, s);
+      if (cudaEventSynchronize(e1) != cudaSuccess) ok = false;
+      float ms = 0.f;
+      cudaEventElapsedTime(&ms, e0, e1);
+      if (rep > 0) tot = std::min(tot, ms);  // best of four after one warm-up launch
+    }
+    if (ok && tot < best) { best = tot; best_seg = sg; best_lines = ln; best_thr = thr; }
+  };
+  if (h->cfg.ndim == 1) time_tile(best_seg, best_lines, best_thr);  // its threads are none of those below
+  for (int sg : {16, 32, 64}) {
     int prev = 0;
     for (int full : {160, kFluxMaxThreads}) {
       const int ln = tile_lines(h, sg, full);
@@ -1197,23 +1234,7 @@ int amrfd_autotune(amrfd_handle* h, double* U, const double* dt_dev, void* strea
         const int thr = tile_threads(h, sg, ln, extra);
         if (thr == last) continue;
         last = thr;
-        if (configure_tile(h, sg, ln, thr)) continue;
-        if (compact(h, s)) continue;
-        FluxParams fp = flux_params(h, U, U, 0);
-        fp.items = h->d_fact; fp.nitems_dev = h->d_counts; fp.counter = h->d_counters;
-        float tot = 1e30f;
-        bool ok = true;
-        for (int rep = 0; rep < 5 && ok; rep++) {
-          if (cudaMemsetAsync(h->d_counters, 0, sizeof(int), s) != cudaSuccess) ok = false;
-          cudaEventRecord(e0, s);
-          if (launch_flux(h->cfg.physics, h->nv, fp, h->flux_grid, h->launch_threads, h->flux_smem, s) != cudaSuccess) ok = false;
-          cudaEventRecord(e1, s);
-          if (cudaEventSynchronize(e1) != cudaSuccess) ok = false;
-          float ms = 0.f;
-          cudaEventElapsedTime(&ms, e0, e1);
-          if (rep > 0) tot = std::min(tot, ms);  // best of four after one warm-up launch
-        }
-        if (ok && tot < best) { best = tot; best_seg = sg; best_lines = h->lines; best_thr = thr; }
+        time_tile(sg, ln, thr);
       }
     }
   }

@@ -1,0 +1,48 @@
+"""The default tile of a handle, on the GPU: threads that have work, segments that fit it."""
+import pytest
+
+from paper_1407_2052_gb300 import workloads as W
+from test_gpu_parity import A
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__ as g
+    g.build()
+
+
+def _tile(physics, n, nb, tune=False):
+    nd = sum(m > 1 for m in n)
+    s = A().Solver(physics, nd, A().SSPRK3, 1.4, 0.4, [W.Domain(n, (1.0 / n[0],) * 3, nb=nb)], glm_cr=0.18)
+    if tune:
+        U = torch.ones(s.nv * n[0], dtype=torch.float64, device="cuda")
+        U[-n[0]:] = 10.0  # Euler's energy
+        s.autotune(U, torch.full((1,), 1e-6, dtype=torch.float64, device="cuda"))
+    t = s.get_tile()
+    s.close()
+    return t
+
+
+@pytest.mark.parametrize("physics", [0, 1])
+@pytest.mark.parametrize("n", [48, 512, 19000, 19500, 70000, 80000, 1000000, 4000000])
+def test_a_tube_takes_no_more_threads_than_a_line_has_work(physics, n):
+    """A tile of one line has few sweeps: beyond them threads wait. Many lines (a large tube)
+    fill the GPU with one warp each."""
+    nb = 1 if n < 32000 else n // 10000
+    seg, lines, threads = _tile(physics, (n, 1, 1), (nb, 1, 1))
+    assert lines == 1 and 32 <= threads <= 160
+    if n >= 1000000:
+        assert seg == 64 and threads == 32
+    if n <= 512:
+        assert seg == 16
+
+
+def test_tuning_a_tube_times_its_default_tile():
+    n = 1000000
+    assert _tile(0, (n, 1, 1), (100, 1, 1), tune=True)[2] <= 64
