@@ -364,20 +364,24 @@ int tile_lines(const amrfd_handle* h, int seg, int threads) {
 // launch, the last wave of tiles shorter).
 // In 1D a tile is one line: few sweeps, and threads beyond them only wait at the barriers
 // (320 threads from 8e4 cells on: 4797 us for 1e6 cells of Euler, 4355 of MHD; with the FP64
-// sweeps 1809 and 2623). From two segments of 64 per SM on it takes those, the longest, and as
-// many threads as 20 warps per SM leave to each, down to one warp: 3e4, 2e5 and 1e6 cells of
-// Euler 138, 245 and 530 us (segments of 16 with 64 threads 147 at 3e4), of MHD 217, 536 and
-// 1510. Below, shorter segments give more CTAs (level at 2e4 cells).
+// sweeps 1809 and 2623). From two segments of 64 per SM on it takes those, the longest, and a
+// thread per sweep, or as few warps as 30 per SM leave to each tile of the largest domain:
+// 3e4, 2e5 and 1e6 cells of Euler 116, 201 and 530 us (segments of 16 with 64 threads 130, 351
+// and 1700), of MHD 168, 466 and 1510 (178, 606 and 3100). The largest domain, since the plain
+// path launches one at a time: 40 tubes of 5000 cells of MHD 8.8 ms with one warp a tile, 6.2
+// with three. Below, shorter segments give more CTAs (level at 2e4 cells).
 void default_tile(const amrfd_handle* h, int& seg, int& lines, int& threads) {
-  long long cells = 0;
-  for (auto& dm : h->hdom) cells += dm.ncell;
+  long long cells = 0, largest = 0;
+  for (auto& dm : h->hdom) {
+    cells += dm.ncell;
+    largest = std::max<long long>(largest, dm.ncell);
+  }
   seg = h->part == 16 ? 32 : 16;
   if (h->cfg.ndim == 1) {
-    const long long tiles = cells / 64;
     lines = 1;
-    if (tiles >= 2LL * h->nsm) {
+    if (cells / 64 >= 2LL * h->nsm) {
       seg = 64;
-      const int fair = (int)(20LL * h->nsm / tiles + 1) * 32;
+      const int fair = (int)(30LL * h->nsm / std::max(1LL, largest / 64) + 1) * 32;
       threads = std::min(fair, std::max(96, tile_threads(h, seg, lines, 1)));
     } else {
       threads = tile_threads(h, seg, lines, 1);

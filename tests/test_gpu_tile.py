@@ -43,6 +43,14 @@ def test_a_tube_takes_no_more_threads_than_a_line_has_work(physics, n):
         assert seg == 16
 
 
+def test_small_tubes_of_a_large_batch_keep_a_thread_per_sweep():
+    """The plain path launches one domain at a time: nothing else fills the GPU then."""
+    doms = [W.Domain((5000, 1, 1), (2e-4, 1.0, 1.0), offset=i * 9 * 5000) for i in range(40)]
+    s = A().Solver(A().MHD_GLM, 1, A().SSPRK3, 1.4, 0.4, doms, glm_cr=0.18)
+    assert s.get_tile()[2] >= 72  # nine variables in parts of 8 cells of a segment of 64
+    s.close()
+
+
 def test_tuning_a_tube_times_its_default_tile():
     n = 1000000
     assert _tile(0, (n, 1, 1), (100, 1, 1), tune=True)[2] <= 64
