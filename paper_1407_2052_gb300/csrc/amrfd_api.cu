@@ -317,13 +317,18 @@ int configure_tile(amrfd_handle* h, int seg, int lines, int threads) {
 // that fills the GPU with 20 warps per SM; shorter parts, hence shorter chains of dependent
 // faces and more warps, where it does not: a launch then lasts as long as one sweep (128^2
 // Euler blast: 43 us with 4 cells, 95 with whole segments of 16 in FP64; on the 256^3 MHD
-// blast parts of 8 to 12 measured 5 to 15 % slower than 16). The line for 16 lies at two waves:
-// just above one, 42x36x42 MHD took 1.03 ms a step with parts of 16 and 0.96 with 8.
+// blast parts of 8 to 12 measured 5 to 15 % slower than 16). The line for 16 lies where the
+// two cross, by whole steps of blasts and of waves (us, 8 cells in segments of 16 and 16 in
+// segments of 32): at 17 waves of faces 48^3 Euler 400 and 446, 486 and 510; at 18 42x36x42
+// MHD 487 and 464, 601 and 590; at 20 20x90x40 MHD 513 and 490, 722 and 666; at 22 512^2 Euler
+// 455 and 448, 321 and 297; at 25 57x38x76 Euler 584 and 542, 715 and 655; at 28 400x380 MHD
+// 598 and 534, 434 and 392; at 31 48^3 MHD 571 and 579, 876 and 826. In 1D 16 cells start later
+// (5e5 cells of MHD 902 and 875; 1e6 of Euler, 31 waves, 531 and 619).
 int choose_part(const amrfd_handle* h) {
   long long cells = 0;
   for (auto& dm : h->hdom) cells += dm.ncell;
   const long long faces = cells * h->cfg.ndim * h->nv / 32, room = 20LL * h->nsm;
-  return faces >= 32 * room ? 16 : (faces >= 8 * room ? 8 : 4);
+  return faces >= (h->cfg.ndim == 1 ? 32 : 18) * room ? 16 : (faces >= 8 * room ? 8 : 4);
 }
 
 // Sweeps per line of the longest segment of a dimension, as build_items cuts it.

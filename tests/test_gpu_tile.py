@@ -54,3 +54,10 @@ def test_small_tubes_of_a_large_batch_keep_a_thread_per_sweep():
 def test_tuning_a_tube_times_its_default_tile():
     n = 1000000
     assert _tile(0, (n, 1, 1), (100, 1, 1), tune=True)[2] <= 64
+
+
+@pytest.mark.parametrize("physics, n, nb, seg", [
+    (0, (48, 48, 48), (3, 3, 3), 16), (0, (57, 38, 76), (3, 2, 4), 32), (0, (512, 512, 1), (1, 1, 1), 32),
+    (1, (36, 36, 36), (3, 3, 3), 16), (1, (20, 90, 40), (1, 6, 2), 32), (1, (400, 380, 1), (8, 4, 1), 32)])
+def test_middling_work_takes_long_segments_from_twenty_waves_of_faces_on(physics, n, nb, seg):
+    assert _tile(physics, n, nb)[0] == seg
