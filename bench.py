@@ -36,15 +36,17 @@ FLUX_BYTES_PER_CELL = 4 * NV * 8
 # FP64 work of the method per cell and direction in the flux pass (flop = DADD + DMUL + 2 DFMA
 # thread instructions; one split flux per cell, one reconstruction per face and bias, no
 # segment overheads), counted by ncu on a build that did all of it in FP64: a + b/S at
-# segments of S cells, a = 254.4. The kernel now does the reconstructions in exact fixed
-# point on the integer units, so this is the work delivered, not the FP64 instructions
-# executed (split flux, conversions).
+# segments of S cells, a = 254.4. The kernel does the reconstructions in exact fixed point on
+# the integer units, so this is work delivered ("equivalent"), no use of the FP64 pipe.
 FLUX_FLOPS_PER_CELL_DIR = 254.4
+# What the flux kernel executes per cell of one launch (all three directions), by ncu on the
+# 128^3 blast's first flux pass with the default tile: warp instructions, FP64 flop, and DRAM
+# bytes (read + write; traffic grows with the cells processed). A later step, with more faces
+# limited, executes more.
+FLUX_WARP_INST_PER_CELL = 920.090131e6 / 128 ** 3
+FLUX_FP64_FLOP_PER_CELL = (2 * 248.169404 + 9.432699 + 0.182142) * 1e6 / 128 ** 3
+FLUX_TRAFFIC_BYTES_PER_CELL = (369.609216 + 416.706048) * 1e6 / 128 ** 3
 FP64_PEAK_TFLOPS_NOMINAL = 1.25   # GB300 FP64, nominal (context only)
-# DRAM bytes per cell of one flux launch (ncu dram__bytes_read + write of the 128^3 blast's
-# first flux pass, tile 64 x 8 lines x 320 threads, scaled by cells): traffic grows with
-# the cells processed
-FLUX_TRAFFIC_BYTES_PER_CELL = (443.714560 + 413.586944) * 1e6 / 128 ** 3
 
 
 def _env_int(k, d):
@@ -88,6 +90,27 @@ def clocks_summary(path, gpu_index):
         return {"sm_mhz": None, "sm_max_mhz": None, "reasons": [], "samples": 0}
     sm.sort()
     return {"sm_mhz": sm[len(sm) // 2], "sm_max_mhz": mx, "reasons": sorted(reasons), "samples": len(sm)}
+
+
+def flux_roofline(seconds, ncell, nsm, sm_mhz, fp64):
+    """Use of what bounds the flux launch, instruction issue: one warp instruction a clock and
+    SM sub-partition. Beside it the FP64 pipe's share, and the method's FP64 work over the
+    launch time, which is no use of that pipe."""
+    issued = FLUX_WARP_INST_PER_CELL * ncell / seconds / 1e9
+    peak = 4 * nsm * sm_mhz * 1e-3
+    executed = FLUX_FP64_FLOP_PER_CELL * ncell / seconds / 1e12
+    equivalent = FLUX_FLOPS_PER_CELL_DIR * 3 * ncell / seconds / 1e12
+    return {"bound": "alu", "unit": "Ginst/s", "achieved": issued, "peak": peak, "frac": issued / peak,
+            "traffic": FLUX_TRAFFIC_BYTES_PER_CELL * ncell, "kernel": "flux_kernel", "launch_ms": seconds * 1e3,
+            "note": "warp instructions of the launch (ncu, 128^3, scaled by cells) over its time",
+            "peak_source": "one warp instruction per clock and SM sub-partition at the SM clock of the timed region",
+            "executed_fp64": {"tflops": executed, "frac": executed / fp64["sustained_tflops"]},
+            "equivalent_fp64": {"tflops": equivalent, "over_peak": equivalent / fp64["sustained_tflops"],
+                                "flop_per_cell_dir": FLUX_FLOPS_PER_CELL_DIR},
+            "fp64_peak_tflops": fp64["sustained_tflops"],
+            "fp64_peak_source": "measured: amrfd_fp64_peak, independent FP64 FMAs on every SM, back to back for 2 s "
+                                "(sustained); burst %.3f TFLOP/s" % fp64["burst_tflops"],
+            "fp64_peak_nominal": FP64_PEAK_TFLOPS_NOMINAL}
 
 
 def aggregate(ms_local, cells_per_rank, steps, world, dist=None, device="cpu"):
@@ -610,16 +633,8 @@ def run_ours(args, rank, world, local_rank):
     hbm_peak = peaks.get("hbm_gbs", 6800.0)
     # the FP64 rate this GPU sustains, measured here (the flux pass runs inside a long step)
     fp64 = A.fp64_peak(seconds=2.0)
-    achieved = FLUX_FLOPS_PER_CELL_DIR * 3 * ncell / flux_avg_s / 1e12
-    roof = {"bound": "alu", "unit": "TFLOP/s", "achieved": achieved, "peak": fp64["sustained_tflops"],
-            "frac": achieved / fp64["sustained_tflops"], "traffic": FLUX_TRAFFIC_BYTES_PER_CELL * ncell,
-            "kernel": "flux_kernel", "launch_ms": flux_avg_s * 1e3,
-            "flop_per_cell_dir": FLUX_FLOPS_PER_CELL_DIR,
-            "note": "achieved: the method's FP64 work over the launch time; the reconstructions run in exact fixed "
-                    "point on the integer units, so the FP64 pipe executes less",
-            "peak_source": "measured: amrfd_fp64_peak, independent FP64 FMAs on every SM, back to back for 2 s "
-                           "(sustained); burst %.3f TFLOP/s" % fp64["burst_tflops"],
-            "peak_nominal": FP64_PEAK_TFLOPS_NOMINAL}
+    nsm = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
+    roof = flux_roofline(flux_avg_s, ncell, nsm, clocks["sm_mhz"] or 2070.0, fp64)
     flux_gbs = FLUX_BYTES_PER_CELL * ncell / flux_avg_s / 1e9
     out = {
         "metric": "3D MHD FD-MP5 cell-updates/s (FP64)",
