@@ -12,18 +12,19 @@
 // arithmetic.
 //
 // Measured, the whole flux launch (FP64 sweeps before, these after): 1024^2 MHD vortex 768
-// and 360 us, 256^3 MHD blast in noise 16.1 and 10.6 ms (it limits at half its faces; 7.3
-// without), 128^3 MHD blast with LIMO3 2.12 and 0.97 ms. What bounds them now: integer
-// issue (50 to 60 % of the slots, about 490 instructions a face and warp where the limiter
-// runs, 230 where not) and, at 40 %, the FP64 pipe (phase A and one conversion a cell).
+// and 352 us, 256^3 MHD blast in noise 16.1 and 10.2 ms (it limits at half its faces; 10.7 in
+// later steps, up to 12.9 while tails run through the box, see wide_sweep), 128^3 MHD blast
+// with LIMO3 2.12 and 0.97 ms. What bounds them now: integer issue (50 to 60 % of the slots,
+// about 490 instructions a face and warp where the limiter runs, 230 where not) and, at 35 %,
+// the FP64 pipe (phase A and one conversion a cell).
 //
 // Scale. A sweep works at one power-of-two scale at which every cell of its part is a whole
 // number: of 66 bits (three limbs) where the cells' exponents span at most 13 binades, of 88
-// (four limbs, 35 binades) or of 110 bits (five limbs, about 1.8 times the work). A sine
-// that crosses zero is past 13 binades in most warps, hence the four: 75x62x96 MHD waves
-// 2.40 ms a step without them and 2.15 with, 42x36x42 0.87 and 0.80. Nothing is rounded then, so the
-// results do not depend on the scale, hence not on where a sweep starts. Where a part spans
-// more than 110 bits, the cells whose window holds a value that is no whole number are left
+// (four limbs, 35 binades) or of 110 bits (five limbs). A sine that crosses zero is past 13
+// binades in most warps, hence the four: 75x62x96 MHD waves 2.40 ms a step without them and
+// 2.15 with, 42x36x42 0.87 and 0.80. Nothing is rounded then, so the results do not depend on
+// the scale, hence not on where a sweep starts. Where a part spans more than 110 bits it is cut
+// (wide_sweep), and the cells whose window still holds a value that is no whole number are left
 // to exact_cell, which takes each by itself at its own window's scale; where a seven-cell
 // window spans more, it carries what the units of 2^-110 of the largest value leave over as
 // doubles besides (Wide), so that a component that is weak next to a strong one keeps its
@@ -154,25 +155,34 @@ AMRFD_HD Limbs<3> limbs(int hi, unsigned lo, int lob) {
   return r;
 }
 
+// The limbs of a mantissa m shifted left by L <= 57, of sign sg.
+AMRFD_HD Limbs<5> limbs5(unsigned mh, unsigned ml, int L, int sg) {
+  const unsigned a0 = shf_l(0u, ml, L), a1 = shf_l(ml, mh, L), a2 = shf_l(mh, 0u, L);  // by L & 31
+  const bool up = L >= 32;
+  const unsigned w0 = up ? 0u : a0, w1 = up ? a0 : a1, w2 = up ? a1 : a2, w3 = up ? a2 : 0u;
+  Limbs<5> r;
+  r.v[0] = (int)(w0 & (unsigned)kLimbMask) * sg;
+  r.v[1] = (int)(shf_r(w0, w1, 22) & (unsigned)kLimbMask) * sg;
+  r.v[2] = (int)(shf_r(w1, w2, 12) & (unsigned)kLimbMask) * sg;
+  r.v[3] = (int)((w2 >> 2) & (unsigned)kLimbMask) * sg;
+  r.v[4] = (int)shf_r(w2, w3, 24) * sg;
+  return r;
+}
 // The limbs of any value below the top, rounded to the unit (half away from zero; exact for
-// whole multiples of it).
+// whole multiples of it); FIT: of one whose exponent lies in [lob >> 20, (lob >> 20) + 57].
+template <bool FIT = false>
 AMRFD_HD Limbs<5> limbs_wide(int hi, unsigned lo, int lob) {
   const int x = hi & 0x7fffffff;
   int L = (x - lob) >> 20;
-  unsigned long long m = ((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32) | lo;
-  if (L < 0) {
-    m = L < -54 ? 0ull : (m + (1ull << (-L - 1))) >> -L;
+  unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+  if (!FIT && L < 0) {
+    const unsigned long long m = ((unsigned long long)mh << 32) | lo;
+    const unsigned long long r = L < -54 ? 0ull : (m + (1ull << (-L - 1))) >> -L;
+    mh = (unsigned)(r >> 32);
+    lo = (unsigned)r;
     L = 0;
   }
-  const int sg = x ? ((hi >> 31) | 1) : 0;
-  Limbs<5> r;
-#pragma unroll
-  for (int l = 0; l < 5; l++) {
-    const int p = kLimb * l - L;  // first bit of the limb in m
-    const unsigned long long t = p >= 0 ? (p < 64 ? m >> p : 0ull) : (p > -kLimb ? m << -p : 0ull);
-    r.v[l] = (int)((unsigned)t & (unsigned)kLimbMask) * sg;
-  }
-  return r;
+  return limbs5(mh, lo, L, x ? ((hi >> 31) | 1) : 0);
 }
 // The same as limbs with four limbs: exponents in [lob >> 20, (lob >> 20) + 35].
 AMRFD_HD Limbs<4> limbs4(int hi, unsigned lo, int lob) {
@@ -260,11 +270,8 @@ AMRFD_HD double to_double(const Limbs<3>& A, const Limbs<3>& B, int lob) {
 #endif
   return scaled(x, adj);
 }
-// The same for one number of four limbs, each below 2^31.
-AMRFD_HD double to_double(const Limbs<4>& d, int lob) {
-  const long long W = (long long)d.v[1] * (1 << 22) + d.v[0];
-  const long long X = (long long)d.v[3] * (1 << 22) + d.v[2] + (W >> 44);  // the sum >> 44
-  const unsigned long long r = (unsigned long long)W & ((1ull << 44) - 1);
+// The double nearest to X 2^44 + r, 0 <= r < 2^44, in units of 2^(adj >> 20).
+AMRFD_HD double round_sum(long long X, unsigned long long r, int adj) {
   const long long a = X ^ (X >> 63);
 #ifdef __CUDACC__
   const int nb = 64 - __clzll(a);
@@ -279,16 +286,41 @@ AMRFD_HD double to_double(const Limbs<4>& d, int lob) {
 #else
   const double x = (double)V;
 #endif
-  return scaled(x, lob - (1075 << 20) + (sh << 20));
+  return scaled(x, adj + (sh << 20));
+}
+// The same for one number of four limbs, each below 2^31.
+AMRFD_HD double to_double(const Limbs<4>& d, int lob) {
+  const long long W = (long long)d.v[1] * (1 << 22) + d.v[0];
+  const long long X = (long long)d.v[3] * (1 << 22) + d.v[2] + (W >> 44);  // the sum >> 44
+  return round_sum(X, (unsigned long long)W & ((1ull << 44) - 1), lob - (1075 << 20));
 }
 AMRFD_HD double to_double(const Limbs<4>& A, const Limbs<4>& B, int lob) {
   return to_double(Limbs<4>{{A.v[0] - B.v[0], A.v[1] - B.v[1], A.v[2] - B.v[2], A.v[3] - B.v[3]}}, lob);
+}
+// Five: one conversion too (two and two more FP64 operations through 128 bits cost a sweep
+// 256 cycles a cell).
+AMRFD_HD double to_double(const Limbs<5>& d, int lob) {
+  constexpr unsigned long long low = (1ull << 44) - 1;
+  const long long W = (long long)d.v[1] * (1 << 22) + d.v[0];
+  const long long X = (long long)d.v[3] * (1 << 22) + d.v[2] + (W >> 44);
+  long long Z = d.v[4] + (X >> 44);  // the sum >> 88, below 2^32
+  unsigned long long x = (unsigned long long)X & low, r = (unsigned long long)W & low;
+  const bool large = (unsigned long long)(Z + (1 << 18)) >= (1ull << 19);  // then the lowest 44 bits into a sticky one
+  int adj = lob - (1075 << 20);
+  if (large) {
+    x |= r != 0;
+    r = x;
+    adj += 44 << 20;
+  } else {
+    Z = (long long)((unsigned long long)Z << 44) + (long long)x;
+  }
+  return round_sum(Z, r, adj);
 }
 AMRFD_HD double to_double(const Limbs<5>& A, const Limbs<5>& B, int lob) {
   Limbs<5> d;
 #pragma unroll
   for (int l = 0; l < 5; l++) d.v[l] = A.v[l] - B.v[l];
-  return scaled(wide_double(to_wide(d)), lob - (1075 << 20));
+  return to_double(d, lob);
 }
 
 // ----------------------------------------------------------------------- MP5
@@ -905,17 +937,37 @@ template <bool LIMO>
 AMRFD_HD double linear_value(line_t gp, line_t gm, int j, int top) {
   constexpr int NC = LIMO ? 4 : 6;
   const int lob = (top - room(5) < kExpUnit ? kExpUnit : top - room(5)) << 20;
-  const Unit un = unit_of(lob);
-  Wide<true> F = {0, 0.0};
+  const bool low = lob == kExpUnit << 20;  // values below the smallest unit count too
+  const Unit un = low ? unit_of(lob) : Unit{0.0, 0.0};
+  Limbs<5> F = {};
+  double rest = 0.0;
 #pragma unroll
   for (int q = 0; q < NC; q++) {
     const int w = LIMO ? (q == 0 ? -10 : (q == 1 ? 60 : (q == 2 ? -30 : -20)))
                        : (q == 0 ? 2 : (q == 1 ? -15 : (q == 2 ? 60 : (q == 3 ? -20 : (q == 4 ? -30 : 3)))));
-    const Wide<true> a = wide_cell<true>(gp, j + q, lob, un), b = wide_cell<true>(gm, j + NC - q, lob, un);
-    F.h += (a.h - b.h) * w;
-    if (lob == kExpUnit << 20) F.r = fma((double)w, a.r - b.r, F.r);  // no large value
+    int ah, bh;
+    unsigned al, bl;
+    cell_words(gp, j + q, ah, al);
+    cell_words(gm, j + NC - q, bh, bl);
+    const Limbs<5> a = limbs_wide(ah, al, lob), b = limbs_wide(bh, bl, lob);
+#pragma unroll
+    for (int l = 0; l < 5; l++) F.v[l] += w * (a.v[l] - b.v[l]);
+    if (low)
+      rest = fma((double)w, wide_cell<true>(gp, j + q, lob, un).r - wide_cell<true>(gm, j + NC - q, lob, un).r, rest);
   }
-  return nearest(lin(1, F, 0, F, un), un, lob);
+  if (!low) return to_double(F, lob);
+  Wide<true> f = {to_wide(F), rest};
+  carry_units(f, un);
+  return nearest(f, un, lob);
+}
+
+// Whether no face can be limited whose cells' exponents are most at most: differences lie below
+// 2 x, 30X (30X - 30mp) below 16000 x^2, LIMO3's a^2 + b^2 below 8 x^2.
+template <bool LIMO>
+AMRFD_HD bool surely_unlimited(int most, double limo_thr) {
+  if (!LIMO) return most - 1022 < -17;
+  const double x = pow2d(most - 1022);
+  return 8.01 * x * x < limo_thr;
 }
 
 // Out of line: its registers stay out of the sweeps'.
@@ -932,10 +984,8 @@ AMRFD_HD_CALL void exact_cell(line_t gp, line_t gm, int i, double limo_thr, doub
     most = m > most ? m : most;
     if (q < NC) top = m > top ? m : top;
   }
-  const double x = pow2d(most - 1022);
   double r;
-  // differences below 2 x: 30X (30X - 30mp) below 16000 x^2, LIMO3's a^2 + b^2 below 8 x^2
-  if (LIMO ? 8.01 * x * x < limo_thr : x < 0x1p-17) {
+  if (surely_unlimited<LIMO>(most, limo_thr)) {
     r = linear_value<LIMO>(gp, gm, j, top);
     record<REC>(tp, tm, f0 + i, fend, fmod, 0, 0);
     record<REC>(tp, tm, f0 + i + 1, fend, fmod, 0, 0);
@@ -1088,11 +1138,112 @@ AMRFD_HD unsigned long long sweep_part(line_t gp, line_t gm, int plen, double li
   return todo;
 }
 
+// The cells of a part whose faces are all surely unlimited (FIT: and whose exponents span at
+// most 57 binades): their differences as a fixed filter (linear_value) by transposed sums, without the face fluxes and FP32 differences of
+// sweep_part.
+template <bool LIMO, bool REC, bool FIT>
+AMRFD_HD void linear_part(line_t gp, line_t gm, int plen, double* out, int ostr, unsigned long long wmask,
+                          unsigned short* tp, unsigned short* tm, int f0, int fend, int fmod, int lob) {
+  constexpr int NC = LIMO ? 4 : 6;
+  constexpr int C0 = LIMO ? 1 : 0;
+  Limbs<5> A[NC];  // A[n]: the cell that lacks n + 1 more
+#pragma unroll
+  for (int q = 0; q < NC; q++) A[q] = Limbs<5>{};
+#pragma unroll 1
+  for (int i = -NC; i < plen; i++) {  // the cell whose last one this is
+    int ph, mh;
+    unsigned pl, ml;
+    cell_words(gp, i + NC + C0, ph, pl);
+    cell_words(gm, i + NC + C0, mh, ml);
+    const Limbs<5> x = limbs_wide<FIT>(ph, pl, lob), y = limbs_wide<FIT>(mh, ml, lob);
+    Limbs<5> F;
+#pragma unroll
+    for (int l = 0; l < 5; l++) {
+      const int g = x.v[l], h = y.v[l];
+      if constexpr (LIMO) {  // -10 g0 + 60 g1 - 30 g2 - 20 g3 + 20 h1 + 30 h2 - 60 h3 + 10 h4
+        F.v[l] = A[0].v[l] + 10 * h;
+        A[0].v[l] = A[1].v[l] - 20 * g - 60 * h;
+        A[1].v[l] = A[2].v[l] - 30 * g + 30 * h;
+        A[2].v[l] = A[3].v[l] + 60 * g + 20 * h;
+        A[3].v[l] = -10 * g;
+      } else {  // 2 g0 - 15 g1 + 60 g2 - 20 g3 - 30 g4 + 3 g5 - 3 h1 + 30 h2 + 20 h3 - 60 h4 + 15 h5 - 2 h6
+        F.v[l] = A[0].v[l] - 2 * h;
+        A[0].v[l] = A[1].v[l] + 3 * g + 15 * h;
+        A[1].v[l] = A[2].v[l] - 30 * g - 60 * h;
+        A[2].v[l] = A[3].v[l] - 20 * g + 20 * h;
+        A[3].v[l] = A[4].v[l] + 60 * g + 30 * h;
+        A[4].v[l] = A[5].v[l] - 15 * g - 3 * h;
+        A[5].v[l] = 2 * g;
+      }
+    }
+    if (i < -1) continue;
+    record<REC>(tp, tm, f0 + i + 1, fend, fmod, 0, 0);
+    if (i < 0) continue;
+    if (wmask & 1ull) *out = to_double(F, lob);
+    out += ostr;
+    wmask >>= 1;
+  }
+}
+
+// fixed_sweep of a part with five limbs: the cells left to exact_cell, and the faces limited.
+// Out of line: most warps hold none, and its registers stay out of the other sweeps'.
+// What comes here is mostly tails ahead of a front: in the MHD blast eight of 27 (variable,
+// direction) pairs, through the whole box. Hence the filter where no face can be limited, and
+// the cuts that keep cells out of exact_cell. 256^3 flux launch in steps 1, 10, 24 and 80:
+// 10.3, 13.0, 19.8 and 14.2 ms with plain five-limb sweeps and each cell over 110 bits by
+// itself, 10.2, 11.0, 12.9 and 10.7 with both; never quarters 12.4 at step 13, from a range of
+// 100, 88 and 76 binades on 12.4, 12.0 and 11.5.
+struct Wide5 {
+  unsigned long long todo;
+  int limited;
+};
+template <bool LIMO, bool REC>
+AMRFD_HD_CALL Wide5 wide_sweep(line_t gp, line_t gm, int plen, double limo_thr, double* out, int ostr,
+                               unsigned long long wmask, unsigned short* tp, unsigned short* tm, int f0, int fend,
+                               int fmod, Span span, unsigned lanes) {
+  constexpr int C0 = LIMO ? 1 : 0;
+  constexpr int NC = LIMO ? 4 : 6;
+  unsigned long long todo = 0ull;
+  int lob, limited = 0;
+  // Halves or quarters where some part spans more than 57 binades: ahead of a front a component
+  // falls off by about three binades a cell, 66 over the cells of a part of 16, 42 over its half's.
+  const int range = span.mn + 1u ? (int)(span.mx >> 20) - (int)((span.mn + 1u) >> 20) : 0;
+  int ns = AMRFD_ANY(lanes, range > 57) && !AMRFD_ANY(lanes, plen < 8) ? 2 : 1;
+  if (ns == 2 && AMRFD_ANY(lanes, range > 76) && !AMRFD_ANY(lanes, plen < 16)) ns = 4;
+#pragma unroll 1
+  for (int s = 0; s < ns; s++) {
+    const int p0 = s * plen / ns, len = (s + 1) * plen / ns - p0;
+    const line_t p = line_at(gp, p0), m = line_at(gm, p0);
+    if (ns > 1) span = window_span<false>(p, m, C0, len + NC);
+    bool bad;
+    const bool fits = span_scale<5>(span, lob, bad);
+    double* o = out + (long long)p0 * ostr;
+    const int fe = s + 1 < ns && f0 + p0 + len + 1 < fend ? f0 + p0 + len + 1 : fend;
+    const bool linear = !AMRFD_ANY(lanes, !surely_unlimited<LIMO>((int)(span.mx >> 20), limo_thr));
+    if (linear && !AMRFD_ANY(lanes, !fits)) {
+      linear_part<LIMO, REC, true>(p, m, len, o, ostr, wmask >> p0, tp, tm, f0 + p0, fe, fmod, lob);
+      continue;
+    }
+    const unsigned long long cells = len < 64 ? (1ull << len) - 1ull : ~0ull;
+    unsigned long long part = 0ull;
+    if (!fits && !window_scale<5, true>(p, m, C0, len + NC, lob, bad))
+      part = partial_cells<LIMO>(p, m, len + NC, lob) & cells;
+    if (linear)
+      linear_part<LIMO, REC, false>(p, m, len, o, ostr, wmask >> p0, tp, tm, f0 + p0, fe, fmod, lob);
+    else if (AMRFD_ANY(lanes, part != cells))
+      part |= sweep_part<LIMO, REC, 5>(p, m, len, limo_thr, o, ostr, wmask >> p0, tp, tm, f0 + p0, fe, fmod, lob,
+                                       limited) & cells;
+    todo |= part << p0;
+  }
+  return {todo, limited};
+}
+
 // One (line, variable): the faces k = 3..plen+3 of the line's extended index (cell j = k-1
 // left of face k) and 60 (Fsum_{k-1} - Fsum_k) of its plen <= 64 cells, Fsum = G+_{k-1} +
 // G-_k + (Y+_k + Y-_k)/2, stored to out[i ostr] where wmask has its bit (the factor
-// 1/(120 dx) is applied by the stage combination). Every lane in `lanes` must call this
-// with the same plen. REC records per face and bias the code of the piece the limiter took:
+// 1/(120 dx) is applied by the stage combination). Every lane in `lanes` must call this: the
+// votes on the number of limbs, before any loop over faces, wait for all of them (parts may
+// differ in length). REC records per face and bias the code of the piece the limiter took:
 // face k at index f0 + k - 3 if below fend (face fmod as face 0). Returns the number of
 // faces at which the lane's limiter was needed.
 // A cell enters the partial sums of the faces it belongs to when it is read (a transposed
@@ -1104,7 +1255,8 @@ AMRFD_HD int fixed_sweep(line_t gp, line_t gm, int plen, double limo_thr, double
                          unsigned long long wmask, unsigned short* tp, unsigned short* tm, int f0, int fend, int fmod,
                          unsigned lanes) {
   constexpr int C0 = LIMO ? 1 : 0;
-  const int nc = plen + 6 - 2 * C0;
+  constexpr int NC = LIMO ? 4 : 6;
+  const int nc = plen + NC;
   int lob, limited = 0;
   bool bad;
   const Span span = window_span<false>(gp, gm, C0, nc);
@@ -1115,10 +1267,9 @@ AMRFD_HD int fixed_sweep(line_t gp, line_t gm, int plen, double limo_thr, double
   } else if (!AMRFD_ANY(lanes, !span_scale<4>(span, lob, bad))) {
     todo = sweep_part<LIMO, REC, 4>(gp, gm, plen, limo_thr, out, ostr, wmask, tp, tm, f0, fend, fmod, lob, limited);
   } else {
-    const bool whole = window_scale<5, true>(gp, gm, C0, nc, lob, bad);
-    todo = whole ? 0ull : partial_cells<LIMO>(gp, gm, nc, lob);
-    if (AMRFD_ANY(lanes, (~todo & all) != 0ull))
-      todo |= sweep_part<LIMO, REC, 5>(gp, gm, plen, limo_thr, out, ostr, wmask, tp, tm, f0, fend, fmod, lob, limited);
+    const Wide5 w = wide_sweep<LIMO, REC>(gp, gm, plen, limo_thr, out, ostr, wmask, tp, tm, f0, fend, fmod, span, lanes);
+    todo = w.todo;
+    limited = w.limited;
   }
   todo &= all;
   while (todo) {
@@ -1225,7 +1376,7 @@ AMRFD_HD_CALL void adjoint_cell(line_t g, TapeLine t, int kb, int ke, int cell, 
 
 template <int N>
 AMRFD_HD double gradient(const Limbs<N>& d, int lob) {
-  if constexpr (N == 4) return to_double(d, lob);
+  if constexpr (N >= 4) return to_double(d, lob);
   else return to_double(d, Limbs<N>{}, lob);
 }
 
