@@ -364,8 +364,8 @@ int tile_lines(const amrfd_handle* h, int seg, int threads) {
 
 // The default tile. Segments of 32 cells, 16 where the domains are too small to fill the GPU
 // otherwise. 320 threads in 3D, where lines abound (whole steps, 320 and 160 threads:
-// 123x95x78 Euler 2.79 and 3.11 ms, 21x168x112 Euler 1.71 and 2.14, 75x62x96 MHD 2.40 and
-// 2.53), and from sixteen tiles per CTA on; 160 below (512^2: 0.111 against 0.119 ms per
+// 21x168x112 Euler 1.56 and 1.71 ms, 123x95x78 Euler 2.65 and 2.66, 75x62x96 MHD 1.59 and
+// 1.59), and from sixteen tiles per CTA on; 160 below (512^2 MHD: 0.097 against 0.106 ms per
 // launch, the last wave of tiles shorter).
 // In 1D a tile is one line: few sweeps, and threads beyond them only wait at the barriers
 // (320 threads from 8e4 cells on: 4797 us for 1e6 cells of Euler, 4355 of MHD; with the FP64
@@ -1237,6 +1237,12 @@ int amrfd_autotune(amrfd_handle* h, double* U, const double* dt_dev, void* strea
     for (int full : {160, kFluxMaxThreads}) {
       const int ln = tile_lines(h, sg, full);
       if (ln == prev) continue;
+      // A warp of two variables takes the width and the limiter of the costlier one, which the
+      // state at hand may not show: 64 x 4 lines won a 256^3 blast's first step (9.9 ms a launch
+      // to 10.2 for 64 x 8) and took 21.5 to 15.0 with tails ahead of the front.
+      const int mixed = ln * line_sweeps(h, sg) % 32;
+      if (h->cfg.ndim == 3 && full < kFluxMaxThreads && mixed && tile_lines(h, sg, kFluxMaxThreads) * line_sweeps(h, sg) % 32 == 0)
+        continue;
       prev = ln;
       int last = 0;
       for (int extra : {0, 1, 3}) {
