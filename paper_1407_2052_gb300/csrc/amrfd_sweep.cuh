@@ -13,7 +13,7 @@
 //
 // Measured, the whole flux launch (FP64 sweeps before, these after): 1024^2 MHD vortex 768
 // and 352 us, 256^3 MHD blast in noise 16.1 and 10.2 ms (it limits at half its faces; 10.7 in
-// later steps, up to 12.9 while tails run through the box, see wide_sweep), 128^3 MHD blast
+// later steps, up to 12.7 while tails run through the box, see wide_sweep), 128^3 MHD blast
 // with LIMO3 2.12 and 0.97 ms. What bounds them now: integer issue (50 to 60 % of the slots,
 // about 490 instructions a face and warp where the limiter runs, 230 where not) and, at 35 %,
 // the FP64 pipe (phase A and one conversion a cell).
@@ -1189,10 +1189,11 @@ AMRFD_HD void linear_part(line_t gp, line_t gm, int plen, double* out, int ostr,
 // Out of line: most warps hold none, and its registers stay out of the other sweeps'.
 // What comes here is mostly tails ahead of a front: in the MHD blast eight of 27 (variable,
 // direction) pairs, through the whole box. Hence the filter where no face can be limited, and
-// the cuts that keep cells out of exact_cell. 256^3 flux launch in steps 1, 10, 24 and 80:
-// 10.3, 13.0, 19.8 and 14.2 ms with plain five-limb sweeps and each cell over 110 bits by
-// itself, 10.2, 11.0, 12.9 and 10.7 with both; never quarters 12.4 at step 13, from a range of
-// 100, 88 and 76 binades on 12.4, 12.0 and 11.5.
+// the cuts that keep cells out of exact_cell: a part over 57 binades goes in halves, one of
+// which, if it does not fit, in quarters (at once from 88 binades on: level with 76 and 110).
+// 256^3 flux launch in steps 1, 10, 24 and 80: 10.3, 13.0, 19.8 and 14.2 ms with plain five-limb
+// sweeps and each cell over 110 bits by itself, 10.2, 10.8, 12.7 and 10.7 with both; halves
+// only 12.6 at step 13, halves or quarters for the whole part 11.5, this 11.2.
 struct Wide5 {
   unsigned long long todo;
   int limited;
@@ -1205,20 +1206,31 @@ AMRFD_HD_CALL Wide5 wide_sweep(line_t gp, line_t gm, int plen, double limo_thr, 
   constexpr int NC = LIMO ? 4 : 6;
   unsigned long long todo = 0ull;
   int lob, limited = 0;
-  // Halves or quarters where some part spans more than 57 binades: ahead of a front a component
-  // falls off by about three binades a cell, 66 over the cells of a part of 16, 42 over its half's.
+  // ahead of a front a component falls off by about three binades a cell: 66 over the cells of
+  // a part of 16, 42 over its half's
   const int range = span.mn + 1u ? (int)(span.mx >> 20) - (int)((span.mn + 1u) >> 20) : 0;
-  int ns = AMRFD_ANY(lanes, range > 57) && !AMRFD_ANY(lanes, plen < 8) ? 2 : 1;
-  if (ns == 2 && AMRFD_ANY(lanes, range > 76) && !AMRFD_ANY(lanes, plen < 16)) ns = 4;
+  const int least = AMRFD_ANY(lanes, plen < 8) ? 4 : (AMRFD_ANY(lanes, plen < 16) ? 2 : 1);
+  int most = 4, size;
+  if (AMRFD_ANY(lanes, range > 57)) most = AMRFD_ANY(lanes, range > 88) ? 1 : 2;
+  most = most < least ? least : most;
 #pragma unroll 1
-  for (int s = 0; s < ns; s++) {
-    const int p0 = s * plen / ns, len = (s + 1) * plen / ns - p0;
-    const line_t p = line_at(gp, p0), m = line_at(gm, p0);
-    if (ns > 1) span = window_span<false>(p, m, C0, len + NC);
-    bool bad;
-    const bool fits = span_scale<5>(span, lob, bad);
+  for (int q = 0; q < 4; q += size) {  // size quarters from the q-th on
+    size = q & 1 ? 1 : most;
+    int p0, len;
+    line_t p, m;
+    bool bad, fits;
+    for (;;) {
+      p0 = q * plen / 4;
+      len = (q + size) * plen / 4 - p0;
+      p = line_at(gp, p0);
+      m = line_at(gm, p0);
+      if (size < 4) span = window_span<false>(p, m, C0, len + NC);
+      fits = span_scale<5>(span, lob, bad);
+      if (size == least || !AMRFD_ANY(lanes, !fits)) break;
+      size >>= 1;
+    }
     double* o = out + (long long)p0 * ostr;
-    const int fe = s + 1 < ns && f0 + p0 + len + 1 < fend ? f0 + p0 + len + 1 : fend;
+    const int fe = q + size < 4 && f0 + p0 + len + 1 < fend ? f0 + p0 + len + 1 : fend;
     const bool linear = !AMRFD_ANY(lanes, !surely_unlimited<LIMO>((int)(span.mx >> 20), limo_thr));
     if (linear && !AMRFD_ANY(lanes, !fits)) {
       linear_part<LIMO, REC, true>(p, m, len, o, ostr, wmask >> p0, tp, tm, f0 + p0, fe, fmod, lob);
