@@ -43,9 +43,9 @@ FLUX_FLOPS_PER_CELL_DIR = 254.4
 # 128^3 blast's first flux pass with the default tile: warp instructions, FP64 flop, and DRAM
 # bytes (read + write; traffic grows with the cells processed). A later step, with more faces
 # limited, executes more.
-FLUX_WARP_INST_PER_CELL = 920.090131e6 / 128 ** 3
-FLUX_FP64_FLOP_PER_CELL = (2 * 248.169404 + 9.432699 + 0.182142) * 1e6 / 128 ** 3
-FLUX_TRAFFIC_BYTES_PER_CELL = (369.609216 + 416.706048) * 1e6 / 128 ** 3
+FLUX_WARP_INST_PER_CELL = 907.261688e6 / 128 ** 3
+FLUX_FP64_FLOP_PER_CELL = (2 * 246.559523 + 7.875058) * 1e6 / 128 ** 3
+FLUX_TRAFFIC_BYTES_PER_CELL = (368.800256 + 414.736128) * 1e6 / 128 ** 3
 FP64_PEAK_TFLOPS_NOMINAL = 1.25   # GB300 FP64, nominal (context only)
 
 
