@@ -184,6 +184,22 @@ AMRFD_HD Limbs<5> limbs_wide(int hi, unsigned lo, int lob) {
   }
   return limbs5(mh, lo, L, x ? ((hi >> 31) | 1) : 0);
 }
+// The same at scales down to the last bit of the subnormals, which have no leading one. What
+// lies below 2^-1042 (no bit in the high word) counts as zero, as in every sweep.
+AMRFD_HD Limbs<5> limbs_low(int hi, unsigned lo, int lob) {
+  const int x = hi & 0x7fffffff;
+  const bool sub = x < 0x100000;
+  unsigned mh = sub ? (unsigned)x : ((unsigned)hi & 0xfffffu) | 0x100000u;
+  int L = (sub ? 1 : x >> 20) - (lob >> 20);
+  if (L < 0) {
+    const unsigned long long m = ((unsigned long long)mh << 32) | lo;
+    const unsigned long long r = L < -54 ? 0ull : (m + (1ull << (-L - 1))) >> -L;
+    mh = (unsigned)(r >> 32);
+    lo = (unsigned)r;
+    L = 0;
+  }
+  return limbs5(mh, lo, L, x ? ((hi >> 31) | 1) : 0);
+}
 // The same as limbs with four limbs: exponents in [lob >> 20, (lob >> 20) + 35].
 AMRFD_HD Limbs<4> limbs4(int hi, unsigned lo, int lob) {
   const int x = hi & 0x7fffffff;
@@ -788,15 +804,15 @@ AMRFD_HD Span window_span(line_t gp, line_t gm, int j, int nc) {
 }
 // The scale (lob) for N limbs; false when some cell is not a whole multiple of its unit or is
 // 2^1008 or more. bad: a value that is not finite. HEAD: bits left free above the largest.
-template <int N, int HEAD = 0>
+template <int N, int HEAD = 0, int LOW = kExpUnit>
 AMRFD_HD bool span_scale(const Span& w, int& lob, bool& bad) {
   int top = (int)(w.mx >> 20);
   bad = top == 2047;
   top = bad ? 2046 : top;
   constexpr int span = room(N) - HEAD;
-  lob = (top - span < kExpUnit ? kExpUnit : top - span) << 20;
+  lob = (top - span < LOW ? LOW : top - span) << 20;
   const unsigned low = w.mn == 0xffffffffu ? w.mn : (w.mn + 1u) >> 20;
-  return low >= (unsigned)(lob >> 20) && top <= kExpMax;
+  return (low >= (unsigned)(lob >> 20) || lob == 1 << 20) && top <= kExpMax;  // 1: the subnormals' own unit
 }
 // Both. FINE looks at the mantissas' trailing zeros, else every mantissa counts as 53 bits.
 template <int N, bool FINE, int HEAD = 0>
@@ -929,6 +945,13 @@ AMRFD_HD double exact_value(line_t gp, line_t gm, int i, double limo_thr, int lo
   return nearest(F, un, lob);
 }
 
+// to_double at a unit below 2^-988: results may be subnormal, and are then whole multiples of
+// the last bit.
+AMRFD_HD double low_double(const Limbs<5>& F, int lob) {
+  if (lob >= kExpUnit << 20) return to_double(F, lob);
+  return to_double(F, 1075 << 20) * 0x1p-537 * pow2d((lob >> 20) - 538);
+}
+
 // A cell both of whose faces are surely unlimited: a fixed filter of its cells, their largest
 // value (with a weight of at least 2) at 110 bits. What rounds, below 2^-110 of that, is far
 // below the rounding of any sum the large values are in. The tails ahead of a front, which
@@ -936,11 +959,8 @@ AMRFD_HD double exact_value(line_t gp, line_t gm, int i, double limo_thr, int lo
 template <bool LIMO>
 AMRFD_HD double linear_value(line_t gp, line_t gm, int j, int top) {
   constexpr int NC = LIMO ? 4 : 6;
-  const int lob = (top - room(5) < kExpUnit ? kExpUnit : top - room(5)) << 20;
-  const bool low = lob == kExpUnit << 20;  // values below the smallest unit count too
-  const Unit un = low ? unit_of(lob) : Unit{0.0, 0.0};
+  const int lob = (top - room(5) < 1 ? 1 : top - room(5)) << 20;
   Limbs<5> F = {};
-  double rest = 0.0;
 #pragma unroll
   for (int q = 0; q < NC; q++) {
     const int w = LIMO ? (q == 0 ? -10 : (q == 1 ? 60 : (q == 2 ? -30 : -20)))
@@ -949,16 +969,11 @@ AMRFD_HD double linear_value(line_t gp, line_t gm, int j, int top) {
     unsigned al, bl;
     cell_words(gp, j + q, ah, al);
     cell_words(gm, j + NC - q, bh, bl);
-    const Limbs<5> a = limbs_wide(ah, al, lob), b = limbs_wide(bh, bl, lob);
+    const Limbs<5> a = limbs_low(ah, al, lob), b = limbs_low(bh, bl, lob);
 #pragma unroll
     for (int l = 0; l < 5; l++) F.v[l] += w * (a.v[l] - b.v[l]);
-    if (low)
-      rest = fma((double)w, wide_cell<true>(gp, j + q, lob, un).r - wide_cell<true>(gm, j + NC - q, lob, un).r, rest);
   }
-  if (!low) return to_double(F, lob);
-  Wide<true> f = {to_wide(F), rest};
-  carry_units(f, un);
-  return nearest(f, un, lob);
+  return low_double(F, lob);
 }
 
 // Whether no face can be limited whose cells' exponents are most at most: differences lie below
@@ -1138,8 +1153,8 @@ AMRFD_HD unsigned long long sweep_part(line_t gp, line_t gm, int plen, double li
   return todo;
 }
 
-// The cells of a part whose faces are all surely unlimited (FIT: and whose exponents span at
-// most 57 binades): their differences as a fixed filter (linear_value) by transposed sums, without the face fluxes and FP32 differences of
+// The cells of a part whose faces are all surely unlimited (FIT: and whose exponents span
+// at most 57 binades, at a scale of 2^-988 or more): their differences as a fixed filter (linear_value) by transposed sums, without the face fluxes and FP32 differences of
 // sweep_part.
 template <bool LIMO, bool REC, bool FIT>
 AMRFD_HD void linear_part(line_t gp, line_t gm, int plen, double* out, int ostr, unsigned long long wmask,
@@ -1155,7 +1170,8 @@ AMRFD_HD void linear_part(line_t gp, line_t gm, int plen, double* out, int ostr,
     unsigned pl, ml;
     cell_words(gp, i + NC + C0, ph, pl);
     cell_words(gm, i + NC + C0, mh, ml);
-    const Limbs<5> x = limbs_wide<FIT>(ph, pl, lob), y = limbs_wide<FIT>(mh, ml, lob);
+    const Limbs<5> x = FIT ? limbs_wide<true>(ph, pl, lob) : limbs_low(ph, pl, lob);
+    const Limbs<5> y = FIT ? limbs_wide<true>(mh, ml, lob) : limbs_low(mh, ml, lob);
     Limbs<5> F;
 #pragma unroll
     for (int l = 0; l < 5; l++) {
@@ -1179,7 +1195,7 @@ AMRFD_HD void linear_part(line_t gp, line_t gm, int plen, double* out, int ostr,
     if (i < -1) continue;
     record<REC>(tp, tm, f0 + i + 1, fend, fmod, 0, 0);
     if (i < 0) continue;
-    if (wmask & 1ull) *out = to_double(F, lob);
+    if (wmask & 1ull) *out = FIT ? to_double(F, lob) : low_double(F, lob);
     out += ostr;
     wmask >>= 1;
   }
@@ -1218,27 +1234,30 @@ AMRFD_HD_CALL Wide5 wide_sweep(line_t gp, line_t gm, int plen, double limo_thr, 
     size = q & 1 ? 1 : most;
     int p0, len;
     line_t p, m;
-    bool bad, fits;
+    bool bad, fits, weak;
     for (;;) {
       p0 = q * plen / 4;
       len = (q + size) * plen / 4 - p0;
       p = line_at(gp, p0);
       m = line_at(gm, p0);
       if (size < 4) span = window_span<false>(p, m, C0, len + NC);
-      fits = span_scale<5>(span, lob, bad);
+      weak = surely_unlimited<LIMO>((int)(span.mx >> 20), limo_thr);
+      fits = weak ? span_scale<5, 0, 1>(span, lob, bad) : span_scale<5>(span, lob, bad);
       if (size == least || !AMRFD_ANY(lanes, !fits)) break;
       size >>= 1;
     }
     double* o = out + (long long)p0 * ostr;
     const int fe = q + size < 4 && f0 + p0 + len + 1 < fend ? f0 + p0 + len + 1 : fend;
-    const bool linear = !AMRFD_ANY(lanes, !surely_unlimited<LIMO>((int)(span.mx >> 20), limo_thr));
-    if (linear && !AMRFD_ANY(lanes, !fits)) {
+    const bool linear = !AMRFD_ANY(lanes, !weak);
+    const bool low = linear && lob < kExpUnit << 20 && span.mx;  // (zeros fit any scale)
+    if (linear && !AMRFD_ANY(lanes, !fits || low)) {
       linear_part<LIMO, REC, true>(p, m, len, o, ostr, wmask >> p0, tp, tm, f0 + p0, fe, fmod, lob);
       continue;
     }
+    if (!linear) fits = span_scale<5>(span, lob, bad);
     const unsigned long long cells = len < 64 ? (1ull << len) - 1ull : ~0ull;
     unsigned long long part = 0ull;
-    if (!fits && !window_scale<5, true>(p, m, C0, len + NC, lob, bad))
+    if (!fits && (low || !window_scale<5, true>(p, m, C0, len + NC, lob, bad)))
       part = partial_cells<LIMO>(p, m, len + NC, lob) & cells;
     if (linear)
       linear_part<LIMO, REC, false>(p, m, len, o, ostr, wmask >> p0, tp, tm, f0 + p0, fe, fmod, lob);

@@ -50,12 +50,12 @@ def lib(tmp_path_factory):
     return L
 
 
-def _tail(rng, n, binades, top):
+def _tail(rng, n, binades, top, end=-900):
     """Full mantissas of any sign, falling off by `binades` a cell from 2^top, to the left or
-    to the right, down to 2^-900 (near underflow the sweeps keep FP64's own precision: see
+    to the right, down to 2^end (near underflow the sweeps keep FP64's own precision: see
     test_weak_cells_beside_strong_ones_keep_their_precision)."""
     e = top - np.floor(binades * np.arange(n)).astype(int)
-    g, h = (np.where(e < -900, 0.0, np.ldexp(rng.uniform(1, 2, n) * rng.choice((-1, 1), n), e)) for _ in range(2))
+    g, h = (np.where(e < end, 0.0, np.ldexp(rng.uniform(1, 2, n) * rng.choice((-1, 1), n), e)) for _ in range(2))
     return (g[::-1].copy(), h[::-1].copy()) if rng.random() < 0.5 else (g, h)
 
 
@@ -100,3 +100,20 @@ def test_tails_round_once_from_any_height(lib, binades, top, limo):
             else:
                 near = abs(want) * Fraction(2) ** -52 + Fraction(float(w.max())) * Fraction(2) ** -100
                 assert abs(Fraction(float(out[i])) - want) <= near, (cells, i)
+
+
+@pytest.mark.parametrize("limo", [0, 1], ids=["mp5", "limo3"])
+@pytest.mark.parametrize("binades, cells", [(1, 64), (2, 21), (3, 16), (5, 19), (8, 2), (12, 16)])
+def test_tails_down_to_underflow_are_swept_too(lib, binades, cells, limo):
+    """From 2^-960 or less into the subnormals and zero: whole multiples of 2^-1074, hence exact.
+    Values below 2^-1042 count as zero."""
+    rng = np.random.default_rng(binades)
+    for top in (-960, -1000, -1015, -1025, -1035):
+        g, h = (np.where(np.abs(x) < 2.0 ** -1042, 0.0, x) for x in _tail(rng, cells + 6, binades, top, -1080))
+        left, out, tp, tm = _call(lib.left, limo, g, h, 1.0)
+        assert not tp.any() and not tm.any() and (left == 0 or binades > 5 or top > -1015)
+        full = _call(lib.sweep, limo, g, h, 1.0)[1]
+        for i, want in enumerate(_reference(limo, g, h, 1.0)):
+            w = np.abs(np.concatenate((g[i:i + 7], h[i:i + 7])))
+            if w.max() < 2.0 ** -967:  # its unit of 2^-110 is the subnormals' or below
+                assert full[i] == float(want), (top, i)
